@@ -281,6 +281,71 @@ __global__ void __launch_bounds__(128) k_kdsplit(Dev d, int w0, int w1) {
     }
 }
 
+constexpr int LB_WARPS = 8, LB_THREADS = LB_WARPS * 32;
+constexpr int LB_COLS = 32;   // columns per round of A (four per warp)
+constexpr int LB_VCAP = 512;  // visits per round (a column has at most 3 x 32)
+constexpr int LB_CCAP = 512;  // candidates per pass of C and D (a visit has at most 16)
+static_assert(LB_COLS == 4 * LB_WARPS && LB_VCAP == 2 * LB_THREADS && 3 * (MAX_COL / SC) <= LB_VCAP, "round sizes");
+// counters[8] hands out work items, counters[9] counts blocks that found no
+// more; the last one resets both for the next launch
+constexpr int CTR_LB_ITEM = 8, CTR_LB_DONE = 9;
+
+// Staged codes: exclusion group (bits 0-29; "no group" differs on the two
+// sides, so one compare decides the group test) | EXTRA_FLAG when the slot
+// has extra excluded partners.  Slots without normal pairs (padding,
+// alchemical) sit at FAR on the i side and -FAR on the j side, out of every
+// list radius.
+constexpr int GROUP_MASK = 0x3fffffff, EXTRA_FLAG = 0x40000000;
+constexpr int NO_GROUP_I = 0x3fffffff, NO_GROUP_J = 0x3ffffffe;
+constexpr float FAR = 536870912.0f;  // 2^29
+
+// exclusive scan over the block (v per thread); every thread gets the total
+__device__ __forceinline__ int block_scan(int v, int *wtot, int &total) {
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += t;
+    }
+    __syncthreads();  // wtot free
+    if (lane == 31) wtot[wib] = x;
+    __syncthreads();
+    int base = 0, tot = 0;
+#pragma unroll
+    for (int q = 0; q < LB_WARPS; ++q) {
+        const int t = wtot[q];
+        base += q < wib ? t : 0;
+        tot += t;
+    }
+    total = tot;
+    return base + x - v;
+}
+
+// R8 plan, by one block before the list kernel: the walkers that rebuild and
+// the prefixes of their alchemical atoms and super-clusters
+__device__ __forceinline__ void list_plan(const Dev &d, int w0, int w1) {
+    __shared__ int wtot[3][LB_WARPS];
+    const int w = w0 + threadIdx.x;
+    const bool on = w < w1 && d.rebuild[w] != 0;
+    const int ns = on ? d.n_sc[w] : 0, na = on ? d.sys[d.walk[w].sys].n_alch : 0;
+    int nt, st, at;
+    const int r = block_scan(on ? 1 : 0, wtot[0], nt);
+    const int sp = block_scan(ns, wtot[1], st);
+    const int ap = block_scan(na, wtot[2], at);
+    if (on) {
+        d.lb_w[r] = w;
+        d.lb_spre[r] = sp;
+        d.lb_apre[r] = ap;
+        d.lb_done[w] = 0;
+    }
+    if (threadIdx.x == 0) {
+        d.lb_tot[0] = nt;
+        d.lb_tot[1] = at;
+        d.lb_tot[2] = st;
+    }
+}
+
 // R6: gather the state into the new slot order (scratch buffers)
 __global__ void k_permute_gather(Dev d, int g0, int g1) {
     const int nthr = gridDim.x * blockDim.x;
@@ -313,8 +378,10 @@ __global__ void k_permute_gather(Dev d, int g0, int g1) {
     }
 }
 
-// R7: write the new layout back and refresh per-slot parameters
-__global__ void k_permute_scatter(Dev d, int g0, int g1) {
+// R7: write the new layout back and refresh per-slot parameters; the first
+// block also plans the list kernel's work
+__global__ void __launch_bounds__(256) k_permute_scatter(Dev d, int g0, int g1, int w0, int w1) {
+    if (blockIdx.x == 0) list_plan(d, w0, w1);
     const int nthr = gridDim.x * blockDim.x;
     for (int g = g0 + blockIdx.x * blockDim.x + threadIdx.x; g < g1; g += nthr) {
         const int w = d.slot_walker[g];
@@ -336,13 +403,17 @@ __global__ void k_permute_scatter(Dev d, int g0, int g1) {
             d.lj[g] = make_float2(ap.y, ap.z);
             d.im[g] = make_float2(ap.w, d.anoise[S.atom_off + a]);
             d.slot_of_atom[W.atom_base + a] = g;
-            d.smeta[g] = make_int2(d.agroup[S.atom_off + a], (int)d.aalch[S.atom_off + a]);
-            d.sexcl[g] = d.aexcl[S.atom_off + a];
+            const int grp = d.agroup[S.atom_off + a], alch = (int)d.aalch[S.atom_off + a];
+            const int4 ex = d.aexcl[S.atom_off + a];
+            d.smeta[g] = make_int2(grp, alch);
+            d.sexcl[g] = ex;
+            d.lcode[g] = alch ? -1 : ((grp >= 0 ? grp : GROUP_MASK) | ((ex.x & ex.y & ex.z & ex.w) != -1 ? EXTRA_FLAG : 0));
         } else {
             d.lj[g] = make_float2(0.f, 0.f);
             d.im[g] = make_float2(0.f, 0.f);
             d.smeta[g] = make_int2(-1, 1);
             d.sexcl[g] = make_int4(-1, -1, -1, -1);
+            d.lcode[g] = -1;
         }
         d.xq[g] = x;
         d.xref[g] = x;
@@ -350,15 +421,37 @@ __global__ void k_permute_scatter(Dev d, int g0, int g1) {
 }
 
 // -------------------------------------------------------------------------
-// R8: cluster-pair list.  One warp per work item (super-cluster S, run of
-// LB_CHUNK candidate column slots k): the k-th column (with its periodic
-// image) within reach of S's box.
-// For every candidate super-cluster T of that column (cyclic half rule) T's
-// 64 slots are staged in shared memory, the 16 x 8 (j-cluster, i-cluster)
-// box tests run lane-parallel, and for each passing pair of clusters lane
-// (ia, jb) = (lane & 7, lane >> 3) tests the atom pair (8 ic + ia of S,
-// 4 jc + jb of T) exactly.  Entries go to the (S, k) sub-list; R8b
-// concatenates the sub-lists of S in k order.
+// R8: cluster-pair list, alchemical list and pair-kernel work items.
+//
+// One block of eight warps per super-cluster S (work items handed out by a
+// global counter, alchemical atoms first):
+//   A  the candidate columns, four per warp: lane l tests the column's l-th
+//      super-cluster T (cyclic half rule, box distance for the three z
+//      images); the visits (T, image) go to shared memory in column, T,
+//      image order
+//   B  per visit the 16 j-clusters of T against S's box, 16 lanes each, and
+//      the candidates compacted in order
+//   C  per warp 8 candidates = 32 j-atoms, one per lane: every i-atom of S is
+//      broadcast from shared memory and tested, two i-atoms per packed FP32
+//      instruction; the lane collects its 64 result bits
+//   D  the candidates with a listed pair are appended to S's list in order
+// The lists need no per-column sub-lists, no compaction pass and no separate
+// launches for the alchemical lists and the work items: the last block of a
+// walker cuts its lists into work items.
+//
+// Bound by instruction issue (67% of the slots; 48% of the ALU pipe, 43% of
+// the FMA pipe).  One j-atom per lane keeps every lane on a candidate
+// j-cluster and puts the distances on the FMA pipe; per two i-atoms a lane
+// spends 8 packed FP32 and 7 ALU instructions, against about 55 for the two
+// half tiles with 64-bit integer arithmetic.  A rebuild of 16 walkers x 12 300
+// atoms (r_list 1.15 nm): 196 us, against 468 us for the four kernels before
+// (one warp per candidate column, compaction, alchemical lists, items); of one
+// such walker: 35 us against 156 us (ncu durations).
+//
+// The decision D < R is exact although it is made in FP32: coordinates are
+// taken relative to S's box, where they are integers below 2^24 (exact in
+// FP32), so D is off by less than tol; a lane that meets |D - R| <= tol
+// (about one pair in 10^5) repeats its 64 tests in integers.
 // -------------------------------------------------------------------------
 __device__ __forceinline__ long long bb_dist2(const int4 &alo, const int4 &ahi, const int4 &blo,
                                               const int4 &bhi, int sx, int sy, int sz) {
@@ -377,170 +470,168 @@ __device__ __forceinline__ bool excluded_meta(int a, int2 ma, int4 ea, int b, in
     return eb.x == a || eb.y == a || eb.z == a || eb.w == a;
 }
 
-constexpr int LB_WARPS = 4;
-// Staged slots: coordinates, and in .w a code = exclusion group (bits 0-29)
-// | EXTRA_FLAG when the slot has extra excluded partners.  Slots without
-// normal pairs (padding, alchemical) sit at FAR_I on the i side and FAR_J on
-// the j side (|d| >= 2^30 - 2^24 per component, so D >= R for every list
-// radius, and 3 (2^30 + 2^24)^2 < 2^63); "no group" has a different code on
-// each side, so that one compare decides the group test.
-constexpr int FAR_I = 1 << 29, FAR_J = -(1 << 29);
-constexpr int GROUP_MASK = 0x3fffffff, EXTRA_FLAG = 0x40000000;
-constexpr int NO_GROUP_I = 0x3fffffff, NO_GROUP_J = 0x3ffffffe;
+struct ListShared {
+    float4 row[SC / 2][2];  // i-atoms ia of i-clusters 2p, 2p + 1 at row 8p + ia: {x x' y y'}, {z z' code code'}
+    float4 ibox[NIC / 2][2];
+    int4 iex[SC];           // extra excluded partners and atom ids of S
+    int iatom[SC];
+    int colcnt[LB_COLS];
+    unsigned visit[LB_VCAP];  // T << 6 | shift bits
+    unsigned vmask[LB_VCAP];  // j-clusters of the visit in reach of S's box
+    int vpre[LB_VCAP + 1];
+    unsigned cand[LB_CCAP];   // visit << 4 | j-cluster
+    int cim[LB_CCAP], cpos[LB_CCAP];
+    unsigned long long mask[LB_CCAP][JC];
+    int wtot[LB_WARPS];
+};
+struct AlchShared {
+    unsigned long long okm[LB_THREADS];
+    int near_sc[LB_THREADS], off[LB_THREADS], wtot[LB_WARPS];
+};
+struct ItemShared {
+    int wtot[LB_WARPS];
+};
 
-__device__ __forceinline__ int slot_code(int2 m, int4 e, bool i_side) {
-    const int g = m.x >= 0 ? m.x : (i_side ? NO_GROUP_I : NO_GROUP_J);
-    return g | ((e.x & e.y & e.z & e.w) != -1 ? EXTRA_FLAG : 0);
+// extra excluded partners: atoms a (list ea) and b (list eb)
+__device__ __forceinline__ bool in_extra(int a, const int4 &ea, int b, const int4 &eb) {
+    return ea.x == b || ea.y == b || ea.z == b || ea.w == b || eb.x == a || eb.y == a || eb.z == a || eb.w == a;
 }
 
-// extra excluded partners of two real atoms (atom ids and lists from memory)
-__device__ __forceinline__ bool excluded_extra(const Dev &d, int gi, int gj) {
-    const int a = d.uq[gi].w, b = d.uq[gj].w;
-    const int4 ea = d.sexcl[gi], eb = d.sexcl[gj];
-    if (ea.x == b || ea.y == b || ea.z == b || ea.w == b) return true;
-    return eb.x == a || eb.y == a || eb.z == a || eb.w == a;
-}
-
-// lane (ia, jb)'s mask byte of one candidate j-cluster: bit ic set when the
-// pair (8 ic + ia of S, slot sj of T) is listed.  SELF: S and T are the
-// same super-cluster with shift 0, where only slot_i < slot_j is listed.
-template <bool SELF>
-__device__ __forceinline__ unsigned tile_masks(const int4 *su, unsigned cand, int ia, int sj, int ujx, int ujy,
-                                               int ujz, int cj, long long R, const Dev &d, int gS, int gT) {
-    unsigned lbyte = 0;
-    for (unsigned m = cand; m; m &= m - 1u) {  // candidate i-clusters, ascending
-        const int ic = __ffs(m) - 1;
-        const int si = ic * IC + ia;
-        const int4 ui = su[si];
-        // D < R implies every component lies in (-2^23, 2^23) (R <= 2^46
-        // because L >= 2 r_list), i.e. this shift is the minimum image
-        const int dx = ujx - ui.x, dy = ujy - ui.y, dz = ujz - ui.z;
-        bool ok = (long long)dx * dx + (long long)dy * dy + (long long)dz * dz < R && ((ui.w ^ cj) & GROUP_MASK) != 0;
-        if (SELF) ok = ok && si < sj;
-        if (ok && ((ui.w | cj) & EXTRA_FLAG)) ok = !excluded_extra(d, gS + si, gT + sj);
-        lbyte |= (unsigned)ok << ic;
+// one lane's 64 tests in integers (coordinates relative to S's box; the
+// staged i side holds them exactly); bit ia * 8 + ic
+__device__ __noinline__ unsigned long long exact_bits(const ListShared &sh, int jx, int jy, int jz, int jcode,
+                                                      long long R) {
+    unsigned long long m = 0;
+    for (int i = 0; i < SC; ++i) {
+        const int ic = i >> 3, ia = i & 7;
+        const float *r = reinterpret_cast<const float *>(&sh.row[(ic >> 1) * IC + ia][0]) + (ic & 1);
+        const long long dx = jx - (int)r[0], dy = jy - (int)r[2], dz = jz - (int)r[4];
+        if (dx * dx + dy * dy + dz * dz < R && ((__float_as_int(r[6]) ^ jcode) & GROUP_MASK) != 0)
+            m |= 1ull << (ia * 8 + ic);
     }
-    return lbyte;
+    return m;
 }
-constexpr int LB_CHUNK = 1;  // candidate-column slots per work item
 
-// work items (S, run of LB_CHUNK candidate-column slots) of the walkers that
-// rebuild are handed out by a global counter (counters[8]); the last warp
-// out (counters[9]) resets both for the next launch
-constexpr int CTR_LB_ITEM = 8, CTR_LB_DONE = 9;
+// word |= BIT when e < 0 and the exclusion groups of the two codes differ
+template <unsigned BIT>
+__device__ __forceinline__ void listed_bit(unsigned &word, float e, int ci, int cj) {
+    asm("{\n\t"
+        ".reg .pred q, p;\n\t"
+        ".reg .b32 t;\n\t"
+        "setp.lt.f32 q, %1, 0f00000000;\n\t"
+        "lop3.and.b32 t|p, %2, %3, %4, 0x28, q;\n\t"  // ((ci ^ cj) & GROUP_MASK) != 0 && q
+        "@p or.b32 %0, %0, %5;\n\t"
+        "}"
+        : "+r"(word)
+        : "f"(e), "r"(ci), "r"(cj), "r"(GROUP_MASK), "n"(BIT));
+}
 
-__global__ void __launch_bounds__(LB_WARPS * 32, 8) k_listbuild(Dev d, int w0, int w1) {
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int ia = lane & 7, jb = lane >> 3;
-    __shared__ int4 s_u[LB_WARPS][SC], t_u[LB_WARPS][SC];
-    __shared__ int4 s_bb[LB_WARPS][2 * NIC + 2], t_bb[LB_WARPS][2 * NJC];
-    __shared__ int s_pre[LA_MAX_WALKERS_PER_LAUNCH + 1], s_wk[LA_MAX_WALKERS_PER_LAUNCH];
-    __shared__ int s_nw;
-    const int nchunk = (d.ncs + LB_CHUNK - 1) / LB_CHUNK;
-    // prefix of the work items over the walkers that rebuild (their actual
-    // super-clusters only), so that walkers without a rebuild cost nothing
-    if (wib == 0) {
-        int acc = 0, nw = 0;
-        for (int base = w0; base < w1; base += 32) {
-            const int w = base + lane;
-            const bool on = w < w1 && d.rebuild[w] != 0;
-            int units = on ? d.n_sc[w] * nchunk : 0, rank = on ? 1 : 0;
+// C: the lane's 64 bits of one j-atom (rel. coordinates jx..jz) against S
+__device__ __forceinline__ unsigned long long test_atom(const ListShared &sh, float jx, float jy, float jz, int jcode,
+                                                        float Rf, float tol, bool &amb) {
+    const f2 nx = pack2(-jx, -jx), ny = pack2(-jy, -jy), nz = pack2(-jz, -jz), nR = pack2(-Rf, -Rf);
+    const float reach = Rf + tol;
+    unsigned half0 = 0u, half1 = 0u;
+    float emin = 3e38f;  // smallest |D - R| met
+#pragma unroll 1
+    for (int p = 0; p < NIC / 2; ++p) {
+        const float4 lo = sh.ibox[p][0], hi = sh.ibox[p][1];
+        const float gx = fmaxf(0.f, fmaxf(lo.x - jx, jx - hi.x)), gy = fmaxf(0.f, fmaxf(lo.y - jy, jy - hi.y)),
+                    gz = fmaxf(0.f, fmaxf(lo.z - jz, jz - hi.z));
+        // no lane within reach of the two i-clusters' box: nothing to test
+        if (!__any_sync(0xffffffffu, fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= reach)) continue;
+        unsigned h0 = 0u, h1 = 0u;
+#define LABF_ROW(IA)                                                                                     \
+    {                                                                                                    \
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(&sh.row[p * IC + IA][0]);              \
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(&sh.row[p * IC + IA][1]);              \
+        const f2 dx = add2(a.x, nx), dy = add2(a.y, ny), dz = add2(b.x, nz);                              \
+        float e0, e1;                                                                                    \
+        unpack2(add2(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), nR), e0, e1);                              \
+        emin = fminf(fminf(emin, fabsf(e0)), fabsf(e1));                                                 \
+        listed_bit<(1u << ((IA & 3) * 8))>(IA < 4 ? h0 : h1, e0, (int)b.y, jcode);                        \
+        listed_bit<(2u << ((IA & 3) * 8))>(IA < 4 ? h0 : h1, e1, (int)(b.y >> 32), jcode);                \
+    }
+        LABF_ROW(0) LABF_ROW(1) LABF_ROW(2) LABF_ROW(3) LABF_ROW(4) LABF_ROW(5) LABF_ROW(6) LABF_ROW(7)
+#undef LABF_ROW
+        half0 |= h0 << (2 * p);
+        half1 |= h1 << (2 * p);
+    }
+    amb = emin <= tol;
+    return ((unsigned long long)half1 << 32) | half0;
+}
+
+__device__ __forceinline__ void list_item(const Dev &d, ListShared &sh, int w, int S_loc) {
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    const WalkerDev &W = d.walk[w];
+    const SysDev &S = d.sys[W.sys];
+    const int s = W.sc_off + S_loc, gS = W.slot_off + S_loc * SC;
+    const int nsc = d.n_sc[w], ncx = S.ncx, cspan = S.cspan;
+    const int U = 1 << 24;
+    const long long R = S.R;
+    const float Rf = (float)R;
+    // conversion of coordinates beyond 2^24 (at most 1 each, so 2 sqrt(3 D) in
+    // D) and the roundings of D, twice over
+    const float tol = fmaf(Rf, 9.5367431640625e-07f, 16.0f * (float)S.Rq);
+    const int4 slo = d.bb_sc[2 * (size_t)s], shi = d.bb_sc[2 * (size_t)s + 1];
+    // ---- stage S ----
+    bool extra = false;
+    if (tid < SC) {
+        const int4 u = d.uq[gS + tid];
+        const int code = d.lcode[gS + tid];
+        const int ic = tid >> 3, ia = tid & 7;
+        float *r = reinterpret_cast<float *>(&sh.row[(ic >> 1) * IC + ia][0]) + (ic & 1);
+        r[0] = code < 0 ? FAR : (float)(u.x - slo.x);
+        r[2] = code < 0 ? FAR : (float)(u.y - slo.y);
+        r[4] = code < 0 ? FAR : (float)(u.z - slo.z);
+        const int g = code & GROUP_MASK;
+        r[6] = __int_as_float((g == GROUP_MASK ? NO_GROUP_I : g) | (code & EXTRA_FLAG));
+        sh.iatom[tid] = u.w;
+        sh.iex[tid] = d.sexcl[gS + tid];
+        extra = code >= 0 && (code & EXTRA_FLAG);
+    } else if (tid < SC + NIC / 2) {
+        const int p = tid - SC;
+        float4 lo = make_float4(4e9f, 4e9f, 4e9f, 0.f), hi = make_float4(-4e9f, -4e9f, -4e9f, 0.f);
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int a = __shfl_up_sync(0xffffffffu, units, o), b = __shfl_up_sync(0xffffffffu, rank, o);
-                if (lane >= o) {
-                    units += a;
-                    rank += b;
-                }
-            }
-            if (on) {
-                s_pre[nw + rank - 1] = acc + units - d.n_sc[w] * nchunk;
-                s_wk[nw + rank - 1] = w;
-            }
-            acc += __shfl_sync(0xffffffffu, units, 31);
-            nw += __shfl_sync(0xffffffffu, rank, 31);
+        for (int h = 0; h < 2; ++h) {
+            const int4 a = d.bb_ic[2 * ((size_t)s * NIC + 2 * p + h)], b = d.bb_ic[2 * ((size_t)s * NIC + 2 * p + h) + 1];
+            if (a.w <= 0) continue;
+            lo = make_float4(fminf(lo.x, (float)(a.x - slo.x)), fminf(lo.y, (float)(a.y - slo.y)),
+                             fminf(lo.z, (float)(a.z - slo.z)), 0.f);
+            hi = make_float4(fmaxf(hi.x, (float)(b.x - slo.x)), fmaxf(hi.y, (float)(b.y - slo.y)),
+                             fmaxf(hi.z, (float)(b.z - slo.z)), 0.f);
         }
-        if (lane == 0) {
-            s_pre[nw] = acc;
-            s_nw = nw;
-        }
+        sh.ibox[p][0] = lo;
+        sh.ibox[p][1] = hi;
     }
-    __syncthreads();
-    const int nw_on = s_nw;
-    const long long total = s_pre[nw_on];
-    for (;;) {
-        long long idx = 0;
-        if (lane == 0) idx = (long long)atomicAdd(&d.counters[CTR_LB_ITEM], 1ull);
-        idx = __shfl_sync(0xffffffffu, idx, 0);
-        if (idx >= total) break;
-        int lo = 0, hi = nw_on - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (s_pre[mid] <= idx) lo = mid; else hi = mid - 1;
-        }
-        const int w = s_wk[lo];
-        const int local = (int)(idx - s_pre[lo]);
-        const int s = d.walk[w].sc_off + local / nchunk;
-        const int k0 = (local % nchunk) * LB_CHUNK;
-        for (int kslot = k0; kslot < k0 + LB_CHUNK && kslot < d.ncs; ++kslot) {
-            const WalkerDev &W = d.walk[w];
-            const SysDev &S = d.sys[W.sys];
-            const int S_loc = s - W.sc_off;
-            const int nsc = d.n_sc[w];
-            const size_t sub = (size_t)s * d.ncs + kslot;
-            if (kslot >= S.cspan * S.cspan) {
-                if (lane == 0) d.sub_n[sub] = 0;
-                continue;
-            }
-            const int4 slo = d.bb_sc[2 * (size_t)s], shi = d.bb_sc[2 * (size_t)s + 1];
-            const int ncx = S.ncx;
-            const int cx0 = (int)(((long long)(slo.x - S.Rq) * ncx) >> 24);
-            const int cx1 = (int)(((long long)(shi.x + S.Rq) * ncx) >> 24);
-            const int cy0 = (int)(((long long)(slo.y - S.Rq) * ncx) >> 24);
-            const int cy1 = (int)(((long long)(shi.y + S.Rq) * ncx) >> 24);
-            const int cx = cx0 + kslot % S.cspan, cy = cy0 + kslot / S.cspan;
-            if (cx > cx1 || cy > cy1) {
-                if (lane == 0) d.sub_n[sub] = 0;
-                continue;
-            }
-            if (kslot == 0 && lane == 0 && (cx1 - cx0 >= S.cspan || cy1 - cy0 >= S.cspan))
-                set_status(d, LA_STATUS_LIST_OVERFLOW);  // cannot happen for boxes inside a column
-            const int gS = W.slot_off + S_loc * SC;
-            __syncwarp();
-            // staged: coordinates (FAR_I for a slot without normal pairs) and
-            // the slot code (exclusion group, extra-partner flag)
-            for (int k = lane; k < SC; k += 32) {
-                int4 u = d.uq[gS + k];
-                const int2 m = d.smeta[gS + k];
-                const int4 e = d.sexcl[gS + k];
-                if (m.y || u.w < 0) u.x = u.y = u.z = FAR_I;
-                u.w = slot_code(m, e, true);
-                s_u[wib][k] = u;
-            }
-            if (lane < 2 * NIC) s_bb[wib][lane] = d.bb_ic[2 * (size_t)s * NIC + lane];
-            __syncwarp();
-            const long long R = S.R;
-            const int U = 1 << 24;
-            const int ty = floordiv(cy, ncx), wy = cy - ty * ncx;
-            const int tx = floordiv(cx, ncx), wx = cx - tx * ncx;
-            const int col = wx + ncx * wy;
-            if (!la_in(d, col, W.n_cols)) {
-                if (lane == 0) d.sub_n[sub] = 0;
-                continue;
-            }
-            const int t0 = d.col_sc[W.col_off + col], tn = d.col_nsc[W.col_off + col];
-            int nent = 0;
-            const size_t ebase = sub * d.sub_cap;
-            const int t_end = min(t0 + tn, nsc);
-            // the column's super-clusters 32 at a time: lane l tests T = tb + l
-            // (half-list rule, then its box against S's box for the three z
-            // shifts); the warp then visits the T with a shift in range in
-            // ascending order
-            for (int tb = t0; tb < t_end; tb += 32) {
-                unsigned zp_l = 0;  // z shifts whose super-cluster boxes are in range
-                {
-                    const int T_loc = tb + lane;
-                    bool partner = T_loc < t_end;
+    const bool s_extra = __syncthreads_or(extra) != 0;
+    const int cx0 = (int)(((long long)(slo.x - S.Rq) * ncx) >> 24);
+    const int cx1 = (int)(((long long)(shi.x + S.Rq) * ncx) >> 24);
+    const int cy0 = (int)(((long long)(slo.y - S.Rq) * ncx) >> 24);
+    const int cy1 = (int)(((long long)(shi.y + S.Rq) * ncx) >> 24);
+    if (tid == 0 && (cx1 - cx0 >= cspan || cy1 - cy0 >= cspan))
+        set_status(d, LA_STATUS_LIST_OVERFLOW);  // cannot happen for boxes inside a column
+    const size_t ebase = (size_t)s * d.ent_cap;
+    int nent = 0;
+    const int ncol = cspan * cspan;
+    for (int c0 = 0; c0 < ncol;) {
+        // ---- A: visits of up to 32 columns, four per warp ----
+        unsigned zp = 0;  // z images in range of this lane's T, 3 bits per own column
+        int t_of[4], bits_of[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int k = c0 + 4 * wib + q;
+            const int cx = cx0 + k % cspan, cy = cy0 + k / cspan;
+            unsigned z = 0;
+            t_of[q] = bits_of[q] = 0;
+            if (k < ncol && cx <= cx1 && cy <= cy1) {
+                const int ty = floordiv(cy, ncx), tx = floordiv(cx, ncx);
+                const int col = cx - tx * ncx + ncx * (cy - ty * ncx);
+                bits_of[q] = (tx + 1) | ((ty + 1) << 2);
+                if (la_in(d, col, W.n_cols)) {
+                    const int T_loc = d.col_sc[W.col_off + col] + lane;
+                    t_of[q] = T_loc;
+                    bool partner = lane < min(d.col_nsc[W.col_off + col], MAX_COL / SC) && T_loc < nsc;
                     // cyclic half list over super-clusters: T is S's partner when it
                     // lies less than half-way round the index circle
                     if (partner && T_loc != S_loc) {
@@ -550,327 +641,360 @@ __global__ void __launch_bounds__(LB_WARPS * 32, 8) k_listbuild(Dev d, int w0, i
                     if (partner) {
                         const int t = W.sc_off + T_loc;
                         const int4 tlo = d.bb_sc[2 * (size_t)t], thi = d.bb_sc[2 * (size_t)t + 1];
-                        if (tlo.w != 0) {
+                        if (tlo.w != 0)
                             for (int tz = -1; tz <= 1; ++tz) {
                                 if (T_loc == S_loc && (tx < 0 || (tx == 0 && (ty < 0 || (ty == 0 && tz < 0))))) continue;
-                                if (bb_dist2(slo, shi, tlo, thi, tx * U, ty * U, tz * U) < R) zp_l |= 1u << (tz + 1);
+                                if (bb_dist2(slo, shi, tlo, thi, tx * U, ty * U, tz * U) < R) z |= 1u << (tz + 1);
                             }
-                        }
-                    }
-                }
-                for (unsigned tmask = __ballot_sync(0xffffffffu, zp_l != 0u); tmask; tmask &= tmask - 1u) {
-                    const int tl = __ffs(tmask) - 1;
-                    const int T_loc = tb + tl;
-                    const unsigned zpass = __shfl_sync(0xffffffffu, zp_l, tl);
-                    const int t = W.sc_off + T_loc;
-                    const int gT = W.slot_off + T_loc * SC;
-                    __syncwarp();
-                    for (int k = lane; k < SC; k += 32) {
-                        int4 u = d.uq[gT + k];
-                        const int2 m = d.smeta[gT + k];
-                        const int4 e = d.sexcl[gT + k];
-                        if (m.y || u.w < 0) u.x = u.y = u.z = FAR_J;
-                        u.w = slot_code(m, e, false);
-                        t_u[wib][k] = u;
-                    }
-                    t_bb[wib][lane] = d.bb_jc[2 * (size_t)t * NJC + lane];
-                    __syncwarp();
-                    for (int tz = -1; tz <= 1; ++tz) {
-                        if (!(zpass & (1u << (tz + 1)))) continue;
-                        const int shx = tx * U, shy = ty * U, shz = tz * U;
-                        const bool self0 = (T_loc == S_loc) && tx == 0 && ty == 0 && tz == 0;
-                        const int shift_bits = (tx + 1) | ((ty + 1) << 2) | ((tz + 1) << 4);
-                        // lane-parallel box tests of the 128 (jc, ic) combinations:
-                        // bit (jc & 3) * 8 + ic of word jc >> 2
-                        unsigned cm0, cm1, cm2, cm3;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int c = lane + 32 * q, jc = c >> 3, ic = c & 7;
-                            const int4 jlo = t_bb[wib][2 * jc], jhi = t_bb[wib][2 * jc + 1];
-                            const int4 ilo = s_bb[wib][2 * ic], ihi = s_bb[wib][2 * ic + 1];
-                            const bool ok = jlo.w > 0 && ilo.w > 0 && bb_dist2(ilo, ihi, jlo, jhi, shx, shy, shz) < R;
-                            const unsigned b = __ballot_sync(0xffffffffu, ok);
-                            if (q == 0) cm0 = b; else if (q == 1) cm1 = b; else if (q == 2) cm2 = b; else cm3 = b;
-                        }
-                        // j-clusters with at least one candidate i-cluster, ascending
-                        // (a non-zero byte of a word -> one bit: the byte flags
-                        // 0x01 at bits 0, 8, 16, 24 times 0x01020408 land at
-                        // bits 24-27 without carries)
-                        const auto nib = [](unsigned w) {
-                            return ((__vcmpne4(w, 0u) & 0x01010101u) * 0x01020408u) >> 24;
-                        };
-                        unsigned jmask = nib(cm0) | (nib(cm1) << 4) | (nib(cm2) << 8) | (nib(cm3) << 12);
-                        for (; jmask; jmask &= jmask - 1u) {
-                            const int jc = __ffs(jmask) - 1;
-                            const unsigned cw = jc < 8 ? (jc < 4 ? cm0 : cm1) : (jc < 12 ? cm2 : cm3);
-                            const unsigned cand = (cw >> ((jc & 3) * 8)) & 0xffu;
-                            const int4 uj = t_u[wib][jc * JC + jb];
-                            const int ujx = uj.x + shx, ujy = uj.y + shy, ujz = uj.z + shz;
-                            const unsigned lbyte =
-                                self0 ? tile_masks<true>(s_u[wib], cand, ia, jc * JC + jb, ujx, ujy, ujz, uj.w, R, d, gS, gT)
-                                      : tile_masks<false>(s_u[wib], cand, ia, jc * JC + jb, ujx, ujy, ujz, uj.w, R, d, gS, gT);
-                            const unsigned imask = __reduce_or_sync(0xffffffffu, lbyte);
-                            if (imask) {
-                                if (nent < d.sub_cap) {
-                                    const size_t e = ebase + nent;
-                                    // i-cluster mask twice: bits 8-15 are pruned by the batched
-                                    // step, bits 16-23 keep the listed set
-                                    if (lane == 0)
-                                        d.sub_hdr[e] = make_int2(gT + jc * JC, shift_bits | (int)(imask << 8) | (int)(imask << 16));
-                                    d.sub_lb[32 * e + lane] = (unsigned char)lbyte;
-                                } else if (lane == 0) {
-                                    set_status(d, LA_STATUS_LIST_OVERFLOW);
-                                }
-                                ++nent;
-                            }
-                        }
                     }
                 }
             }
-            if (lane == 0) d.sub_n[sub] = min(nent, d.sub_cap);
-            __syncwarp();
+            zp |= z << (3 * q);
+            const int cnt = __reduce_add_sync(0xffffffffu, __popc(z));
+            if (lane == 0) sh.colcnt[4 * wib + q] = cnt;
         }
-    }
-    // the last warp out resets the work counters for the next launch
-    if (lane == 0) {
-        __threadfence();
-        const unsigned long long done = atomicAdd(&d.counters[CTR_LB_DONE], 1ull);
-        if (done == (unsigned long long)gridDim.x * LB_WARPS - 1ull) {
-            d.counters[CTR_LB_ITEM] = 0ull;
-            d.counters[CTR_LB_DONE] = 0ull;
-            __threadfence();
+        __syncthreads();
+        // the leading columns whose visits fit the buffer (all of them, but for
+        // very crowded boxes)
+        const int cc = sh.colcnt[lane];
+        int incl = cc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
         }
-    }
-}
-
-// R8b: concatenate the sub-lists of each super-cluster in column-slot order
-__global__ void __launch_bounds__(128) k_listcompact(Dev d, int w0, int w1) {
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    __shared__ int s_off[4][32];
-    const int nwarp = gridDim.x * (blockDim.x >> 5);
-    const int s_begin = d.walk[w0].sc_off, s_end = d.walk[w1 - 1].sc_off + d.walk[w1 - 1].sc_cap;
-    for (int s = s_begin + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); s < s_end; s += nwarp) {
-        int lo = w0, hi = w1 - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (d.walk[mid].sc_off <= s) lo = mid; else hi = mid - 1;
-        }
-        if (!d.rebuild[lo]) continue;
-        if (s - d.walk[lo].sc_off >= d.n_sc[lo]) {  // capacity slot without a super-cluster
-            if (lane == 0) d.sc_nent[s] = 0;
-            continue;
-        }
-        const size_t ebase = (size_t)s * d.ent_cap;
-        int n = 0;
-        // 32 sub-lists at a time: their sizes by one load per lane and a warp
-        // scan, then every entry of the 32 copied by a flat lane loop (the
-        // sub-list of flat index f found by binary search over the offsets)
-        for (int k0 = 0; k0 < d.ncs; k0 += 32) {
-            const int k = k0 + lane;
-            const int m = k < d.ncs ? d.sub_n[(size_t)s * d.ncs + k] : 0;
-            int incl = m;
+        const int ncols = __popc(__ballot_sync(0xffffffffu, incl <= LB_VCAP));
+        const int nvis = __shfl_sync(0xffffffffu, incl, ncols - 1);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int col = 4 * wib + q;
+            int pos = __shfl_sync(0xffffffffu, incl - cc, col);
+            const unsigned z = (zp >> (3 * q)) & 7u;
+            const int n = __popc(z);
+            int x = n;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
+                const int t = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += t;
             }
-            const int tot = __shfl_sync(0xffffffffu, incl, 31);
-            s_off[wib][lane] = incl - m;
-            __syncwarp();
-            for (int f = lane; f < tot && n + f < d.ent_cap; f += 32) {
-                int lo = 0, hi = 31;  // the last sub-list starting at or before f
+            if (col < ncols) {
+                pos += x - n;
+                for (unsigned m = z; m; m &= m - 1u)
+                    sh.visit[pos++] = ((unsigned)t_of[q] << 6) | bits_of[q] | ((unsigned)(__ffs(m) - 1) << 4);
+            }
+        }
+        __syncthreads();
+        c0 += ncols;
+        // ---- B: the visits' j-clusters against S's box ----
+        for (int vb = 2 * wib; vb < nvis; vb += 2 * LB_WARPS) {
+            const int v = vb + (lane >> 4);
+            bool ok = false;
+            if (v < nvis) {
+                const unsigned vis = sh.visit[v];
+                const size_t b = 2 * ((size_t)(W.sc_off + (int)(vis >> 6)) * NJC + (lane & 15));
+                const int4 jlo = d.bb_jc[b], jhi = d.bb_jc[b + 1];
+                ok = jlo.w > 0 && bb_dist2(slo, shi, jlo, jhi, ((int)(vis & 3) - 1) * U, ((int)((vis >> 2) & 3) - 1) * U,
+                                           ((int)((vis >> 4) & 3) - 1) * U) < R;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, ok);
+            if ((lane & 15) == 0 && v < nvis) sh.vmask[v] = (m >> (lane & 16)) & 0xffffu;
+        }
+        __syncthreads();
+        {
+            const int n0 = 2 * tid < nvis ? __popc(sh.vmask[2 * tid]) : 0;
+            const int n1 = 2 * tid + 1 < nvis ? __popc(sh.vmask[2 * tid + 1]) : 0;
+            int tot;
+            const int pre = block_scan(n0 + n1, sh.wtot, tot);
+            sh.vpre[2 * tid] = pre;
+            sh.vpre[2 * tid + 1] = pre + n0;
+            if (tid == 0) sh.vpre[LB_VCAP] = tot;
+        }
+        __syncthreads();
+        for (int v0 = 0; v0 < nvis;) {
+            // the visits [v0, v1) whose candidates fit a pass
+            const int base = sh.vpre[v0];
+            int v1 = nvis;
+            if (sh.vpre[LB_VCAP] - base > LB_CCAP) {
+                int lo = v0 + 1, hi = nvis;  // largest v1 with vpre[v1] - base <= LB_CCAP
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
-                    if (s_off[wib][mid] <= f) lo = mid; else hi = mid - 1;
+                    if (sh.vpre[mid] - base <= LB_CCAP) lo = mid; else hi = mid - 1;
                 }
-                const size_t src = ((size_t)s * d.ncs + k0 + lo) * d.sub_cap + (f - s_off[wib][lo]);
-                const size_t dst = ebase + n + f;
-                d.ent_hdr[dst] = d.sub_hdr[src];
-                const uint4 *ps = reinterpret_cast<const uint4 *>(d.sub_lb + 32 * src);
-                uint4 *pd = reinterpret_cast<uint4 *>(d.ent_lb + 32 * dst);
-                pd[0] = ps[0];
-                pd[1] = ps[1];
+                v1 = lo;
             }
-            __syncwarp();
-            n += tot;
+            const int nc = (v1 < LB_VCAP ? sh.vpre[v1] : sh.vpre[LB_VCAP]) - base;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int v = 2 * tid + h;
+                if (v < v0 || v >= v1) continue;
+                int pos = sh.vpre[v] - base;
+                for (unsigned m = sh.vmask[v]; m; m &= m - 1u) sh.cand[pos++] = ((unsigned)v << 4) | (__ffs(m) - 1);
+            }
+            __syncthreads();
+            // ---- C: atom tests, eight candidates per warp ----
+            for (int g = wib; 8 * g < nc; g += LB_WARPS) {
+                const int c = 8 * g + (lane >> 2), q = lane & 3;
+                int rx = 0, ry = 0, rz = 0, jcode = NO_GROUP_J, gj = 0;
+                bool real = false, self0 = false;
+                if (c < nc) {
+                    const unsigned cd = sh.cand[c], vis = sh.visit[cd >> 4];
+                    const int T_loc = (int)(vis >> 6), sj = (int)(cd & 15u) * JC + q;
+                    gj = W.slot_off + T_loc * SC + sj;
+                    const int4 u = d.uq[gj];
+                    const int code = d.lcode[gj];
+                    real = code >= 0;
+                    rx = u.x + ((int)(vis & 3) - 1) * U - slo.x;
+                    ry = u.y + ((int)((vis >> 2) & 3) - 1) * U - slo.y;
+                    rz = u.z + ((int)((vis >> 4) & 3) - 1) * U - slo.z;
+                    const int gr = code & GROUP_MASK;
+                    jcode = (gr == GROUP_MASK ? NO_GROUP_J : gr) | (code & EXTRA_FLAG);
+                    self0 = T_loc == S_loc && (vis & 63u) == 21u;  // no shift
+                }
+                bool amb;
+                unsigned long long m = test_atom(sh, real ? (float)rx : -FAR, real ? (float)ry : -FAR,
+                                                 real ? (float)rz : -FAR, jcode, Rf, tol, amb);
+                if (amb) m = exact_bits(sh, rx, ry, rz, jcode, R);
+                if (self0) {  // the same super-cluster: only slot_i < slot_j
+                    const int sj = gj - gS, a = sj >> 3, b = sj & 7;
+                    const unsigned long long ones = 0x0101010101010101ull;
+                    m &= ((1ull << a) - 1ull) * ones | (ones & ((1ull << (8 * b)) - 1ull)) << a;
+                }
+                if (__any_sync(0xffffffffu, m != 0ull && (s_extra || (jcode & EXTRA_FLAG))) && m != 0ull) {
+                    const int b = d.uq[gj].w;
+                    const int4 eb = d.sexcl[gj];
+                    for (unsigned long long k = m; k; k &= k - 1ull) {
+                        const int bit = __ffsll((long long)k) - 1, i = (bit & 7) * IC + (bit >> 3);
+                        if (in_extra(sh.iatom[i], sh.iex[i], b, eb)) m &= ~(1ull << bit);
+                    }
+                }
+                unsigned f = (unsigned)m | (unsigned)(m >> 32);
+                f |= f >> 16;
+                f = (f | (f >> 8)) & 0xffu;
+                f |= __shfl_xor_sync(0xffffffffu, f, 1);
+                f |= __shfl_xor_sync(0xffffffffu, f, 2);
+                if (c < nc) {
+                    sh.mask[c][q] = m;
+                    if (q == 0) sh.cim[c] = (int)f;
+                }
+            }
+            __syncthreads();
+            // ---- D: append the candidates with a listed pair ----
+            for (int b = 0; b < nc; b += LB_THREADS) {
+                const int c = b + tid;
+                const unsigned im = c < nc ? (unsigned)sh.cim[c] : 0u;
+                int tot;
+                const int e = nent + block_scan(im ? 1 : 0, sh.wtot, tot);
+                nent += tot;
+                if (c < nc) {
+                    sh.cpos[c] = im && e < d.ent_cap ? e : -1;
+                    if (im && e < d.ent_cap) {
+                        // i-cluster mask twice: bits 8-15 are pruned by the batched
+                        // step, bits 16-23 keep the listed set
+                        const unsigned cd = sh.cand[c], vis = sh.visit[cd >> 4];
+                        d.ent_hdr[ebase + e] = make_int2(W.slot_off + (int)(vis >> 6) * SC + (int)(cd & 15u) * JC,
+                                                         (int)((vis & 63u) | (im << 8) | (im << 16)));
+                    }
+                }
+            }
+            __syncthreads();
+            for (int k = tid; k < nc * JC; k += LB_THREADS) {
+                const int e = sh.cpos[k >> 2];
+                if (e >= 0)
+                    *reinterpret_cast<unsigned long long *>(d.ent_lb + 32 * (ebase + e) + 8 * (k & 3)) = sh.mask[k >> 2][k & 3];
+            }
+            __syncthreads();
+            v0 = v1;
         }
-        if (n > d.ent_cap && lane == 0) set_status(d, LA_STATUS_LIST_OVERFLOW);
-        if (lane == 0) d.sc_nent[s] = min(n, d.ent_cap);
+    }
+    if (tid == 0) {
+        if (nent > d.ent_cap) set_status(d, LA_STATUS_LIST_OVERFLOW);
+        d.sc_nent[s] = min(nent, d.ent_cap);
     }
 }
 
-// -------------------------------------------------------------------------
-// R9: alchemical list: one block per (walker, alchemical atom).  Super-cluster
-// boxes are tested lane-parallel; the 64 slots of each box in range are then
-// tested exactly (two per lane) by the block's warps in turn, and the hits
-// are written in super-cluster and slot order (deterministic output order).
-// -------------------------------------------------------------------------
-constexpr int AL_WARPS = 4;
-
-__global__ void __launch_bounds__(AL_WARPS * 32) k_alchlist(Dev d, int w0, int w1, int a0, int a1) {
-    // one block per (walker, alchemical atom); the super-clusters are box
-    // tested one per thread, 128 per round, the near ones compacted in
-    // ascending order and tested slot by slot by the block's warps in turn,
-    // and warp 0 writes the hits in (super-cluster, slot) order
-    constexpr int NT = AL_WARPS * 32;
-    __shared__ unsigned long long okm[NT];
-    __shared__ int near_sc[NT];
-    __shared__ int wcnt[AL_WARPS];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    for (int it = a0 + blockIdx.x; it < a1; it += gridDim.x) {
-        int lo = w0, hi = w1 - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (d.walk[mid].alch_base <= it) lo = mid; else hi = mid - 1;
-        }
-        const int w = lo;
-        if (!d.rebuild[w]) continue;
-        const WalkerDev &W = d.walk[w];
-        const SysDev &S = d.sys[W.sys];
-        const int r = it - W.alch_base;
-        const int a = d.alch_atoms[S.alch_off + r];
-        if (!la_in(d, a, S.n_atoms)) continue;
-        const int ga = d.slot_of_atom[W.atom_base + a];
-        if (!la_in(d, ga, d.n_slots)) continue;
-        const int4 ua = d.uq[ga];
-        const int2 ma = d.smeta[ga];
-        const int4 ea = d.sexcl[ga];
-        const int U = 1 << 24;
-        int cnt = 0;
-        const int nsc = d.n_sc[w];
-        int *out = d.alch_slot + (size_t)it * d.alch_cap;
-        for (int b0 = 0; b0 < nsc; b0 += NT) {
-            // super-cluster box within the list radius of the atom (any image)
-            bool near = false;
-            if (b0 + (int)threadIdx.x < nsc) {
-                const size_t t = (size_t)(W.sc_off + b0 + threadIdx.x);
-                const int4 tlo = d.bb_sc[2 * t], thi = d.bb_sc[2 * t + 1];
-                if (tlo.w > 0) {
-                    long long D = 0;
-                    const int uc[3] = {ua.x, ua.y, ua.z};
-                    const int lc[3] = {tlo.x, tlo.y, tlo.z}, hc[3] = {thi.x, thi.y, thi.z};
-                    for (int c = 0; c < 3; ++c) {
-                        long long best = -1;
-                        for (int sh = -1; sh <= 1; ++sh) {
-                            const long long gap = max(0, max(lc[c] + sh * U - uc[c], uc[c] - (hc[c] + sh * U)));
-                            if (best < 0 || gap < best) best = gap;
-                        }
-                        D += best * best;
-                    }
-                    near = D < S.R;
-                }
-            }
-            // compaction in ascending order: warp counts, then offsets
-            const unsigned nm = __ballot_sync(0xffffffffu, near);
-            if (lane == 0) wcnt[wib] = __popc(nm);
-            __syncthreads();
-            int off = 0, nn = 0;
-            for (int q = 0; q < AL_WARPS; ++q) {
-                off += q < wib ? wcnt[q] : 0;
-                nn += wcnt[q];
-            }
-            if (near) near_sc[off + __popc(nm & ((1u << lane) - 1u))] = b0 + threadIdx.x;
-            __syncthreads();
-            for (int kk = wib; kk < nn; kk += AL_WARPS) {
-                const int gbase = W.slot_off + near_sc[kk] * SC;
-                unsigned bits[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int g = gbase + lane + 32 * h;
-                    const int4 ub = d.uq[g];
-                    const int2 mb = d.smeta[g];
-                    bool ok = false;
-                    if (ub.w >= 0 && !mb.y) {
-                        const long long dx = torus_delta(ub.x, ua.x), dy = torus_delta(ub.y, ua.y),
-                                        dz = torus_delta(ub.z, ua.z);
-                        ok = dx * dx + dy * dy + dz * dz < S.R && !excluded_meta(a, ma, ea, ub.w, mb, d.sexcl[g]);
-                    }
-                    bits[h] = __ballot_sync(0xffffffffu, ok);
-                }
-                if (lane == 0) okm[kk] = ((unsigned long long)bits[1] << 32) | bits[0];
-            }
-            __syncthreads();
-            if (wib == 0) {
-                for (int kk = 0; kk < nn; ++kk) {
-                    const int gbase = W.slot_off + near_sc[kk] * SC;
-                    const unsigned long long om = okm[kk];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const unsigned mh = h ? (unsigned)(om >> 32) : (unsigned)om;
-                        const int pos = cnt + __popc(mh & ((1u << lane) - 1u));
-                        if (((mh >> lane) & 1u) && pos < d.alch_cap) out[pos] = gbase + lane + 32 * h;
-                        cnt += __popc(mh);
-                    }
-                }
-            }
-            __syncthreads();
-        }
-        if (wib == 0) {
-            if (cnt > d.alch_cap) {
-                if (lane == 0) set_status(d, LA_STATUS_ALCH_OVERFLOW);
-                cnt = d.alch_cap;
-            }
-            if (lane == 0) d.alch_cnt[it] = cnt;
-        }
-    }
-}
-
-// -------------------------------------------------------------------------
-// R10: pair-kernel work items (chunks of `chunk` entries of one
-// super-cluster), per walker; clears the rebuild flag.  In the batched step
-// (prune_fresh) a walker with pruning on has its fresh list pruned by this
-// step's pair pass.
-// -------------------------------------------------------------------------
-__global__ void k_items(Dev d, int w0, int prune_fresh) {
-    const int w = w0 + blockIdx.x;
-    if (!d.rebuild[w]) return;
+// alchemical list of one (walker, alchemical atom): super-cluster boxes are
+// tested one per thread, the near ones compacted in ascending order and
+// tested slot by slot by the block's warps in turn; the hits are written in
+// (super-cluster, slot) order
+__device__ __forceinline__ void alch_item(const Dev &d, AlchShared &sh, int w, int r) {
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     const WalkerDev &W = d.walk[w];
-    __shared__ int wsum[32];
-    __shared__ int carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
+    const SysDev &S = d.sys[W.sys];
+    const int it = W.alch_base + r;
+    const int a = d.alch_atoms[S.alch_off + r];
+    if (!la_in(d, a, S.n_atoms)) return;
+    const int ga = d.slot_of_atom[W.atom_base + a];
+    if (!la_in(d, ga, d.n_slots)) return;
+    const int4 ua = d.uq[ga];
+    const int2 ma = d.smeta[ga];
+    const int4 ea = d.sexcl[ga];
+    const int U = 1 << 24;
+    int cnt = 0;
     const int nsc = d.n_sc[w];
-    for (int base = 0; base < nsc; base += blockDim.x) {
+    int *out = d.alch_slot + (size_t)it * d.alch_cap;
+    for (int b0 = 0; b0 < nsc; b0 += LB_THREADS) {
+        // super-cluster box within the list radius of the atom (any image)
+        bool near = false;
+        if (b0 + tid < nsc) {
+            const size_t t = (size_t)(W.sc_off + b0 + tid);
+            const int4 tlo = d.bb_sc[2 * t], thi = d.bb_sc[2 * t + 1];
+            if (tlo.w > 0) {
+                long long D = 0;
+                const int uc[3] = {ua.x, ua.y, ua.z};
+                const int lc[3] = {tlo.x, tlo.y, tlo.z}, hc[3] = {thi.x, thi.y, thi.z};
+                for (int c = 0; c < 3; ++c) {
+                    long long best = -1;
+                    for (int sh3 = -1; sh3 <= 1; ++sh3) {
+                        const long long gap = max(0, max(lc[c] + sh3 * U - uc[c], uc[c] - (hc[c] + sh3 * U)));
+                        if (best < 0 || gap < best) best = gap;
+                    }
+                    D += best * best;
+                }
+                near = D < S.R;
+            }
+        }
+        int nn;
+        const int pos = block_scan(near ? 1 : 0, sh.wtot, nn);
+        if (near) sh.near_sc[pos] = b0 + tid;
+        __syncthreads();
+        for (int kk = wib; kk < nn; kk += LB_WARPS) {
+            const int gbase = W.slot_off + sh.near_sc[kk] * SC;
+            unsigned bits[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int g = gbase + lane + 32 * h;
+                const int4 ub = d.uq[g];
+                const int2 mb = d.smeta[g];
+                const int4 eb = d.sexcl[g];
+                bool ok = false;
+                if (ub.w >= 0 && !mb.y) {
+                    const long long dx = torus_delta(ub.x, ua.x), dy = torus_delta(ub.y, ua.y),
+                                    dz = torus_delta(ub.z, ua.z);
+                    ok = dx * dx + dy * dy + dz * dz < S.R && !excluded_meta(a, ma, ea, ub.w, mb, eb);
+                }
+                bits[h] = __ballot_sync(0xffffffffu, ok);
+            }
+            if (lane == 0) sh.okm[kk] = ((unsigned long long)bits[1] << 32) | bits[0];
+        }
+        __syncthreads();
+        int tot;
+        const int off = block_scan(tid < nn ? __popcll(sh.okm[tid]) : 0, sh.wtot, tot);
+        sh.off[tid] = cnt + off;
+        __syncthreads();
+        for (int kk = wib; kk < nn; kk += LB_WARPS) {
+            const int gbase = W.slot_off + sh.near_sc[kk] * SC;
+            const unsigned long long om = sh.okm[kk];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int b = lane + 32 * h;
+                const int pos2 = sh.off[kk] + __popcll(om & ((1ull << b) - 1ull));
+                if (((om >> b) & 1ull) && pos2 < d.alch_cap) out[pos2] = gbase + b;
+            }
+        }
+        cnt += tot;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        if (cnt > d.alch_cap) set_status(d, LA_STATUS_ALCH_OVERFLOW);
+        d.alch_cnt[it] = min(cnt, d.alch_cap);
+    }
+}
+
+// pair-kernel work items of a walker (chunks of `chunk` entries of one
+// super-cluster); clears the rebuild flag.  In the batched step (prune_fresh)
+// a walker with pruning on has its fresh list pruned by this step's pair pass.
+// Entry counts may come from other blocks of the launch: read past L1.
+__device__ __forceinline__ void make_items(const Dev &d, ItemShared &sh, int w, int prune_fresh) {
+    const WalkerDev &W = d.walk[w];
+    const int nsc = d.n_sc[w];
+    int done = 0;
+    for (int base = 0; base < nsc; base += LB_THREADS) {
         const int sl = base + threadIdx.x;
-        const int ne = sl < nsc ? d.sc_nent[W.sc_off + sl] : 0;
+        const int ne = sl < nsc ? __ldcg(d.sc_nent + W.sc_off + sl) : 0;
         const int nch = (ne + d.chunk - 1) / d.chunk;
-        // block exclusive scan of nch
-        int v = nch;
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += t;
-        }
-        if (lane == 31) wsum[wid] = v;
-        __syncthreads();
-        if (wid == 0) {
-            int t = lane < (int)(blockDim.x >> 5) ? wsum[lane] : 0;
-            for (int o = 1; o < 32; o <<= 1) {
-                int u = __shfl_up_sync(0xffffffffu, t, o);
-                if (lane >= o) t += u;
-            }
-            wsum[lane] = t;
-        }
-        __syncthreads();
-        const int excl = carry + v - nch + (wid > 0 ? wsum[wid - 1] : 0);
-        for (int c = 0; c < nch; ++c) {
-            const int item = excl + c;
-            if (item < W.item_cap) {
-                const int e0 = c * d.chunk, e1 = min(ne, e0 + d.chunk);
-                d.items[W.item_base + item] = make_int4(W.sc_off + sl, e0, e1, w);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = excl + nch;
-        __syncthreads();
+        int tot;
+        const int first = done + block_scan(nch, sh.wtot, tot);
+        done += tot;
+        for (int c = 0; c < nch; ++c)
+            if (first + c < W.item_cap)
+                d.items[W.item_base + first + c] = make_int4(W.sc_off + sl, c * d.chunk, min(ne, (c + 1) * d.chunk), w);
     }
     if (threadIdx.x == 0) {
-        if (carry > W.item_cap) set_status(d, LA_STATUS_LIST_OVERFLOW);
-        d.n_items[w] = min(carry, W.item_cap);
+        if (done > W.item_cap) set_status(d, LA_STATUS_LIST_OVERFLOW);
+        d.n_items[w] = min(done, W.item_cap);
         d.rebuild[w] = 0;
         d.near[w] = 0;
         if (prune_fresh && d.sys[W.sys].prune_disp2 > 0.f) d.prune_now[w] = d.step[w] + 1ull;
         atomicAdd(&d.counters[0], 1ull);
+    }
+}
+
+// work items alone (the autotuner's other chunk sizes)
+__global__ void __launch_bounds__(LB_THREADS) k_items(Dev d, int w0) {
+    __shared__ ItemShared sh;
+    const int w = w0 + blockIdx.x;
+    if (d.rebuild[w]) make_items(d, sh, w, 0);
+}
+
+__global__ void __launch_bounds__(LB_THREADS, 4) k_listbuild(Dev d, int prune_fresh) {
+    __shared__ union {
+        ListShared list;
+        AlchShared alch;
+        ItemShared item;
+    } sh;
+    __shared__ int s_w[LA_MAX_WALKERS_PER_LAUNCH], s_pre[2][LA_MAX_WALKERS_PER_LAUNCH];
+    __shared__ int s_idx, s_last;
+    const int tid = threadIdx.x;
+    const int nw = d.lb_tot[0], n_alch = d.lb_tot[1], total = n_alch + d.lb_tot[2];
+    if (tid < nw) {
+        s_w[tid] = d.lb_w[tid];
+        s_pre[0][tid] = d.lb_apre[tid];
+        s_pre[1][tid] = d.lb_spre[tid];
+    }
+    // the next item's index is fetched one item ahead
+    int next = 0;
+    if (tid == 0) next = (int)atomicAdd(&d.counters[CTR_LB_ITEM], 1ull);
+    for (;;) {
+        if (tid == 0) s_idx = next;
+        __syncthreads();
+        const int idx = s_idx;
+        if (idx >= total) break;
+        if (tid == 0) next = (int)atomicAdd(&d.counters[CTR_LB_ITEM], 1ull);
+        const bool alch = idx < n_alch;
+        const int v = alch ? idx : idx - n_alch;
+        const int *pre = s_pre[alch ? 0 : 1];
+        int lo = 0, hi = nw - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (pre[mid] <= v) lo = mid; else hi = mid - 1;
+        }
+        const int w = s_w[lo];
+        if (alch) {
+            alch_item(d, sh.alch, w, v - pre[lo]);
+            __syncthreads();
+            continue;
+        }
+        list_item(d, sh.list, w, v - pre[lo]);
+        if (tid == 0) {
+            __threadfence();
+            s_last = atomicAdd(&d.lb_done[w], 1u) == (unsigned)d.n_sc[w] - 1u;
+        }
+        __syncthreads();
+        if (s_last) {  // the walker's last super-cluster: cut its lists into work items
+            __threadfence();
+            make_items(d, sh.item, w, prune_fresh);
+        }
+        __syncthreads();
+    }
+    // the last block out resets the work counters for the next launch
+    if (tid == 0) {
+        __threadfence();
+        const unsigned long long done = atomicAdd(&d.counters[CTR_LB_DONE], 1ull);
+        if (done == (unsigned long long)gridDim.x - 1ull) {
+            d.counters[CTR_LB_ITEM] = 0ull;
+            d.counters[CTR_LB_DONE] = 0ull;
+            __threadfence();
+        }
     }
 }
 
@@ -952,28 +1076,15 @@ void launch_rebuild(const Dev &d, const HostView &hv, int w0, int w1, cudaStream
     k_colsort<<<cg, 256, 0, s>>>(d, w0);
     k_kdsplit<<<kb, 128, 0, s>>>(d, w0, w1);
     k_permute_gather<<<sb, 256, 0, s>>>(d, g0, g1);
-    k_permute_scatter<<<sb, 256, 0, s>>>(d, g0, g1);
-    {
-        long long nlb = ((long long)nsc * hv.ncs + LB_WARPS - 1) / LB_WARPS;
-        int lb = (int)(nlb < (long long)hv.n_sm * 8 ? nlb : (long long)hv.n_sm * 8);  // resident grid
-        k_listbuild<<<lb < 1 ? 1 : lb, LB_WARPS * 32, 0, s>>>(d, w0, w1);
-        k_listcompact<<<kb, 128, 0, s>>>(d, w0, w1);
-    }
-    if (a1 > a0) {
-        int ab = a1 - a0;
-        ab = ab > hv.n_sm * 8 ? hv.n_sm * 8 : ab;
-        k_alchlist<<<ab, AL_WARPS * 32, 0, s>>>(d, w0, w1, a0, a1);
-    }
-    k_items<<<nw, 256, 0, s>>>(d, w0, batched ? 1 : 0);
+    k_permute_scatter<<<sb, LB_THREADS, 0, s>>>(d, g0, g1, w0, w1);
+    const int lb = nsc + a1 - a0 < hv.n_sm * 4 ? nsc + a1 - a0 : hv.n_sm * 4;  // resident grid
+    k_listbuild<<<lb < 1 ? 1 : lb, LB_THREADS, 0, s>>>(d, batched ? 1 : 0);
 }
 
 void launch_items(const Dev &d, const HostView &, int w0, int w1, cudaStream_t s) {
-    k_items<<<w1 - w0, 256, 0, s>>>(d, w0, 0);
+    k_items<<<w1 - w0, LB_THREADS, 0, s>>>(d, w0);
 }
 
-int rebuild_kernel_count(const HostView &hv, int w0, int w1) {
-    const int a0 = hv.alch_base[w0], a1 = hv.alch_base[w1 - 1] + hv.n_alch[w1 - 1];
-    return a1 > a0 ? 11 : 10;
-}
+int rebuild_kernel_count(const HostView &, int, int) { return 8; }
 
 }  // namespace labf

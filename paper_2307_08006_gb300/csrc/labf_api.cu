@@ -41,7 +41,7 @@ struct Layout {
     int W = 0, n_stages = 0, total_bins = 0, max_bins = 0, P_max = 1;
     long long slots = 0, scs = 0, cols = 0, atoms_w = 0, alch_w = 0, items = 0, bo = 0;
     long long atoms_s = 0, alch_s = 0, bonds = 0, angles = 0, posres = 0, fb = 0, lh = 0, lr = 0;
-    int ent_cap = 0, alch_cap = 0, chunk = 32, max_n = 0, ncs = 1, sub_cap = 0;
+    int ent_cap = 0, alch_cap = 0, chunk = 32, max_n = 0;
     size_t bytes = 0;
 };
 
@@ -138,7 +138,7 @@ void compute_layout(const la_system_desc *sys, int n_sys, const la_options *opt,
     const double fac = (opt && opt->list_capacity_factor >= 1.0) ? opt->list_capacity_factor : 1.6;
     L.chunk = (opt && opt->chunk_entries > 0) ? opt->chunk_entries : 32;
     const double pi = 3.14159265358979323846;
-    double ent_est = 0.0, alch_est = 0.0, sub_est = 0.0;
+    double ent_est = 0.0, alch_est = 0.0;
     for (int s = 0; s < n_sys; ++s) {
         const la_system_desc &S = sys[s];
         SysLayout sl{};
@@ -196,11 +196,6 @@ void compute_layout(const la_system_desc *sys, int n_sys, const la_options *opt,
         // floor(3 + 2 Rq ncx / 2^24) columns are within reach
         sl.Rq = (int)std::ceil(sl.r_list / S.box * 16777216.0) + 1;
         sl.cspan = (int)std::floor(3.0 + 2.0 * sl.Rq * (double)sl.ncx / 16777216.0);
-        L.ncs = std::max(L.ncs, sl.cspan * sl.cspan);
-        const double col_jc = std::max(sl.rho * wc * wc * (h + 2.0 * sl.r_list + 2.0 * ej),
-                                       rho_dense * wc * wc * (h_tall + 2.0 * sl.r_list + 2.0 * ej)) / JC;
-        const double col_cap = 3.0 * NJC * (std::max(sl.rho * wc * wc * S.box, (double)cmax) / SC + 2.0);
-        sub_est = std::max(sub_est, std::min(col_jc, col_cap));
         alch_est = std::max(alch_est, sl.rho * 4.0 / 3.0 * pi * std::pow(sl.r_list, 3));
         L.sys.push_back(sl);
         L.W += sl.W;
@@ -229,7 +224,6 @@ void compute_layout(const la_system_desc *sys, int n_sys, const la_options *opt,
     // the cyclic half list gives each super-cluster about half its neighbourhood
     L.ent_cap = (int)std::ceil(fac * 0.6 * ent_est) + 64;
     L.alch_cap = ((int)std::ceil(fac * alch_est) + 64 + 31) / 32 * 32;
-    L.sub_cap = ((int)std::ceil(fac * sub_est) + 32 + 31) / 32 * 32;
     const int chunks = (L.ent_cap + L.chunk - 1) / L.chunk;
     L.items = L.scs * chunks;
 }
@@ -328,9 +322,12 @@ size_t carve(const Layout &L, char *base, size_t cap, Dev &d, void **io, int *io
     d.t_col = a.take<int>(L.slots);
     d.t_pos = a.take<int>(L.slots);
     d.bucket = a.take<int>(L.atoms_w);
-    d.sub_hdr = a.take<int2>(L.scs * (long long)L.ncs * L.sub_cap);
-    d.sub_lb = a.take<unsigned char>(32 * L.scs * (long long)L.ncs * L.sub_cap);
-    d.sub_n = a.take<int>(L.scs * (long long)L.ncs);
+    d.lcode = a.take<int>(L.slots);
+    d.lb_tot = a.take<int>(3);
+    d.lb_w = a.take<int>(L.W);
+    d.lb_apre = a.take<int>(L.W);
+    d.lb_spre = a.take<int>(L.W);
+    d.lb_done = a.take<unsigned int>(L.W);
     const int iof = std::max(IO_FLOATS_MIN, 8 * L.max_n);
     *io = a.take<float>(iof);
     *io_floats = iof;
@@ -723,8 +720,6 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     d.n_walkers = L.W;
     d.n_stages = L.n_stages;
     d.ent_cap = L.ent_cap;
-    d.ncs = L.ncs;
-    d.sub_cap = L.sub_cap;
     d.alch_cap = L.alch_cap;
     d.max_bins = L.max_bins;
     d.P_max = L.P_max;
@@ -996,7 +991,6 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     HostView &hv = h->hv;
     hv.n_walkers = L.W;
     hv.n_sm = h->n_sm;
-    hv.ncs = L.ncs;
     hv.slot_off = h->slot_off.data();
     hv.slot_cap = h->slot_cap.data();
     hv.sc_cap = h->sc_cap.data();

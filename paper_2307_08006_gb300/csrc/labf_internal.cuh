@@ -131,6 +131,12 @@ struct Dev {
     int *t_old;
     int4 *t_uq;
     int *t_col, *t_pos, *bucket;
+    int *lcode;                   // per slot: exclusion group | extra-partner flag, -1: no normal pairs
+    // the list kernel's plan: totals (walkers that rebuild, their alchemical
+    // atoms, their super-clusters), those walkers, the prefixes of both, and
+    // per walker the super-clusters finished
+    int *lb_tot, *lb_w, *lb_apre, *lb_spre;
+    unsigned int *lb_done;
     // per walker atoms
     int *slot_of_atom;
     // columns and super-clusters
@@ -141,12 +147,6 @@ struct Dev {
     int *sc_nent;
     int2 *ent_hdr;                // (j-cluster base global slot, shift bits | imask << 8)
     unsigned char *ent_lb;        // 32 per entry: lane l's bit ic = pair (8 ic + (l & 7), l >> 3)
-    // per (super-cluster, candidate column) sub-lists written by the list
-    // builder and compacted into ent_* in a fixed order
-    int ncs, sub_cap;
-    int2 *sub_hdr;
-    unsigned char *sub_lb;
-    int *sub_n;
     int4 *items;                  // (global sc, e0, e1, walker)
     int *n_items;
     // alchemical lists and partial sums
@@ -240,6 +240,33 @@ __device__ __forceinline__ float fix_to_float(unsigned long long v) {
     const int hi = (int)(v >> 32);
     const unsigned lo = (unsigned)(v & 0xffffffffull);
     return fmaf((float)lo, FIX_TO_F, (float)hi);
+}
+
+// Packed FP32 pairs (two IEEE results per instruction, each rounded as the
+// scalar instruction rounds it).
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f2 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
 __device__ __forceinline__ float min_image(float dx, float L, float Linv) {

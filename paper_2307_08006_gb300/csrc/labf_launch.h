@@ -11,7 +11,7 @@ namespace labf {
 
 // Host copies of the per-walker offsets the launchers size grids with.
 struct HostView {
-    int n_walkers = 0, n_sm = 0, pair_blocks = 0, ncs = 1;
+    int n_walkers = 0, n_sm = 0, pair_blocks = 0;
     int pair_variant = 0;  // 0: 8 warps/CTA, 80 regs; 1: 4 warps, 72; 2: 4 warps, 64
     const int *slot_off = nullptr, *slot_cap = nullptr, *sc_cap = nullptr, *n_cols = nullptr;
     const int *alch_base = nullptr, *n_alch = nullptr, *item_cap = nullptr;
