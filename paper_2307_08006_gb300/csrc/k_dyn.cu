@@ -160,7 +160,17 @@ __global__ void k_bonded(Dev d, int w0, int w1) {
     const int b0 = d.walk[w0].bo_off;
     const int b1 = d.walk[w1 - 1].bo_off + d.walk[w1 - 1].n_bo;
     const int nthr = gridDim.x * blockDim.x;
-    for (int t = b0 + blockIdx.x * blockDim.x + threadIdx.x; t < b1; t += nthr) bonded_term<ENERGY>(d, t, w0, w1);
+    // warps run together (32 terms at a time) for the energy sums
+    for (int tw = b0 + blockIdx.x * blockDim.x + (threadIdx.x & ~31); tw < b1; tw += nthr) {
+        const int t = tw + (threadIdx.x & 31);
+        long long fix = 0;
+        int key = -1;
+        if (t < b1) bonded_term<ENERGY>(d, t, w0, w1, fix, key);
+        if (ENERGY) {
+            __syncwarp();
+            add_energies(d, fix, key);
+        }
+    }
 }
 
 // walker terms, one warp per walker
@@ -170,10 +180,8 @@ __global__ void k_walker(Dev d, int w0, int w1) {
     if (w < w1) walker_work<ENERGY>(d, w, threadIdx.x & 31);
 }
 
-// ABF fold / bias / final B of lambda, one block per stage
-__global__ void k_lambda(Dev d, int s0, int prime) {
-    lambda_work<false>(d, s0 + blockIdx.x, prime, threadIdx.x, blockDim.x);
-}
+// ABF fold / bias / final B of lambda, one warp per stage
+__global__ void k_lambda(Dev d, int s0, int prime) { lambda_work<false>(d, s0 + blockIdx.x, prime, threadIdx.x); }
 
 // ---------------------------------------------------------------------------
 // host launchers
@@ -209,7 +217,7 @@ void launch_walker(const Dev &d, int w0, int w1, bool energy, cudaStream_t s) {
 }
 
 void launch_lambda(const Dev &d, int s0, int s1, bool prime, cudaStream_t s) {
-    k_lambda<<<s1 - s0, 128, 0, s>>>(d, s0, prime ? 1 : 0);
+    k_lambda<<<s1 - s0, 32, 0, s>>>(d, s0, prime ? 1 : 0);
 }
 
 }  // namespace labf

@@ -56,7 +56,7 @@ struct PairShared {
     float4 jx[WARPS][EPC][JC];  // prepared j-atoms (shift applied)
     float2 jl[WARPS][EPC][JC];
     unsigned char lb[WARPS][EPC][32];
-    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1];
+    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], first;
 };
 
 // counters[4] hands out work items; counters[5] counts warps that found no
@@ -139,8 +139,8 @@ __device__ __forceinline__ void flush_j2(const Dev &d, int gjA, int gjB, bool ha
 // ballot per tile), which later steps read; every tile that is skipped adds
 // exact zeros, so results do not depend on the pruning.
 template <bool ENERGY, int WARPS, int MSHIFT, bool PRUNE>
-__device__ __forceinline__ void item_entries(const Dev &d, PairShared<WARPS> &sh, const SysDev &S, int4 it, int gS,
-                                             float &elj, float &erf, int &npair) {
+__device__ __forceinline__ int item_entries(const Dev &d, PairShared<WARPS> &sh, const SysDev &S, int4 it, int gS,
+                                            float &elj, float &erf, int &npair) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int ia = lane & 7, jb = lane >> 3;
     const float L = S.boxf, rc2 = S.rc2, krf2 = 2.0f * S.krf, krf = S.krf, crf = S.crf;
@@ -149,6 +149,7 @@ __device__ __forceinline__ void item_entries(const Dev &d, PairShared<WARPS> &sh
 #pragma unroll
     for (int ic = 0; ic < NIC; ++ic) fi[ic][0] = fi[ic][1] = fi[ic][2] = 0.f;
     unsigned touched = 0;
+    int v_next = 0;
     const size_t ebase = (size_t)it.x * d.ent_cap;
     for (int eb = it.y; eb < it.z; eb += EPC) {
         const int ne = min(EPC, it.z - eb);
@@ -259,19 +260,22 @@ __device__ __forceinline__ void item_entries(const Dev &d, PairShared<WARPS> &sh
             }
             flush_j2(d, gA, gB, two, ia, a, b);
         }
+        // the next item's index, fetched just before the last flush: its round
+        // trip is hidden, and no warp holds an item it cannot start yet
+        if (eb + EPC >= it.z && lane == 0) v_next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
         flush_i(d, gS, ia, jb, touched, fi);  // every 32 entries (EPC)
         touched = 0;
         if (PRUNE && lane < ne) d.ent_hdr[ebase + eb + lane].y = (hy_l & ~0xff00) | (int)(keep_l << 8);
     }
+    return v_next;
 }
 
 // the re-pruning form, out of line: the common form's code stays as it is
 template <int WARPS>
-__device__ __noinline__ void item_entries_prune(const Dev &d, PairShared<WARPS> &sh, const SysDev &S, int4 it,
-                                                int gS) {
+__device__ __noinline__ int item_entries_prune(const Dev &d, PairShared<WARPS> &sh, const SysDev &S, int4 it, int gS) {
     float elj = 0.f, erf = 0.f;
     int npair = 0;
-    item_entries<false, WARPS, 8, true>(d, sh, S, it, gS, elj, erf, npair);
+    return item_entries<false, WARPS, 8, true>(d, sh, S, it, gS, elj, erf, npair);
 }
 
 // work items of the normal pairs, handed out by a global counter
@@ -280,14 +284,10 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int n
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nw = w1 - w0;
     const int total = sh.pre[nw];
-    // the next item's index is fetched one item ahead, so that the atomic's
-    // round trip overlaps the current item's work
-    int v_next = 0;
-    if (lane == 0) v_next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
+    int v_next = sh.first + wib;  // the block's first items came with one atomic
     for (;;) {
         const int v = __shfl_sync(FULL, v_next, 0);
         if (v >= total) break;
-        if (lane == 0) v_next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
         int lo = 0, hi = nw - 1;
         while (lo < hi) {
             int mid = (lo + hi + 1) >> 1;
@@ -297,8 +297,10 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int n
         const WalkerDev &W = d.walk[w];
         const SysDev &S = d.sys[W.sys];
         const int4 it = d.items[W.item_base + (v - sh.pre[lo])];
-        if (!la_in(d, it.x - W.sc_off, W.sc_cap) || !la_in(d, it.z - 1, d.ent_cap) || !la_in(d, it.y, it.z))
-            continue;  // item skipped
+        if (!la_in(d, it.x - W.sc_off, W.sc_cap) || !la_in(d, it.z - 1, d.ent_cap) || !la_in(d, it.y, it.z)) {  // item skipped
+            if (lane == 0) v_next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
+            continue;
+        }
         const int sc = it.x;
         const int gS = W.slot_off + (sc - W.sc_off) * SC;
         __syncwarp();
@@ -308,8 +310,8 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int n
         sh.slj[wib][lane + 32] = d.lj[gS + lane + 32];
         float elj = 0.f, erf = 0.f;
         int npair = 0;
-        if (MSHIFT == 8 && d.prune_now[w] != 0ull) item_entries_prune<WARPS>(d, sh, S, it, gS);
-        else item_entries<ENERGY, WARPS, MSHIFT, false>(d, sh, S, it, gS, elj, erf, npair);
+        if (MSHIFT == 8 && d.prune_now[w] != 0ull) v_next = item_entries_prune<WARPS>(d, sh, S, it, gS);
+        else v_next = item_entries<ENERGY, WARPS, MSHIFT, false>(d, sh, S, it, gS, elj, erf, npair);
         if (ENERGY) {
             const double el = warp_sum((double)elj), er = warp_sum((double)erf);
             int np = npair;
@@ -336,59 +338,70 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int n
     }
 }
 
-// Fused launch: a walker's terms (walker_work) need all its alchemical
-// items, and a stage's lambda update (lambda_work) needs all its walkers.
-// Each finished item, plus one extra trigger item per walker, arrives on
-// the walker's counter; the warp that arrives last does the walker's work and
-// arrives on the stage's counter, whose last arrival does the stage's work.
-// Writers fence before arriving; counters are reset by the last arrival.
-// No warp waits for another.
-__device__ __forceinline__ void arrive_walker(const Dev &d, int w, int lane) {
-    __threadfence();
-    unsigned old = 0;
-    if (lane == 0) old = atomicAdd(&d.wdone[w], 1u);
-    old = __shfl_sync(FULL, old, 0);
-    const WalkerDev &W = d.walk[w];
-    if (old != (unsigned)d.sys[W.sys].n_alch) return;  // n_alch + 1 arrivals
-    if (lane == 0) d.wdone[w] = 0u;
-    __threadfence();
-    walker_work<false>(d, w, lane);
-    __threadfence();
-    const int si = W.stage;
+// Fused launch: a stage's lambda update (lambda_work) needs the partial sums
+// of all its walkers' alchemical items and their restraint terms.  Each
+// finished item, plus one restraint item per walker, arrives on the stage's
+// counter; the warp that arrives last does the stage's work (a writer's lane
+// fences before it arrives; the counter is reset by the last arrival).  No
+// warp waits for another.  One hand-off instead of two (walker, then stage)
+// and the restraints beside the alchemical items shorten the chain that ends
+// a launch of a small system.
+__device__ __forceinline__ void arrive_stage(const Dev &d, int w, int lane) {
+    const int si = d.walk[w].stage;
     const StageDev &st = d.stage[si];
-    unsigned old2 = 0;
-    if (lane == 0) old2 = atomicAdd(&d.sdone[si], 1u);
-    old2 = __shfl_sync(FULL, old2, 0);
-    if (old2 != (unsigned)(st.w1 - st.w0 - 1)) return;
+    const unsigned last = (unsigned)((st.w1 - st.w0) * (d.sys[st.sys].n_alch + 1)) - 1u;
+    __syncwarp();
+    unsigned old = 0;
+    if (lane == 0) {
+        __threadfence();
+        old = atomicAdd(&d.sdone[si], 1u);
+    }
+    old = __shfl_sync(FULL, old, 0);
+    if (old != last) return;
     if (lane == 0) d.sdone[si] = 0u;
     __threadfence();
-    lambda_work<true>(d, si, 0, lane, 32);
+    lambda_work<true>(d, si, 0, lane);
 }
 
+// walker in [w0, w1) that owns alchemical item it: the last one whose first
+// item is not beyond it (32 walkers per load)
+__device__ __forceinline__ int walker_of_alch(const Dev &d, int w0, int w1, int it, int lane) {
+    int n = 0;
+    for (int b = w0; b < w1; b += 32)
+        n += __popc(__ballot_sync(FULL, b + lane < w1 && d.walk[min(b + lane, w1 - 1)].alch_base <= it));
+    return w0 + n - 1;
+}
+
+// Alchemical items [a0, a1), one warp each, then (FUSED) one restraint item
+// per walker; unit `unit` of `units` takes every units-th item.
 template <bool ENERGY, int WARPS, bool FUSED>
-__device__ __forceinline__ void alch_items(const Dev &d, int w0, int w1, int a0, int a1, int blk, int nblk) {
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int nwarps = nblk * WARPS;
+__device__ __forceinline__ void alch_items(const Dev &d, int w0, int w1, int a0, int a1, int unit, int units) {
+    const int lane = threadIdx.x & 31;
     const int aend = FUSED ? a1 + (w1 - w0) : a1;
-    for (int it = a0 + blk * WARPS + wib; it < aend; it += nwarps) {
-        if (FUSED && it >= a1) {  // trigger item of walker w0 + (it - a1)
-            arrive_walker(d, w0 + (it - a1), lane);
+    for (int it = a0 + unit; it < aend; it += units) {
+        if (FUSED && it >= a1) {  // restraint item of walker w0 + (it - a1)
+            walker_restraints(d, w0 + (it - a1), lane);
+            arrive_stage(d, w0 + (it - a1), lane);
             continue;
         }
-        int lo = w0, hi = w1 - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (d.walk[mid].alch_base <= it) lo = mid; else hi = mid - 1;
-        }
-        const int w = lo;
+        const int w = walker_of_alch(d, w0, w1, it, lane);
         const WalkerDev &W = d.walk[w];
         const SysDev &S = d.sys[W.sys];
+        const bool derivs = ENERGY || S.theta_stats;
         const int r = it - W.alch_base;
         int a = d.alch_atoms[S.alch_off + r];
         bool item_ok = la_in(d, a, S.n_atoms);
         if (!item_ok) a = 0;
         int ga = d.slot_of_atom[W.atom_base + a];
         if (!la_in(d, ga, d.n_slots)) ga = W.slot_off, item_ok = false;  // no pairs, still arrives
+        const int cnt = item_ok ? d.alch_cnt[it] : 0;
+        const int *lst = d.alch_slot + (size_t)it * d.alch_cap;
+        // the list is read two rounds ahead and the environment atoms one round
+        // ahead of the arithmetic
+        auto slot_at = [&](int k) { return k < cnt ? checked_slot(d, lst[k]) : ga; };
+        int gb = slot_at(lane), gb_next = slot_at(lane + 32);
+        float4 xb = d.xq[gb];
+        float2 lb = d.lj[gb];
         const float4 xa = d.xq[ga];
         const float2 la = d.lj[ga];
         double lvd, led, dlvd, dled;
@@ -401,33 +414,34 @@ __device__ __forceinline__ void alch_items(const Dev &d, int w0, int w1, int a0,
         const float sa = (float)((double)S.sc_alpha * ipow(1.0 - lvd, S.sc_m));
         const float dsdl = (float)(-(double)S.sc_m * S.sc_alpha * ipow(1.0 - lvd, S.sc_m - 1));
         const float eps_a = 0.25f * la.y * la.y;
-        const double inv2eps = 0.5 / (double)eps_a;  // d e4 / d eps_a = e4 / (2 eps_a)
+        const double inv2eps = derivs ? 0.5 / (double)eps_a : 0.0;  // d e4 / d eps_a = e4 / (2 eps_a)
         const float rc2 = S.rc2, krf = S.krf, crf = S.crf;
         float fax = 0.f, fay = 0.f, faz = 0.f;
         double sv = 0.0, se = 0.0, usc_s = 0.0, urf_s = 0.0;
         double th0 = 0.0, th1 = 0.0, th2 = 0.0, th3 = 0.0, th4 = 0.0, th5 = 0.0;
         int npair = 0;
-        const int cnt = item_ok ? d.alch_cnt[it] : 0;
-        const int *lst = d.alch_slot + (size_t)it * d.alch_cap;
-        for (int k = lane; k < cnt; k += 32) {
-            const int gb = lst[k];
-            if (!la_in(d, gb, d.n_slots)) continue;
-            const float4 xb = d.xq[gb];
-            const float2 lb = d.lj[gb];
-            const float dx = min_image(xa.x - xb.x, S.boxf, S.box_invf);
-            const float dy = min_image(xa.y - xb.y, S.boxf, S.box_invf);
-            const float dz = min_image(xa.z - xb.z, S.boxf, S.box_invf);
+        for (int k = lane; __any_sync(FULL, k < cnt); k += 32) {
+            const float4 xc = xb;
+            const float2 lc = lb;
+            const int gc = gb;
+            gb = gb_next;
+            xb = d.xq[gb];
+            lb = d.lj[gb];
+            gb_next = slot_at(k + 64);
+            const float dx = min_image(xa.x - xc.x, S.boxf, S.box_invf);
+            const float dy = min_image(xa.y - xc.y, S.boxf, S.box_invf);
+            const float dz = min_image(xa.z - xc.z, S.boxf, S.box_invf);
             const float r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 >= rc2) continue;
+            if (k >= cnt || r2 >= rc2) continue;
             ++npair;
             const float rinv = rsqrtf(r2);
             const float r2inv = rinv * rinv;
             const float rf_shape = rinv + krf * r2 - crf;
-            const float qq = xa.w * xb.w;
+            const float qq = xa.w * xc.w;
             const float rf_u = qq * rf_shape;
             const float rf_f = qq * (rinv * r2inv - 2.0f * krf);
-            const float sg = la.x + lb.x;
-            const float e4 = la.y * lb.y;
+            const float sg = la.x + lc.x;
+            const float e4 = la.y * lc.y;
             float sc_f = 0.f, usc = 0.f, dsc = 0.f, g = 0.f, g1 = 0.f, g2 = 0.f, rho6 = 0.f;
             if (e4 > 0.f) {
                 const float q2 = r2 / (sg * sg);
@@ -445,12 +459,14 @@ __device__ __forceinline__ void alch_items(const Dev &d, int w0, int w1, int a0,
             fax = fmaf(fs, dx, fax);
             fay = fmaf(fs, dy, fay);
             faz = fmaf(fs, dz, faz);
-            add_force(d, gb, -fs * dx, -fs * dy, -fs * dz);
+            add_force(d, gc, -fs * dx, -fs * dy, -fs * dz);
             sv += (double)dsc;
             se += (double)rf_u;
-            usc_s += (double)usc;
-            urf_s += (double)(le * rf_u);
-            if (S.theta_stats || ENERGY) {
+            if (ENERGY) {
+                usc_s += (double)usc;
+                urf_s += (double)(le * rf_u);
+            }
+            if (derivs) {
                 if (e4 > 0.f) {
                     th0 += (double)usc * inv2eps;
                     th3 += (double)dsc * inv2eps;
@@ -459,7 +475,7 @@ __device__ __forceinline__ void alch_items(const Dev &d, int w0, int w1, int a0,
                     th4 += 0.5 * (double)(dlvn * e4 * g1 * ds_dsig + lvn * e4 * g2 * ds_dsig * dsdl);
                 }
                 // d/dq_a of coul q_a q_b shape = sqrt(coul) * (q_b sqrt(coul)) * shape
-                const float qb_c = S.sqrt_coul * xb.w;
+                const float qb_c = S.sqrt_coul * xc.w;
                 th2 += (double)(le * qb_c * rf_shape);
                 th5 += (double)(qb_c * rf_shape);
             }
@@ -469,9 +485,11 @@ __device__ __forceinline__ void alch_items(const Dev &d, int w0, int w1, int a0,
         faz = warp_sumf(faz);
         sv = warp_sum(sv);
         se = warp_sum(se);
-        usc_s = warp_sum(usc_s);
-        urf_s = warp_sum(urf_s);
-        if (S.theta_stats || ENERGY) {
+        if (ENERGY) {
+            usc_s = warp_sum(usc_s);
+            urf_s = warp_sum(urf_s);
+        }
+        if (derivs) {
             th0 = warp_sum(th0); th1 = warp_sum(th1); th2 = warp_sum(th2);
             th3 = warp_sum(th3); th4 = warp_sum(th4); th5 = warp_sum(th5);
         }
@@ -480,19 +498,21 @@ __device__ __forceinline__ void alch_items(const Dev &d, int w0, int w1, int a0,
             for (int o = 16; o > 0; o >>= 1) npair += __shfl_xor_sync(FULL, npair, o);
         }
         if (lane == 0) {
-            add_force(d, ga, fax, fay, faz);
             double *o = d.alch_out + 4 * (size_t)it;
             o[0] = sv;
             o[1] = se;
-            o[2] = usc_s;
-            o[3] = urf_s;
-            if (S.theta_stats || ENERGY) {
+            if (ENERGY) {
+                o[2] = usc_s;
+                o[3] = urf_s;
+            }
+            if (derivs) {
                 double *t = d.alch_th + 6 * (size_t)it;
                 t[0] = th0; t[1] = th1; t[2] = th2; t[3] = th3; t[4] = th4; t[5] = th5;
             }
             if (ENERGY) atomicAdd(&d.counters[2], (unsigned long long)npair);
         }
-        if (FUSED) arrive_walker(d, w, lane);
+        if (FUSED) arrive_stage(d, w, lane);
+        if (lane == 0) add_force(d, ga, fax, fay, faz);
     }
 }
 
@@ -501,7 +521,11 @@ __device__ __forceinline__ void bonded_items(const Dev &d, int w0, int w1, int b
     const int b0 = d.walk[w0].bo_off;
     const int b1 = d.walk[w1 - 1].bo_off + d.walk[w1 - 1].n_bo;
     const int nthr = nblk * blockDim.x;
-    for (int t = b0 + blk * blockDim.x + threadIdx.x; t < b1; t += nthr) bonded_term<false>(d, t, w0, w1);
+    for (int t = b0 + blk * blockDim.x + threadIdx.x; t < b1; t += nthr) {
+        long long fix;
+        int key;
+        bonded_term<false>(d, t, w0, w1, fix, key);
+    }
 }
 
 // WARPS x 32 threads per CTA; MINB: resident CTAs per SM the register
@@ -509,26 +533,40 @@ __device__ __forceinline__ void bonded_items(const Dev &d, int w0, int w1, int b
 // registers), 4 warps / 7 CTAs (72), 4 warps / 8 CTAs (64).
 template <bool ENERGY, int WARPS, int MINB, bool FUSED>
 __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w1, int nblk_pairs, int a0, int a1,
-                                                          int nblk_bonded) {
+                                                          int nblk_bonded, int alch_warps) {
     __shared__ PairShared<WARPS> sh;
-    // grid: [alchemical items][bonded terms][normal pairs]; the first two
-    // come first so that they run alongside the normal pairs
+    // grid: [alchemical items][bonded terms][normal pairs]; the first two come
+    // first so that they run alongside the normal pairs.  (The alchemical
+    // blocks return here: when their warps went on to the normal pairs, the
+    // compiler treated the pair loop as divergent code, 10% more instructions.)
     const int nblk_alch = gridDim.x - nblk_pairs - nblk_bonded;
     if ((int)blockIdx.x < nblk_alch) {
-        alch_items<ENERGY, WARPS, FUSED>(d, w0, w1, a0, a1, blockIdx.x, nblk_alch);
+        if ((int)(threadIdx.x >> 5) < alch_warps)
+            alch_items<ENERGY, WARPS, FUSED>(d, w0, w1, a0, a1, (threadIdx.x >> 5) * nblk_alch + blockIdx.x,
+                                             alch_warps * nblk_alch);
         return;
     }
     if (FUSED && (int)blockIdx.x < nblk_alch + nblk_bonded) {
         bonded_items(d, w0, w1, blockIdx.x - nblk_alch, nblk_bonded);
         return;
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {  // prefix of the walkers' work items
         int acc = 0;
-        for (int w = w0; w < w1; ++w) {
-            sh.pre[w - w0] = acc;
-            acc += d.n_items[w];
+        for (int b = 0; b < w1 - w0; b += 32) {
+            const int k = b + threadIdx.x, n = k < w1 - w0 ? d.n_items[w0 + k] : 0;
+            int x = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(FULL, x, o);
+                if ((int)threadIdx.x >= o) x += t;
+            }
+            if (k < w1 - w0) sh.pre[k] = acc + x - n;
+            acc += __shfl_sync(FULL, x, 31);
         }
-        sh.pre[w1 - w0] = acc;
+        if (threadIdx.x == 0) {
+            sh.pre[w1 - w0] = acc;
+            sh.first = (int)atomicAdd(&d.counters[CTR_ITEM], (unsigned long long)WARPS);
+        }
     }
     __syncthreads();
     normal_items<ENERGY, WARPS, FUSED ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
@@ -545,7 +583,14 @@ static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cud
         nblk = nblk < 1 ? 1 : nblk;
     }
     const int a0 = hv.alch_base[w0], a1 = hv.alch_base[w1 - 1] + hv.n_alch[w1 - 1];
-    const int ablk = (a1 - a0 + (fused ? w1 - w0 : 0) + WARPS - 1) / WARPS;
+    // alchemical warps per block: one, or as few as keep the blocks at one per
+    // SM.  They live on FP64 sums, and an SM's FP64 pipe does 1.9 lanes per
+    // clock: eight of them in one block took turns on it (42 instead of 30 us
+    // for the fused launch of 8 walkers x 772 atoms with theta statistics).
+    const int aitems = a1 - a0 + (fused ? w1 - w0 : 0);
+    int awarps = (aitems + hv.n_sm - 1) / hv.n_sm;
+    awarps = awarps < 1 ? 1 : (awarps > WARPS ? WARPS : awarps);
+    const int ablk = (aitems + awarps - 1) / awarps;
     int bblk = 0;
     if (fused) {  // bonded terms: about four per thread
         const int nbo = hv.bo_off[w1 - 1] + hv.n_bo[w1 - 1] - hv.bo_off[w0];
@@ -553,8 +598,8 @@ static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cud
         bblk = bblk > hv.n_sm ? hv.n_sm : bblk;
     }
     const int grid = ablk + bblk + nblk;
-    if (fused) k_pairs<ENERGY, WARPS, MINB, true><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, bblk);
-    else k_pairs<ENERGY, WARPS, MINB, false><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, 0);
+    if (fused) k_pairs<ENERGY, WARPS, MINB, true><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, bblk, awarps);
+    else k_pairs<ENERGY, WARPS, MINB, false><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, 0, awarps);
 }
 
 void launch_pairs_fused(const Dev &d, const HostView &hv, int n_stages, cudaStream_t s) {

@@ -311,7 +311,7 @@ size_t carve(const Layout &L, char *base, size_t cap, Dev &d, void **io, int *io
     d.th_sd = a.take<double>((size_t)L.total_bins * L.P_max);
     d.status = a.take<unsigned int>(4);
     d.counters = a.take<unsigned long long>(16);
-    d.wdone = a.take<unsigned int>(L.W);
+    a.take<unsigned int>(L.W);  // unused; keeps the state prefix as older checkpoints have it
     d.sdone = a.take<unsigned int>(L.n_stages);
     if (state_bytes) *state_bytes = (a.off + ALIGN - 1) / ALIGN * ALIGN;
     // scratch: rewritten before every use
@@ -323,6 +323,7 @@ size_t carve(const Layout &L, char *base, size_t cap, Dev &d, void **io, int *io
     d.t_pos = a.take<int>(L.slots);
     d.bucket = a.take<int>(L.atoms_w);
     d.lcode = a.take<int>(L.slots);
+    d.wdir = a.take<double>(4 * (size_t)L.W);
     d.lb_tot = a.take<int>(3);
     d.lb_w = a.take<int>(L.W);
     d.lb_apre = a.take<int>(L.W);

@@ -8,10 +8,10 @@ namespace labf {
 // ---------------------------------------------------------------------------
 // bonds (1/2 k (r - r0)^2), angles (1/2 k (theta - theta0)^2) and positional
 // restraints (1/2 k |x - x0|^2): term t of the bonded items of walkers
-// [w0, w1)
+// [w0, w1); with ENERGY the term's energy in fixed point and its index
 // ---------------------------------------------------------------------------
 template <bool ENERGY>
-__device__ __forceinline__ void bonded_term(const Dev &d, int t, int w0, int w1) {
+__device__ __forceinline__ void bonded_term(const Dev &d, int t, int w0, int w1, long long &fix, int &key) {
     int lo = w0, hi = w1 - 1;  // walker owning item t
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
@@ -82,24 +82,48 @@ __device__ __forceinline__ void bonded_term(const Dev &d, int t, int w0, int w1)
             eterm = 6;
         }
     }
-    if (ENERGY) atomicAdd((unsigned long long *)&d.eterm[N_ETERMS * w + eterm],
-                          (unsigned long long)__double2ll_rn((double)e * E_TO_FIX));
+    if (ENERGY) {
+        fix = __double2ll_rn((double)e * E_TO_FIX);
+        key = N_ETERMS * w + eterm;
+    }
+}
+
+// adds the lanes' fixed-point energies (key: index of eterm, -1: none) with
+// one atomic per warp and kind of term; integer sums give the same bits in any
+// order.  Per-term atomics on one address took 14-22 us for 16 k-33 k terms.
+__device__ __forceinline__ void add_energies(const Dev &d, long long fix, int key) {
+    constexpr unsigned ALL = 0xffffffffu;
+    for (unsigned rest = __ballot_sync(ALL, key >= 0); rest;) {
+        const int k0 = __shfl_sync(ALL, key, __ffs(rest) - 1);
+        const bool in = key == k0;
+        // 26-bit pieces: 32 of them fit a 32-bit sum
+        const unsigned lo = __reduce_add_sync(ALL, in ? (unsigned)fix & 0x3ffffffu : 0u);
+        const unsigned mid = __reduce_add_sync(ALL, in ? (unsigned)(fix >> 26) & 0x3ffffffu : 0u);
+        const int hi = __reduce_add_sync(ALL, in ? (int)(fix >> 52) : 0);
+        if ((threadIdx.x & 31) == 0)
+            atomicAdd((unsigned long long *)&d.eterm[k0],
+                      ((unsigned long long)(long long)hi << 52) + ((unsigned long long)mid << 26) + lo);
+        rest &= ~__ballot_sync(ALL, in);
+    }
 }
 
 // ---------------------------------------------------------------------------
 // per walker, one warp: flat-bottom COM restraint, lambda-dependent distance
-// restraint, lambda-switched well, and the sum of the alchemical partials
-// into s = dU/dlambda.  Lane-strided loops and fixed shuffle trees: the
-// result is deterministic.  The alchemical partials may come from other SMs
-// of the same launch: they are read past L1.
+// restraint and lambda-switched well.  Their forces are added, and their
+// dU/dlambda, energy and k1 derivatives go to wdir (lane-strided loops and
+// fixed shuffle trees: the result is deterministic).  They need only the
+// positions and lambda, so the fused launch runs them beside the alchemical
+// items instead of after them.
 // ---------------------------------------------------------------------------
-template <bool ENERGY>
-__device__ __forceinline__ void walker_work(const Dev &d, int w, int lane) {
+__device__ __forceinline__ void walker_restraints(const Dev &d, int w, int lane) {
     const WalkerDev &W = d.walk[w];
     const SysDev &S = d.sys[W.sys];
+    double2 *out = reinterpret_cast<double2 *>(d.wdir + 4 * (size_t)w);
+    if (!(S.n_fb_a > 0 && S.n_fb_b > 0) && S.n_lr <= 0 && S.n_lh <= 0) {
+        if (lane < 2) out[lane] = make_double2(0.0, 0.0);
+        return;
+    }
     const int *soa = d.slot_of_atom + W.atom_base;
-    double lv, le, dlv, dle;
-    lambda_path(d.lam[w], S.b_v, S.b_e, lv, le, dlv, dle);
     double e_rest = 0.0;
 
     // ---- flat-bottom restraint on |COM_a - COM_b| ----
@@ -197,101 +221,224 @@ __device__ __forceinline__ void walker_work(const Dev &d, int w, int lane) {
     }
     const double v0 = warp_sum(dl_dir), v1 = warp_sum(e_lh) + e_rest, v2 = warp_sum(dk1), v3 = warp_sum(d2k1);
     if (lane == 0) {
-        // ---- s = dU/dlambda: alchemical partials in atom order ----
-        double sv = 0.0, se = 0.0, usc = 0.0, urf = 0.0;
-        for (int r = 0; r < S.n_alch; ++r) {
-            const double *o = d.alch_out + 4 * (size_t)(W.alch_base + r);
-            sv += __ldcg(o + 0);
-            se += __ldcg(o + 1);
-            usc += __ldcg(o + 2);
-            urf += __ldcg(o + 3);
-        }
-        d.s[w] = dlv * sv + dle * se + v0;
-        if (S.theta_stats || ENERGY) {
-            double *th = d.wth + (size_t)w * 2 * d.P_max;
-            for (int r = 0; r < S.n_alch; ++r) {
-                const double *o = d.alch_th + 6 * (size_t)(W.alch_base + r);
-                th[3 * r + 0] = __ldcg(o + 0);
-                th[3 * r + 1] = __ldcg(o + 1);
-                th[3 * r + 2] = __ldcg(o + 2);
-                th[d.P_max + 3 * r + 0] = dlv * __ldcg(o + 3);
-                th[d.P_max + 3 * r + 1] = dlv * __ldcg(o + 4);
-                th[d.P_max + 3 * r + 2] = dle * __ldcg(o + 5);
-            }
-            th[S.P - 1] = v2;
-            th[d.P_max + S.P - 1] = v3;
-        }
+        out[0] = make_double2(v0, v1);
+        out[1] = make_double2(v2, v3);
+    }
+}
+
+// dU/dlambda from the partials (one expression for every form of the step)
+__device__ __forceinline__ double sample_of(double dlv, double sv, double dle, double se, double direct) {
+    return __dadd_rn(__fma_rn(dlv, sv, __dmul_rn(dle, se)), direct);
+}
+
+// Sum over the walker's alchemical atoms of component c of their partial sums
+// (written by other SMs of the launch: read past L1), by four neighbouring
+// lanes: lane q of the four adds the atoms r = q mod 4 in order, then the
+// four are added as (0 + 1) + (2 + 3).  Every form of the step adds so, hence
+// the same bits.  Four short chains of FP64 adds and loads instead of one.
+__device__ __forceinline__ double alch_sum4(const Dev &d, int alch_base, int n_alch, int c, int q, bool on) {
+    const double *o = d.alch_out + 4 * (size_t)alch_base + c;
+    double v = 0.0;
+    if (on) {
+#pragma unroll 4
+        for (int r = q; r < n_alch; r += 4) v += __ldcg(o + 4 * r);
+    }
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 2);
+}
+
+// value and lambda derivative of theta parameter p (3 per alchemical atom,
+// then k1) of walker w
+__device__ __forceinline__ void theta_terms(const Dev &d, const WalkerDev &W, const SysDev &S, int w, int p, double dlv,
+                                            double dle, double &th, double &d2) {
+    if (p == S.P - 1) {
+        const double2 k1 = __ldcg(reinterpret_cast<const double2 *>(d.wdir + 4 * (size_t)w) + 1);
+        th = k1.x;
+        d2 = k1.y;
+        return;
+    }
+    const int r = p / 3, c = p - 3 * r;
+    const double *o = d.alch_th + 6 * (size_t)(W.alch_base + r) + c;
+    th = __ldcg(o);
+    d2 = (c < 2 ? dlv : dle) * __ldcg(o + 3);
+}
+
+// the walker's restraints and its sample, one warp (one-task launches); with
+// ENERGY also the energy terms and the theta derivatives
+template <bool ENERGY>
+__device__ __forceinline__ void walker_work(const Dev &d, int w, int lane) {
+    const WalkerDev &W = d.walk[w];
+    const SysDev &S = d.sys[W.sys];
+    double lv, le, dlv, dle;
+    lambda_path(d.lam[w], S.b_v, S.b_e, lv, le, dlv, dle);
+    walker_restraints(d, w, lane);
+    __syncwarp();
+    // four lanes per component
+    const double v = alch_sum4(d, W.alch_base, S.n_alch, (lane >> 2) & 3, lane & 3, lane < (ENERGY ? 16 : 8));
+    const double se = __shfl_sync(0xffffffffu, v, 4), usc = __shfl_sync(0xffffffffu, v, 8),
+                 urf = __shfl_sync(0xffffffffu, v, 12);
+    const double *dir = d.wdir + 4 * (size_t)w;
+    if (lane == 0) {
+        d.s[w] = sample_of(dlv, v, dle, se, __ldcg(dir));
         if (ENERGY) {
             long long *et = d.eterm + N_ETERMS * w;
             atomicAdd((unsigned long long *)&et[2], (unsigned long long)__double2ll_rn(usc * E_TO_FIX));
             atomicAdd((unsigned long long *)&et[3], (unsigned long long)__double2ll_rn(urf * E_TO_FIX));
-            atomicAdd((unsigned long long *)&et[6], (unsigned long long)__double2ll_rn(v1 * E_TO_FIX));
-            d.dl_direct[w] = v0;
+            atomicAdd((unsigned long long *)&et[6], (unsigned long long)__double2ll_rn(__ldcg(dir + 1) * E_TO_FIX));
+            d.dl_direct[w] = __ldcg(dir);
         }
+    }
+    if (ENERGY) {
+        double *th = d.wth + (size_t)w * 2 * d.P_max;
+        for (int p = lane; p < S.P; p += 32) theta_terms(d, W, S, w, p, dlv, dle, th[p], th[d.P_max + p]);
     }
 }
 
 // ---------------------------------------------------------------------------
 // ABF: fold the samples of a stage's walkers, merge every shared_freq steps,
-// bias = min(1, n/n_full) * mean, final B of lambda.
+// bias = min(1, n/n_full) * mean, final B of lambda.  One warp per stage,
+// lane = walker, 32 walkers at a time.
 // prime = 1: only G = -s + bias (no sample, no step).
+// SAMPLE: the samples are computed here from the alchemical partials (fused
+// launch), otherwise walker_work has left them in s.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double abf_bias(const Dev &d, const SysDev &S, const StageDev &st, int w) {
-    if (!S.abf_on) return 0.0;
-    const int k = bin_of(d.lam[w], st);
-    const size_t lk = (size_t)w * d.max_bins + k;
-    const double sum = d.abf_sum[st.bin_off + k] + d.dl_sum[lk];
-    const double cnt = (double)(d.abf_count[st.bin_off + k] + d.dl_count[lk]);
-    if (cnt <= 0.0) return 0.0;
+__device__ __forceinline__ double abf_bias(const SysDev &S, double sum, double cnt) {
+    if (!S.abf_on || cnt <= 0.0) return 0.0;
     return fmin(1.0, cnt / S.n_full) * sum / cnt;
 }
 
-template <bool WARP>
-__device__ __forceinline__ void group_sync() {
-    if (WARP) __syncwarp(); else __syncthreads();
-}
-
-// the work of stage si by a group of nt threads (a warp or a block); every
-// bin, parameter and walker is handled whole by one thread, so the result
-// does not depend on nt.  s and the theta samples may come from other SMs
-// of the same launch: they are read past L1.
-template <bool WARP>
-__device__ __forceinline__ void lambda_work(const Dev &d, int si, int prime, int tid, int nt) {
+template <bool SAMPLE>
+__device__ __forceinline__ void lambda_work(const Dev &d, int si, int prime, int lane) {
+    constexpr unsigned ALL = 0xffffffffu;
     const StageDev &st = d.stage[si];
-    if (st.w1 <= st.w0) return;  // (create refuses stages without walkers)
+    const int w0 = st.w0, nw = st.w1 - st.w0;
+    if (nw <= 0) return;  // (create refuses stages without walkers)
     const SysDev &S = d.sys[st.sys];
+    const int K = S.shared_freq;  // 0: merged only by the host (la_abf_import)
+    const bool one = nw <= 32;    // the walkers' values stay in registers
+    double s = 0.0, sum = 0.0, plam = 0.0;
+    unsigned long long cnt = 0, stepn = 0;
+    int k = -1;
     if (!prime) {
-        // fold each walker's sample into its own statistics (independent)
-        for (int w = st.w0 + tid; w < st.w1; w += nt) {
-            const int k = bin_of(d.lam[w], st);
-            const size_t lk = (size_t)w * d.max_bins + k;
-            const double sv = __ldcg(d.s + w);
-            d.dl_sum[lk] += sv;
-            d.dl_sumsq[lk] += sv * sv;
-            d.dl_count[lk] += 1ull;
-        }
-        // theta statistics: per parameter, walkers in order
-        if (S.theta_stats) {
-            for (int p = tid; p < S.P; p += nt) {
-                for (int w = st.w0; w < st.w1; ++w) {
-                    const size_t b = (size_t)(st.bin_off + bin_of(d.lam[w], st)) * d.P_max + p;
-                    const double *th = d.wth + (size_t)w * 2 * d.P_max;
-                    const double thp = __ldcg(th + p);
-                    d.th_d2[b] += __ldcg(th + d.P_max + p);
-                    d.th_d[b] += thp;
-                    d.th_sd[b] += __ldcg(d.s + w) * thp;
+        for (int b = 0; b < nw; b += 32) {
+            const int w = w0 + b + lane;
+            const bool on = b + lane < nw;
+            double dlv = 0.0, dle = 0.0;
+            k = -1;
+            s = 0.0;
+            double sv = 0.0, se = 0.0;
+            if (SAMPLE) {  // four lanes per walker, eight walkers at a time
+                for (int q = 0; q < 32 && b + q < nw; q += 8) {
+                    const int v = b + q + (lane >> 2);
+                    const bool von = v < nw;
+                    const int base = von ? d.walk[w0 + v].alch_base : 0;
+                    const double a = alch_sum4(d, base, S.n_alch, 0, lane & 3, von);
+                    const double e = alch_sum4(d, base, S.n_alch, 1, lane & 3, von);
+                    const double a8 = __shfl_sync(ALL, a, 4 * (lane & 7)), e8 = __shfl_sync(ALL, e, 4 * (lane & 7));
+                    if ((lane & 24) == q) {
+                        sv = a8;
+                        se = e8;
+                    }
+                }
+            }
+            if (on) {
+                const double lam = d.lam[w];
+                plam = d.plam[w];
+                stepn = d.step[w];
+                if (SAMPLE || S.theta_stats) {
+                    double lv, le;
+                    lambda_path(lam, S.b_v, S.b_e, lv, le, dlv, dle);
+                }
+                if (SAMPLE) {
+                    s = sample_of(dlv, sv, dle, se, __ldcg(d.wdir + 4 * (size_t)w));
+                    d.s[w] = s;
+                } else {
+                    s = __ldcg(d.s + w);
+                }
+                k = bin_of(lam, st);
+            }
+            if (K == 1) {
+                // every step merges: the walker-local statistics are zero before
+                // the fold and again after it, so the samples go straight to the
+                // shared ones, a bin's walkers in order by the bin's first lane
+                const unsigned grp = __match_any_sync(ALL, k);
+                const int lead = __ffs(grp) - 1;
+                const bool mine = on && lane == lead;
+                double s2 = 0.0;
+                if (mine) {
+                    sum = d.abf_sum[st.bin_off + k];
+                    s2 = d.abf_sumsq[st.bin_off + k];
+                    cnt = d.abf_count[st.bin_off + k];
+                }
+                for (unsigned rest = grp; __any_sync(ALL, mine && rest); rest &= rest - 1u) {
+                    const double v = __shfl_sync(ALL, s, rest ? __ffs(rest) - 1 : 0);
+                    if (mine && rest) {
+                        sum = __dadd_rn(sum, v);
+                        s2 = __dadd_rn(s2, __dmul_rn(v, v));
+                        ++cnt;
+                    }
+                }
+                if (mine) {
+                    d.abf_sum[st.bin_off + k] = sum;
+                    d.abf_sumsq[st.bin_off + k] = s2;
+                    d.abf_count[st.bin_off + k] = cnt;
+                }
+                sum = __shfl_sync(ALL, sum, lead);
+                cnt = __shfl_sync(ALL, cnt, lead);
+            } else if (on) {  // each walker's own statistics
+                const size_t lk = (size_t)w * d.max_bins + k;
+                d.dl_sum[lk] = __dadd_rn(d.dl_sum[lk], s);
+                d.dl_sumsq[lk] = __dadd_rn(d.dl_sumsq[lk], __dmul_rn(s, s));
+                d.dl_count[lk] += 1ull;
+            }
+            if (S.theta_stats) {
+                // per parameter (lane), walkers in order; a run of walkers in one
+                // bin keeps the bin's sums in registers
+                const int n = min(32, nw - b);
+                for (int p0 = 0; p0 < S.P; p0 += 32) {
+                    const int p = p0 + lane;
+                    int cur = -1;
+                    double t2 = 0.0, t1 = 0.0, ts = 0.0;
+                    for (int j = 0; j < n; ++j) {
+                        const int kj = __shfl_sync(ALL, k, j);
+                        const double sj = __shfl_sync(ALL, s, j), vj = __shfl_sync(ALL, dlv, j),
+                                     ej = __shfl_sync(ALL, dle, j);
+                        if (p >= S.P) continue;
+                        double th, d2;
+                        theta_terms(d, d.walk[w0 + b + j], S, w0 + b + j, p, vj, ej, th, d2);
+                        if (kj != cur) {
+                            if (cur >= 0) {
+                                const size_t q = (size_t)(st.bin_off + cur) * d.P_max + p;
+                                d.th_d2[q] = t2;
+                                d.th_d[q] = t1;
+                                d.th_sd[q] = ts;
+                            }
+                            const size_t q = (size_t)(st.bin_off + kj) * d.P_max + p;
+                            t2 = d.th_d2[q];
+                            t1 = d.th_d[q];
+                            ts = d.th_sd[q];
+                            cur = kj;
+                        }
+                        t2 += d2;
+                        t1 += th;
+                        ts += sj * th;
+                    }
+                    if (cur >= 0) {
+                        const size_t q = (size_t)(st.bin_off + cur) * d.P_max + p;
+                        d.th_d2[q] = t2;
+                        d.th_d[q] = t1;
+                        d.th_sd[q] = ts;
+                    }
                 }
             }
         }
-        group_sync<WARP>();
-        const unsigned long long stepn = d.step[st.w0] + 1ull;
-        const int K = S.shared_freq;  // 0: merged only by the host (la_abf_import)
-        if (K > 0 && stepn % (unsigned long long)K == 0ull) {
-            for (int k = tid; k < st.n_bins; k += nt) {
-                double s1 = d.abf_sum[st.bin_off + k], s2 = d.abf_sumsq[st.bin_off + k];
-                unsigned long long c = d.abf_count[st.bin_off + k];
-                for (int w = st.w0; w < st.w1; ++w) {
-                    const size_t lk = (size_t)w * d.max_bins + k;
+        __syncwarp();
+        if (K > 1 && (d.step[w0] + 1ull) % (unsigned long long)K == 0ull) {
+            for (int q = lane; q < st.n_bins; q += 32) {
+                double s1 = d.abf_sum[st.bin_off + q], s2 = d.abf_sumsq[st.bin_off + q];
+                unsigned long long c = d.abf_count[st.bin_off + q];
+                for (int w = w0; w < st.w1; ++w) {
+                    const size_t lk = (size_t)w * d.max_bins + q;
                     s1 += d.dl_sum[lk];
                     s2 += d.dl_sumsq[lk];
                     c += d.dl_count[lk];
@@ -299,19 +446,32 @@ __device__ __forceinline__ void lambda_work(const Dev &d, int si, int prime, int
                     d.dl_sumsq[lk] = 0.0;
                     d.dl_count[lk] = 0ull;
                 }
-                d.abf_sum[st.bin_off + k] = s1;
-                d.abf_sumsq[st.bin_off + k] = s2;
-                d.abf_count[st.bin_off + k] = c;
+                d.abf_sum[st.bin_off + q] = s1;
+                d.abf_sumsq[st.bin_off + q] = s2;
+                d.abf_count[st.bin_off + q] = c;
             }
         }
-        group_sync<WARP>();
+        __syncwarp();
     }
-    for (int w = st.w0 + tid; w < st.w1; w += nt) {
-        const double G = -__ldcg(d.s + w) + abf_bias(d, S, st, w);
+    for (int b = 0; b < nw; b += 32) {
+        const int w = w0 + b + lane;
+        if (b + lane >= nw) continue;
+        if (prime || !one) {
+            s = __ldcg(d.s + w);
+            k = bin_of(d.lam[w], st);
+            plam = d.plam[w];
+            stepn = d.step[w];
+        }
+        if (prime || !one || K != 1) {
+            const size_t lk = (size_t)w * d.max_bins + k;
+            sum = d.abf_sum[st.bin_off + k] + d.dl_sum[lk];
+            cnt = d.abf_count[st.bin_off + k] + d.dl_count[lk];
+        }
+        const double G = -s + abf_bias(S, sum, (double)cnt);
         d.G[w] = G;
         if (!prime) {
-            if (S.lambda_dynamics) d.plam[w] += 0.5 * S.dt_d * G;
-            d.step[w] += 1ull;
+            if (S.lambda_dynamics) d.plam[w] = plam + 0.5 * S.dt_d * G;
+            d.step[w] = stepn + 1ull;
             d.pending[w] = 1;
         }
     }

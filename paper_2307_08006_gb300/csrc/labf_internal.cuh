@@ -166,7 +166,8 @@ struct Dev {
     double *th_d2, *th_d, *th_sd;
     // status and counters
     unsigned int *status;
-    unsigned int *wdone, *sdone;  // arrivals per walker / per stage in the fused pair launch
+    unsigned int *sdone;          // arrivals per stage in the fused pair launch
+    double *wdir;                 // per walker: restraints' dU/dlambda, energy, dU/dk1, d2U/dl dk1
     float4 *xprune;               // positions at the last pruning, per slot
     int *prune;                   // per walker: pruning requested (displacement or fresh list)
     int *near;                    // per walker: an atom of its system moved NEAR_FRACTION skin/2
