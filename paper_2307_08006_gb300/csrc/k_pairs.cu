@@ -34,6 +34,8 @@
 #include "labf_internal.cuh"
 #include "labf_launch.h"
 
+#include <type_traits>
+
 namespace labf {
 
 constexpr int EPC = 32;  // entries prepared per pass (one per lane)
@@ -55,6 +57,18 @@ struct PairShared {
     float2 slj[WARPS][SC];
     float4 jx[WARPS][EPC][JC];  // prepared j-atoms (shift applied)
     float2 jl[WARPS][EPC][JC];
+    unsigned char lb[WARPS][EPC][32];
+    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], first;
+};
+
+// Shared memory of the latency form: the super-cluster's i-clusters two by
+// two (row (p, ia): atom ia of i-clusters 2p and 2p + 1 as {x x' y y'},
+// {z z' q q'}, {s s' e e'}) and the prepared j-atoms with every value twice
+// (position negated), so that packed operands are loaded as they are.
+template <int WARPS>
+struct PairSharedLat {
+    float4 si[WARPS][3][SC / 2];
+    float4 j[WARPS][EPC][3 * JC];
     unsigned char lb[WARPS][EPC][32];
     int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], first;
 };
@@ -110,7 +124,7 @@ __device__ __forceinline__ void flush_i(const Dev &d, int gS, int ia, int jb, un
 // Each sum is ((a0 + a4) + (a2 + a6)) + ((a1 + a5) + (a3 + a7)), whether or
 // not B is present.
 __device__ __forceinline__ void flush_j2(const Dev &d, int gjA, int gjB, bool has_b, int ia, const float (&a)[3],
-                                         const float (&b)[3]) {
+                                         const float (&b)[3], bool has_a = true) {
     const bool h4 = (ia & 4) != 0, h2 = (ia & 2) != 0, h1 = (ia & 1) != 0;
     float v[3];
 #pragma unroll
@@ -127,7 +141,7 @@ __device__ __forceinline__ void flush_j2(const Dev &d, int gjA, int gjB, bool ha
     const float kk = h1 ? w1 : w0, ss = h1 ? w0 : w1;
     const float c = kk + __shfl_xor_sync(FULL, ss, 1);
     const int comp = ia & 3;
-    if (comp < 3 && (!h4 || has_b)) atomicAdd(d.F + 3 * (size_t)(h4 ? gjB : gjA) + comp, f2fix(-c));
+    if (comp < 3 && (h4 ? has_b : has_a)) atomicAdd(d.F + 3 * (size_t)(h4 ? gjB : gjA) + comp, f2fix(-c));
 }
 
 // One work item's entries, prepared and evaluated 32 at a time; the
@@ -278,9 +292,197 @@ __device__ __noinline__ int item_entries_prune(const Dev &d, PairShared<WARPS> &
     return item_entries<false, WARPS, 8, true>(d, sh, S, it, gS, elj, erf, npair);
 }
 
-// work items of the normal pairs, handed out by a global counter
+// The same item for launches with few items (at most LAT_ITEMS_PER_SM per SM:
+// one or two boxes, small batches), where an item's own latency decides, not
+// the issue rate.  The eight tiles of an entry are evaluated without branches,
+// two i-clusters per packed FP32 instruction, so that their dependency chains
+// overlap; unlisted tiles add exact zeros, and every sum keeps the order of
+// the common form (i-forces: one entry after the other; j-forces: i-clusters
+// ascending), so the forces are the same bits.  The common form tests each
+// i-cluster and skips 46% of the tiles, with one chain at a time.
+template <int WARPS, int MSHIFT, bool PRUNE>
+__device__ __forceinline__ int item_entries_lat(const Dev &d, PairSharedLat<WARPS> &sh, const SysDev &S, int4 it, int gS) {
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int ia = lane & 7, jb = lane >> 3;
+    const float L = S.boxf, rc2 = S.rc2, rp2 = S.rprune2, krf2 = 2.0f * S.krf;
+    const f2 nkrf2 = pack2(-krf2, -krf2), c12 = pack2(12.f, 12.f), c6 = pack2(-6.f, -6.f);
+    f2 fi[NIC / 2][3];
+#pragma unroll
+    for (int p = 0; p < NIC / 2; ++p) fi[p][0] = fi[p][1] = fi[p][2] = 0ull;
+    unsigned touched = 0;
+    int v_next = 0;
+    const size_t ebase = (size_t)it.x * d.ent_cap;
+    for (int eb = it.y; eb < it.z; eb += EPC) {
+        const int ne = min(EPC, it.z - eb);
+        int gj_l = 0, hy_l = 0;
+        unsigned im_l = 0, keep_l = 0;
+        __syncwarp();
+        if (lane < ne) {
+            const int2 hdr = d.ent_hdr[ebase + eb + lane];
+            gj_l = hdr.x;
+            hy_l = hdr.y;
+            im_l = ((unsigned)hdr.y >> (PRUNE ? 16 : MSHIFT)) & 0xffu;
+            if (!la_in(d, gj_l, d.n_slots - JC + 1)) gj_l = 0, im_l = 0;  // entry skipped
+            const float sx = (float)((hdr.y & 3) - 1) * L;
+            const float sy = (float)(((hdr.y >> 2) & 3) - 1) * L;
+            const float sz = (float)(((hdr.y >> 4) & 3) - 1) * L;
+#pragma unroll
+            for (int q = 0; q < JC; ++q) {
+                const float4 x = d.xq[gj_l + q];
+                const float2 l = d.lj[gj_l + q];
+                const float nx = -(x.x + sx), ny = -(x.y + sy), nz = -(x.z + sz);
+                float4 *row = &sh.j[wib][lane][3 * q];
+                row[0] = make_float4(nx, nx, ny, ny);
+                row[1] = make_float4(nz, nz, x.w, x.w);
+                row[2] = make_float4(l.x, l.x, l.y, l.y);
+            }
+            const uint4 *src = reinterpret_cast<const uint4 *>(d.ent_lb + 32 * (ebase + eb + lane));
+            uint4 *dst = reinterpret_cast<uint4 *>(&sh.lb[wib][lane][0]);
+            dst[0] = src[0];
+            dst[1] = src[1];
+        }
+        unsigned emask = __ballot_sync(FULL, im_l != 0u);
+        __syncwarp();
+        auto entry = [&](int k, unsigned lb, float (&fj)[3]) {
+            const ulonglong2 *rj = reinterpret_cast<const ulonglong2 *>(&sh.j[wib][k][3 * jb]);
+            const ulonglong2 j0 = rj[0], j1 = rj[1], j2 = rj[2];
+            unsigned kb = 0;  // this lane's pairs within r_c + margin, per i-cluster
+            fj[0] = fj[1] = fj[2] = 0.f;
+#pragma unroll
+            for (int p = 0; p < NIC / 2; ++p) {
+                const ulonglong2 *si = reinterpret_cast<const ulonglong2 *>(&sh.si[wib][0][p * IC + ia]);
+                const ulonglong2 i0 = si[0], i1 = si[SC / 2], i2 = si[SC];
+                const unsigned b0 = 1u << (2 * p), b1 = 2u << (2 * p);
+                const f2 dx = add2(i0.x, j0.x), dy = add2(i0.y, j0.y), dz = add2(i1.x, j1.x);
+                const f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+                float r20, r21;
+                unpack2(r2, r20, r21);
+                if (PRUNE) {
+                    kb |= ((lb & b0) && r20 < rp2) ? b0 : 0u;
+                    kb |= ((lb & b1) && r21 < rp2) ? b1 : 0u;
+                }
+                const bool in0 = (lb & b0) && r20 < rc2, in1 = (lb & b1) && r21 < rc2;
+                const f2 rinv = pack2(rsqrtf(r20), rsqrtf(r21));
+                const f2 r2inv = mul2(rinv, rinv);
+                const f2 sg = add2(i2.x, j2.x);
+                const f2 sr2 = mul2(mul2(sg, sg), r2inv);
+                const f2 sr6 = mul2(mul2(sr2, sr2), sr2);
+                const f2 e4s6 = mul2(mul2(i2.y, j2.y), sr6);
+                const f2 qq = mul2(i1.y, j1.y);
+                const f2 b = fma2(qq, rinv, mul2(e4s6, fma2(c12, sr6, c6)));
+                float f0, f1;
+                unpack2(fma2(b, r2inv, mul2(qq, nkrf2)), f0, f1);
+                f0 = in0 ? f0 : 0.f;
+                f1 = in1 ? f1 : 0.f;
+                const f2 fs = pack2(f0, f1);
+                fi[p][0] = fma2(fs, dx, fi[p][0]);
+                fi[p][1] = fma2(fs, dy, fi[p][1]);
+                fi[p][2] = fma2(fs, dz, fi[p][2]);
+                float d0, d1;
+                unpack2(dx, d0, d1);
+                fj[0] = fmaf(f1, d1, fmaf(f0, d0, fj[0]));
+                unpack2(dy, d0, d1);
+                fj[1] = fmaf(f1, d1, fmaf(f0, d0, fj[1]));
+                unpack2(dz, d0, d1);
+                fj[2] = fmaf(f1, d1, fmaf(f0, d0, fj[2]));
+            }
+            if (PRUNE) {
+                const unsigned keep = __reduce_or_sync(FULL, kb);
+                keep_l = lane == k ? keep : keep_l;
+            }
+        };
+        touched = __reduce_or_sync(FULL, im_l);
+        // two entries per round (an odd last one runs with a copy of itself
+        // without pairs); the reduction of the round before shares the block
+        // with their arithmetic
+        float a[3] = {0.f, 0.f, 0.f}, b[3] = {0.f, 0.f, 0.f};
+        int gA = 0, gB = 0;
+        bool any = false, two = false;
+        while (emask) {
+            const int k0 = __ffs(emask) - 1;
+            emask &= emask - 1u;
+            const bool pair = emask != 0u;
+            const int k1 = pair ? __ffs(emask) - 1 : k0;
+            emask &= emask - 1u;
+            const unsigned lb0 = sh.lb[wib][k0][lane], lb1 = pair ? sh.lb[wib][k1][lane] : 0u;
+            float na[3], nb[3];
+            if (PRUNE && !pair) {
+                entry(k0, lb0, na);
+                nb[0] = nb[1] = nb[2] = 0.f;
+            } else {
+                entry(k0, lb0, na);
+                entry(k1, lb1, nb);
+            }
+            flush_j2(d, gA, gB, two, ia, a, b, any);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                a[c] = na[c];
+                b[c] = nb[c];
+            }
+            gA = __shfl_sync(FULL, gj_l, k0) + jb;
+            gB = __shfl_sync(FULL, gj_l, k1) + jb;
+            any = true;
+            two = pair;
+        }
+        flush_j2(d, gA, gB, two, ia, a, b, any);
+        if (eb + EPC >= it.z && lane == 0) v_next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
+        float f[NIC][3];
+#pragma unroll
+        for (int p = 0; p < NIC / 2; ++p)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                unpack2(fi[p][c], f[2 * p][c], f[2 * p + 1][c]);
+                fi[p][c] = 0ull;
+            }
+        flush_i(d, gS, ia, jb, touched, f);
+        if (PRUNE && lane < ne) d.ent_hdr[ebase + eb + lane].y = (hy_l & ~0xff00) | (int)(keep_l << 8);
+    }
+    return v_next;
+}
+
+template <int WARPS>
+__device__ __noinline__ int item_entries_lat_prune(const Dev &d, PairSharedLat<WARPS> &sh, const SysDev &S, int4 it,
+                                                   int gS) {
+    return item_entries_lat<WARPS, 8, true>(d, sh, S, it, gS);
+}
+
+// the item's super-cluster into shared memory, in the layout of either form
+template <int WARPS>
+__device__ __forceinline__ void stage_cluster(const Dev &d, PairShared<WARPS> &sh, int wib, int k, int g) {
+    sh.sxq[wib][k] = d.xq[g];
+    sh.slj[wib][k] = d.lj[g];
+}
+template <int WARPS>
+__device__ __forceinline__ void stage_cluster(const Dev &d, PairSharedLat<WARPS> &sh, int wib, int k, int g) {
+    const float4 x = d.xq[g];
+    const float2 l = d.lj[g];
+    // slot k: atom k & 7 of i-cluster k >> 3
+    float *row = reinterpret_cast<float *>(&sh.si[wib][0][(k >> 4) * IC + (k & 7)]) + ((k >> 3) & 1);
+    row[0] = x.x;
+    row[2] = x.y;
+    row[2 * SC] = x.z;
+    row[2 * SC + 2] = x.w;
+    row[4 * SC] = l.x;
+    row[4 * SC + 2] = l.y;
+}
+
 template <bool ENERGY, int WARPS, int MSHIFT>
-__device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int nblk, PairShared<WARPS> &sh) {
+__device__ __forceinline__ int run_item(const Dev &d, PairShared<WARPS> &sh, const SysDev &S, int w, int4 it, int gS,
+                                        float &elj, float &erf, int &npair) {
+    if (MSHIFT == 8 && d.prune_now[w] != 0ull) return item_entries_prune<WARPS>(d, sh, S, it, gS);
+    return item_entries<ENERGY, WARPS, MSHIFT, false>(d, sh, S, it, gS, elj, erf, npair);
+}
+template <bool ENERGY, int WARPS, int MSHIFT>
+__device__ __forceinline__ int run_item(const Dev &d, PairSharedLat<WARPS> &sh, const SysDev &S, int w, int4 it, int gS,
+                                        float &, float &, int &) {
+    static_assert(!ENERGY, "the latency form evaluates forces only");
+    if (MSHIFT == 8 && d.prune_now[w] != 0ull) return item_entries_lat_prune<WARPS>(d, sh, S, it, gS);
+    return item_entries_lat<WARPS, MSHIFT, false>(d, sh, S, it, gS);
+}
+
+// work items of the normal pairs, handed out by a global counter
+template <bool ENERGY, int WARPS, int MSHIFT, class Shared>
+__device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int nblk, Shared &sh) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nw = w1 - w0;
     const int total = sh.pre[nw];
@@ -304,14 +506,11 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int n
         const int sc = it.x;
         const int gS = W.slot_off + (sc - W.sc_off) * SC;
         __syncwarp();
-        sh.sxq[wib][lane] = d.xq[gS + lane];
-        sh.sxq[wib][lane + 32] = d.xq[gS + lane + 32];
-        sh.slj[wib][lane] = d.lj[gS + lane];
-        sh.slj[wib][lane + 32] = d.lj[gS + lane + 32];
+        stage_cluster(d, sh, wib, lane, gS + lane);
+        stage_cluster(d, sh, wib, lane + 32, gS + lane + 32);
         float elj = 0.f, erf = 0.f;
         int npair = 0;
-        if (MSHIFT == 8 && d.prune_now[w] != 0ull) v_next = item_entries_prune<WARPS>(d, sh, S, it, gS);
-        else v_next = item_entries<ENERGY, WARPS, MSHIFT, false>(d, sh, S, it, gS, elj, erf, npair);
+        v_next = run_item<ENERGY, WARPS, MSHIFT>(d, sh, S, w, it, gS, elj, erf, npair);
         if (ENERGY) {
             const double el = warp_sum((double)elj), er = warp_sum((double)erf);
             int np = npair;
@@ -528,13 +727,19 @@ __device__ __forceinline__ void bonded_items(const Dev &d, int w0, int w1, int b
     }
 }
 
+// Items per SM up to which the latency form is taken.  Fused launch, common /
+// latency form: 0.4 items per SM (4 x 257 atoms) 33 / 19 us, 5 (8 x 772 atoms)
+// 43 / 32 us, 19 (2 x 9020 atoms) 47 / 48 us, 92 (144 x 772 atoms) 127 / 128 us,
+// 200 (16 x 12 300 atoms) 252 / 308 us.
+constexpr int LAT_ITEMS_PER_SM = 8;
+
 // WARPS x 32 threads per CTA; MINB: resident CTAs per SM the register
 // allocation is sized for.  Variants (autotuned): 8 warps / 3 CTAs (80
 // registers), 4 warps / 7 CTAs (72), 4 warps / 8 CTAs (64).
-template <bool ENERGY, int WARPS, int MINB, bool FUSED>
+template <bool ENERGY, int WARPS, int MINB, bool FUSED, bool LAT>
 __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w1, int nblk_pairs, int a0, int a1,
                                                           int nblk_bonded, int alch_warps) {
-    __shared__ PairShared<WARPS> sh;
+    __shared__ std::conditional_t<LAT, PairSharedLat<WARPS>, PairShared<WARPS>> sh;
     // grid: [alchemical items][bonded terms][normal pairs]; the first two come
     // first so that they run alongside the normal pairs.  (The alchemical
     // blocks return here: when their warps went on to the normal pairs, the
@@ -572,14 +777,14 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w
     normal_items<ENERGY, WARPS, FUSED ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
 }
 
-template <bool ENERGY, int WARPS, int MINB>
+template <bool ENERGY, int WARPS, int MINB, bool LAT>
 static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s, bool fused = false) {
     int nblk = hv.pair_blocks * 8 / WARPS;  // pair_blocks counts 8-warp CTAs
-    if (w1 - w0 < hv.n_walkers) {           // a subset of walkers: size the grid to its work
-        int items = 0;
-        for (int w = w0; w < w1; ++w) items += hv.item_cap[w];
-        int need = (items + WARPS - 1) / WARPS;
-        nblk = need < nblk ? need : nblk;
+    {  // no more blocks than a quarter above the items need (the queue serves any number)
+        long long items = 0;
+        for (int w = w0; w < w1; ++w) items += hv.items[w];
+        const long long need = (items + items / 4 + WARPS - 1) / WARPS;
+        nblk = need < nblk ? (int)need : nblk;
         nblk = nblk < 1 ? 1 : nblk;
     }
     const int a0 = hv.alch_base[w0], a1 = hv.alch_base[w1 - 1] + hv.n_alch[w1 - 1];
@@ -598,23 +803,32 @@ static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cud
         bblk = bblk > hv.n_sm ? hv.n_sm : bblk;
     }
     const int grid = ablk + bblk + nblk;
-    if (fused) k_pairs<ENERGY, WARPS, MINB, true><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, bblk, awarps);
-    else k_pairs<ENERGY, WARPS, MINB, false><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, 0, awarps);
+    if (fused) k_pairs<ENERGY, WARPS, MINB, true, LAT><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, bblk, awarps);
+    else k_pairs<ENERGY, WARPS, MINB, false, LAT><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, 0, awarps);
+}
+
+// launches whose items leave an SM few enough of them take the latency form
+static bool few_items(const HostView &hv, int w0, int w1) {
+    long long n = 0;
+    for (int w = w0; w < w1; ++w) n += hv.items[w];
+    return n <= (long long)LAT_ITEMS_PER_SM * hv.n_sm;
+}
+
+static void launch_pairs_any(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s, bool fused) {
+    if (hv.pair_variant == 0 && few_items(hv, w0, w1)) launch_pairs_v<false, 4, 4, true>(d, hv, w0, w1, s, fused);
+    else if (hv.pair_variant == 1) launch_pairs_v<false, 4, 7, false>(d, hv, w0, w1, s, fused);
+    else if (hv.pair_variant == 2) launch_pairs_v<false, 4, 8, false>(d, hv, w0, w1, s, fused);
+    else launch_pairs_v<false, 8, 3, false>(d, hv, w0, w1, s, fused);
 }
 
 void launch_pairs_fused(const Dev &d, const HostView &hv, int n_stages, cudaStream_t s) {
-    const int W = hv.n_walkers;
     (void)n_stages;
-    if (hv.pair_variant == 1) launch_pairs_v<false, 4, 7>(d, hv, 0, W, s, true);
-    else if (hv.pair_variant == 2) launch_pairs_v<false, 4, 8>(d, hv, 0, W, s, true);
-    else launch_pairs_v<false, 8, 3>(d, hv, 0, W, s, true);
+    launch_pairs_any(d, hv, 0, hv.n_walkers, s, true);
 }
 
 void launch_pairs(const Dev &d, const HostView &hv, int w0, int w1, bool energy, cudaStream_t s) {
-    if (energy) launch_pairs_v<true, 8, 3>(d, hv, w0, w1, s);
-    else if (hv.pair_variant == 1) launch_pairs_v<false, 4, 7>(d, hv, w0, w1, s);
-    else if (hv.pair_variant == 2) launch_pairs_v<false, 4, 8>(d, hv, w0, w1, s);
-    else launch_pairs_v<false, 8, 3>(d, hv, w0, w1, s);
+    if (energy) launch_pairs_v<true, 8, 3, false>(d, hv, w0, w1, s);
+    else launch_pairs_any(d, hv, w0, w1, s, false);
 }
 
 }  // namespace labf

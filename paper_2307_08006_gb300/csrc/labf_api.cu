@@ -344,7 +344,7 @@ struct la_handle {
     std::vector<SysDev> sys;
     std::vector<WalkerDev> walk;
     std::vector<StageDev> stages;
-    std::vector<int> slot_off, slot_cap, sc_cap, n_cols, alch_base, n_alch, item_cap, bo_off, n_bo;
+    std::vector<int> slot_off, slot_cap, sc_cap, n_cols, alch_base, n_alch, item_cap, bo_off, n_bo, items;
     std::vector<int> sys_w0;       // first walker of each system
     std::vector<int> sys_stage0;   // first stage of each system
     std::vector<int> sys_nstage;
@@ -652,6 +652,8 @@ int tune_pairs(la_handle *h, cudaStream_t s, bool use_cache) {
         int rc = rebuild_items(h, s);
         if (rc != LA_OK) return rc;
     }
+    CU(h, cudaMemcpyAsync(h->items.data(), h->d.n_items, sizeof(int) * h->L.W, cudaMemcpyDeviceToHost, s));
+    CU(h, cudaStreamSynchronize(s));
     return refresh_forces(h, s);
 }
 
@@ -1001,6 +1003,8 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     hv.item_cap = h->item_cap.data();
     hv.bo_off = h->bo_off.data();
     hv.n_bo = h->n_bo.data();
+    h->items = h->item_cap;  // until the first lists are counted
+    hv.items = h->items.data();
     set_pair_blocks(h, h->opt.pair_ctas_per_sm > 0 ? h->opt.pair_ctas_per_sm : 4);
     h->hv.pair_variant = h->opt.pair_variant;
     // graph_steps < 0: no graph (one batched launch sequence per step)
@@ -1016,6 +1020,8 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     if (rc != LA_OK) return rc;
     rc = sync_status(h, s, nullptr);
     if (rc != LA_OK) return rc;
+
+    CU(h, cudaMemcpy(h->items.data(), d.n_items, sizeof(int) * L.W, cudaMemcpyDeviceToHost));
 
     // ---- launch-shape autotuner (pair kernel only; the state does not move) ----
     if (h->opt.autotune) {

@@ -1,0 +1,54 @@
+"""The batched step's forms against the one-walker-per-launch step, bit for
+bit: both sides of the line between the pair kernel's latency and common
+forms, stages of more walkers than a warp has lanes, merged every step and
+every few steps, with and without theta statistics."""
+import numpy as np
+import pytest
+
+from paper_2307_08006_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def water(seed):
+    sp = synth.water_box(137, 5, seed=seed, box=1.7, r_cut=0.7)
+    rng = np.random.default_rng(seed)
+    return synth.with_changes(sp, x=((sp.x + rng.normal(0.0, 0.01, sp.x.shape)) % sp.box).astype(np.float32))
+
+
+def run_both(spec, run, steps, **options):
+    from paper_2307_08006_gb300 import labf
+
+    state = synth.initial_state(spec, run, lam0=list(np.linspace(0.02, 0.98, run.n_walkers)))
+    out = []
+    for plain in (False, True):
+        eng = labf.engine_for(spec, run, state, options=options)
+        (eng.step_plain if plain else eng.step)(steps)
+        o = eng.get_states()
+        o.update(eng.read_abf(0, 0))
+        if run.theta_stats:
+            o.update(eng.read_theta(0, 0))
+        out.append(o)
+        eng.close()
+    for k in ("x", "v", "lam", "plam", "step", "sum", "sumsq", "count"):
+        assert np.array_equal(out[0][k], out[1][k]), k
+    if run.theta_stats:
+        for k in ("sum_d2", "sum_d", "sum_sd"):
+            assert np.array_equal(out[0][k], out[1][k]), k
+
+
+@pytest.mark.parametrize("walkers, margin", [(1, 0.0), (4, 0.05), (10, 0.05), (40, 0.05), (40, 0.0)])
+def test_pair_forms(walkers, margin):
+    """1 to 40 walkers of 416 atoms: well below the line (latency form), near
+    it and above it (common form), with and without pruned tiles."""
+    run = synth.water_run(seed=3, walkers_per_stage=1, n_bins=8)
+    run.stages = [synth.Stage(0.0, 1.0, 8, walkers)]
+    run_both(water(31), run, 23, prune_margin=margin)
+
+
+@pytest.mark.parametrize("walkers, shared_freq, theta", [(1, 1, True), (3, 2, True), (33, 1, True), (70, 3, False),
+                                                         (64, 1, False)])
+def test_stage_sizes(walkers, shared_freq, theta):
+    run = synth.lj_fluid_run(seed=9, n_walkers=walkers, n_bins=7)
+    run.shared_freq, run.theta_stats = shared_freq, theta
+    run_both(synth.lj_fluid(seed=12), run, 11)
