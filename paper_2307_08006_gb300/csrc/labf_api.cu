@@ -329,7 +329,8 @@ size_t carve(const Layout &L, char *base, size_t cap, Dev &d, void **io, int *io
     d.lb_apre = a.take<int>(L.W);
     d.lb_spre = a.take<int>(L.W);
     d.lb_done = a.take<unsigned int>(L.W);
-    const int iof = std::max(IO_FLOATS_MIN, 8 * L.max_n);
+    // every walker's x and v (la_get_states), at least a walker's scratch
+    const int iof = (int)std::max<long long>(std::max(IO_FLOATS_MIN, 8 * L.max_n), 6 * L.atoms_w);
     *io = a.take<float>(iof);
     *io_floats = iof;
     return (a.off + ALIGN - 1) / ALIGN * ALIGN;
@@ -356,7 +357,12 @@ struct la_handle {
     cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
     long long graph_launches_per_step = 0;
     int n_sm = 0, dev = 0;
-    unsigned *h_status = nullptr;  // pinned
+    // page-locked: [0] the status word posted by the last call, [1] the one read
+    // by sync_status, then from STAGE_OFF on the staging area of small
+    // read-outs (held under stage_mutex until the caller's arrays are filled)
+    unsigned *h_status = nullptr;
+    size_t stage_cap = 0;
+    std::mutex stage_mutex;
     cudaEvent_t status_ev = nullptr;
     int sticky = LA_OK;
     long long steps = 0, launches = 0, launches_per_step = 0;
@@ -426,9 +432,9 @@ int check_posted(la_handle *h) {
 }
 
 int sync_status(la_handle *h, cudaStream_t s, unsigned *bits) {
+    CU(h, cudaMemcpyAsync(h->h_status + 1, h->d.status, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     CU(h, cudaStreamSynchronize(s));
-    unsigned st = 0;
-    CU(h, cudaMemcpy(&st, h->d.status, sizeof st, cudaMemcpyDeviceToHost));
+    const unsigned st = *(volatile unsigned *)(h->h_status + 1);
     if (bits) *bits = st;
     int code = status_to_code(st);
     if (code != LA_OK) {
@@ -436,6 +442,33 @@ int sync_status(la_handle *h, cudaStream_t s, unsigned *bits) {
         return fail(h, code, "device error: %s", status_text(st));
     }
     return LA_OK;
+}
+
+// Small read-outs: device arrays are copied into the page-locked staging area
+// (asynchronously: a copy to pageable memory waits for itself), and the
+// caller reads them after one synchronisation.
+constexpr size_t STAGE_OFF = 256;
+struct Stage {
+    la_handle *h;
+    cudaStream_t s;
+    std::lock_guard<std::mutex> lock;
+    size_t off = STAGE_OFF;
+    Stage(la_handle *handle, cudaStream_t stream) : h(handle), s(stream), lock(handle->stage_mutex) {}
+    // n values of a device array; valid after the next sync on the stream
+    template <class T>
+    cudaError_t fetch(const T *dev, size_t n, const T **host) {
+        *host = (const T *)((char *)h->h_status + off);
+        off += (n * sizeof(T) + 15) / 16 * 16;
+        if (off > STAGE_OFF + h->stage_cap) return cudaErrorInvalidValue;  // (sized for every read-out)
+        return cudaMemcpyAsync((void *)*host, dev, n * sizeof(T), cudaMemcpyDeviceToHost, s);
+    }
+};
+
+// the largest read-out: theta sums of a stage with its bin statistics and every
+// walker's own ones
+size_t stage_bytes(const Layout &L) {
+    const size_t nb = L.max_bins, W = L.W, P = L.P_max;
+    return 8 * (3 * nb * P + 3 * nb + 3 * W * nb + 3 * W + 2 * P + 64) + 16 * 16;
 }
 
 // one batched MD step over walkers [w0, w1)
@@ -454,12 +487,8 @@ int kernels_per_step(la_handle *h) { return 1 + 1 + rebuild_kernel_count(h->hv, 
 
 // evaluate forces, dU/dlambda and G at the current state of walkers [w0, w1)
 int prime(la_handle *h, int w0, int w1, bool force_rebuild, bool energy, cudaStream_t s) {
-    if (force_rebuild) {
-        std::vector<int> one(w1 - w0, 1);
-        CU(h, cudaMemcpyAsync(h->d.rebuild + w0, one.data(), sizeof(int) * one.size(),
-                              cudaMemcpyHostToDevice, s));
-        CU(h, cudaStreamSynchronize(s));
-    }
+    // (any non-zero value marks a walker)
+    if (force_rebuild) CU(h, cudaMemsetAsync(h->d.rebuild + w0, 1, sizeof(int) * (w1 - w0), s));
     const size_t g0 = h->slot_off[w0], g1 = (size_t)h->slot_off[w1 - 1] + h->slot_cap[w1 - 1];
     CU(h, cudaMemsetAsync(h->d.F + 3 * g0, 0, 3 * (g1 - g0) * sizeof(unsigned long long), s));
     if (energy) CU(h, cudaMemsetAsync(h->d.eterm + (size_t)N_ETERMS * w0, 0,
@@ -1010,8 +1039,9 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     // graph_steps < 0: no graph (one batched launch sequence per step)
     h->graph_steps = h->opt.graph_steps > 0 ? h->opt.graph_steps : (h->opt.graph_steps < 0 ? 0 : 10);
 
-    CU(h, cudaMallocHost((void **)&h->h_status, sizeof(unsigned)));
-    *h->h_status = 0;
+    h->stage_cap = stage_bytes(L);
+    CU(h, cudaMallocHost((void **)&h->h_status, STAGE_OFF + h->stage_cap));
+    h->h_status[0] = h->h_status[1] = 0;
     CU(h, cudaEventCreateWithFlags(&h->status_ev, cudaEventDisableTiming));
     CU(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     CU(h, cudaStreamCreateWithFlags(&h->cap_stream2, cudaStreamNonBlocking));
@@ -1103,12 +1133,12 @@ int la_read_abf(la_handle *h, int sys, int stage, double *sum, double *sumsq, in
     cudaStream_t s = (cudaStream_t)stream;
     const StageDev &st = h->stages[h->sys_stage0[sys] + stage];
     const int nb = st.n_bins;
-    std::vector<double> s1(nb), s2(nb);
-    std::vector<unsigned long long> c(nb);
-    CU(h, cudaMemcpyAsync(s1.data(), h->d.abf_sum + st.bin_off, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
-    CU(h, cudaMemcpyAsync(s2.data(), h->d.abf_sumsq + st.bin_off, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
-    CU(h, cudaMemcpyAsync(c.data(), h->d.abf_count + st.bin_off, sizeof(unsigned long long) * nb,
-                          cudaMemcpyDeviceToHost, s));
+    Stage stage_io(h, s);
+    const double *s1, *s2;
+    const unsigned long long *c;
+    CU(h, stage_io.fetch(h->d.abf_sum + st.bin_off, nb, &s1));
+    CU(h, stage_io.fetch(h->d.abf_sumsq + st.bin_off, nb, &s2));
+    CU(h, stage_io.fetch(h->d.abf_count + st.bin_off, nb, &c));
     int rc = sync_status(h, s, nullptr);
     if (rc != LA_OK) return rc;
     // TI read-out (Sec. 2.3): Riemann sum of bin means
@@ -1152,18 +1182,17 @@ int la_energy_forces(la_handle *h, int walker, uint32_t flags, double *energy_te
     const WalkerDev &W = h->walk[walker];
     const SysDev &S = h->sys[W.sys];
     if (forces) launch_forces_out(h->d, walker, S.n_atoms, forces, s);
-    long long et[N_ETERMS];
-    double sw = 0.0;
-    std::vector<double> th(2 * h->L.P_max);
-    CU(h, cudaMemcpyAsync(et, h->d.eterm + (size_t)N_ETERMS * walker, sizeof et, cudaMemcpyDeviceToHost, s));
-    CU(h, cudaMemcpyAsync(&sw, h->d.s + walker, sizeof sw, cudaMemcpyDeviceToHost, s));
-    CU(h, cudaMemcpyAsync(th.data(), h->d.wth + (size_t)walker * 2 * h->L.P_max, sizeof(double) * th.size(),
-                          cudaMemcpyDeviceToHost, s));
+    Stage stage_io(h, s);
+    const long long *et;
+    const double *sw, *th;
+    CU(h, stage_io.fetch(h->d.eterm + (size_t)N_ETERMS * walker, N_ETERMS, &et));
+    CU(h, stage_io.fetch(h->d.s + walker, 1, &sw));
+    CU(h, stage_io.fetch(h->d.wth + (size_t)walker * 2 * h->L.P_max, 2 * h->L.P_max, &th));
     rc = sync_status(h, s, nullptr);
     if (rc != LA_OK) return rc;
     if (energy_terms)
         for (int k = 0; k < LA_N_TERMS; ++k) energy_terms[k] = (double)et[k] / E_TO_FIX;
-    if (dUdl) *dUdl = sw;
+    if (dUdl) *dUdl = *sw;
     for (int p = 0; p < S.P; ++p) {
         if (dUdtheta) dUdtheta[p] = th[p];
         if (d2Udl_dtheta) d2Udl_dtheta[p] = th[h->L.P_max + p];
@@ -1259,23 +1288,21 @@ int la_get_states(la_handle *h, float *x, float *v, double *lam, double *plam, u
     if (!h) return LA_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const int W = h->L.W;
-    float *io = (float *)h->io;
-    size_t off = 0;  // float offset of walker w's block in x and v
-    for (int w = 0; w < W; ++w) {
-        const int n = h->sys[h->walk[w].sys].n_atoms;
-        if (x || v) {
-            // the staging area is reused walker after walker: stream order puts
-            // each copy-out before the next walker's gather
-            launch_state_io(h->d, w, n, io, io + 3 * (size_t)n, false, s);
-            if (x) CU(h, cudaMemcpyAsync(x + off, io, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, s));
-            if (v) CU(h, cudaMemcpyAsync(v + off, io + 3 * (size_t)n, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, s));
-        }
-        off += 3 * (size_t)n;
-    }
-    if (lam) CU(h, cudaMemcpyAsync(lam, h->d.lam, sizeof(double) * W, cudaMemcpyDeviceToHost, s));
-    if (plam) CU(h, cudaMemcpyAsync(plam, h->d.plam, sizeof(double) * W, cudaMemcpyDeviceToHost, s));
-    if (step) CU(h, cudaMemcpyAsync(step, h->d.step, sizeof(uint64_t) * W, cudaMemcpyDeviceToHost, s));
+    const size_t rows = h->L.atoms_w;
+    float *xo = x ? (float *)h->io : nullptr, *vo = v ? (float *)h->io + 3 * rows : nullptr;
+    if (x || v) launch_states_io(h->d, (int)rows, xo, vo, false, s);
+    if (x) CU(h, cudaMemcpyAsync(x, xo, sizeof(float) * 3 * rows, cudaMemcpyDeviceToHost, s));
+    if (v) CU(h, cudaMemcpyAsync(v, vo, sizeof(float) * 3 * rows, cudaMemcpyDeviceToHost, s));
+    Stage stage_io(h, s);
+    const double *l = nullptr, *p = nullptr;
+    const unsigned long long *st = nullptr;
+    if (lam) CU(h, stage_io.fetch(h->d.lam, W, &l));
+    if (plam) CU(h, stage_io.fetch(h->d.plam, W, &p));
+    if (step) CU(h, stage_io.fetch(h->d.step, W, &st));
     CU(h, cudaStreamSynchronize(s));
+    if (lam) memcpy(lam, l, sizeof(double) * W);
+    if (plam) memcpy(plam, p, sizeof(double) * W);
+    if (step) memcpy(step, st, sizeof(uint64_t) * W);
     return LA_OK;
 }
 
@@ -1286,24 +1313,16 @@ int la_set_states(la_handle *h, const float *x, const float *v, const double *la
     if (h->sticky != LA_OK) return fail(h, LA_ERR_STATE, "handle in error state: %s", h->err.c_str());
     cudaStream_t s = (cudaStream_t)stream;
     const int W = h->L.W;
-    float *io = (float *)h->io;
-    std::vector<int> one(W, 1);
+    const size_t rows = h->L.atoms_w;
     // every walker's lists and forces are stale from here on, whatever follows
     h->dirty = true;
     int rc = [&]() -> int {
-        CU(h, cudaMemcpyAsync(h->d.rebuild, one.data(), sizeof(int) * W, cudaMemcpyHostToDevice, s));
-        size_t off = 0;
-        for (int w = 0; w < W; ++w) {
-            const int n = h->sys[h->walk[w].sys].n_atoms;
-            if (x || v) {
-                // read back the current state first when one of the two stays unchanged
-                if (!x || !v) launch_state_io(h->d, w, n, io, io + 3 * (size_t)n, false, s);
-                if (x) CU(h, cudaMemcpyAsync(io, x + off, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, s));
-                if (v)
-                    CU(h, cudaMemcpyAsync(io + 3 * (size_t)n, v + off, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, s));
-                launch_state_io(h->d, w, n, io, io + 3 * (size_t)n, true, s);
-            }
-            off += 3 * (size_t)n;
+        CU(h, cudaMemsetAsync(h->d.rebuild, 1, sizeof(int) * W, s));
+        if (x || v) {
+            float *xi = x ? (float *)h->io : nullptr, *vi = v ? (float *)h->io + 3 * rows : nullptr;
+            if (x) CU(h, cudaMemcpyAsync(xi, x, sizeof(float) * 3 * rows, cudaMemcpyHostToDevice, s));
+            if (v) CU(h, cudaMemcpyAsync(vi, v, sizeof(float) * 3 * rows, cudaMemcpyHostToDevice, s));
+            launch_states_io(h->d, (int)rows, xi, vi, true, s);
         }
         if (lam) CU(h, cudaMemcpyAsync(h->d.lam, lam, sizeof(double) * W, cudaMemcpyHostToDevice, s));
         if (plam) CU(h, cudaMemcpyAsync(h->d.plam, plam, sizeof(double) * W, cudaMemcpyHostToDevice, s));
@@ -1315,7 +1334,7 @@ int la_set_states(la_handle *h, const float *x, const float *v, const double *la
         h->sticky = rc;
         return rc;
     }
-    return sync_status(h, s, nullptr);  // also keeps `one` alive until the copy is done
+    return sync_status(h, s, nullptr);  // the caller's arrays are free again
 }
 
 // ---- checkpoints: the arena's state prefix plus a header ----
@@ -1498,21 +1517,18 @@ int la_read_theta(la_handle *h, int sys, int stage, double *sum_d2, double *sum_
     cudaStream_t s = (cudaStream_t)stream;
     const StageDev &st = h->stages[h->sys_stage0[sys] + stage];
     const int P = h->sys[sys].P, PM = h->L.P_max, nb = st.n_bins, MB = h->L.max_bins;
-    std::vector<double> th[3];
+    Stage stage_io(h, s);
+    const double *th[3];
     double *srcs[3] = {h->d.th_d2, h->d.th_d, h->d.th_sd};
-    for (int q = 0; q < 3; ++q) {
-        th[q].resize((size_t)nb * PM);
-        CU(h, cudaMemcpyAsync(th[q].data(), srcs[q] + (size_t)st.bin_off * PM, sizeof(double) * th[q].size(),
-                              cudaMemcpyDeviceToHost, s));
-    }
+    for (int q = 0; q < 3; ++q) CU(h, stage_io.fetch(srcs[q] + (size_t)st.bin_off * PM, (size_t)nb * PM, &th[q]));
     // samples per bin (merged and walker-local) and their dU/dlambda sums
-    std::vector<double> s1(nb), l1((size_t)h->L.W * MB);
-    std::vector<unsigned long long> c(nb), lc((size_t)h->L.W * MB);
-    CU(h, cudaMemcpyAsync(s1.data(), h->d.abf_sum + st.bin_off, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
-    CU(h, cudaMemcpyAsync(c.data(), h->d.abf_count + st.bin_off, sizeof(unsigned long long) * nb,
-                          cudaMemcpyDeviceToHost, s));
-    CU(h, cudaMemcpyAsync(l1.data(), h->d.dl_sum, sizeof(double) * l1.size(), cudaMemcpyDeviceToHost, s));
-    CU(h, cudaMemcpyAsync(lc.data(), h->d.dl_count, sizeof(unsigned long long) * lc.size(), cudaMemcpyDeviceToHost, s));
+    const double *s1, *l1;
+    const unsigned long long *c, *lc;
+    const size_t rows = (size_t)(st.w1 - st.w0) * MB, row0 = (size_t)st.w0 * MB;
+    CU(h, stage_io.fetch(h->d.abf_sum + st.bin_off, nb, &s1));
+    CU(h, stage_io.fetch(h->d.abf_count + st.bin_off, nb, &c));
+    CU(h, stage_io.fetch(h->d.dl_sum + row0, rows, &l1));
+    CU(h, stage_io.fetch(h->d.dl_count + row0, rows, &lc));
     int rc = sync_status(h, s, nullptr);
     if (rc != LA_OK) return rc;
     double *outs[3] = {sum_d2, sum_d, sum_sd};
@@ -1527,7 +1543,7 @@ int la_read_theta(la_handle *h, int sys, int stage, double *sum_d2, double *sum_
         for (int p = 0; p < P; ++p) dA_dtheta[p] = 0.0;
         for (int k = 0; k < nb; ++k) {
             double sum = s1[k], cnt = (double)c[k];
-            for (int w = st.w0; w < st.w1; ++w) {
+            for (int w = 0; w < st.w1 - st.w0; ++w) {
                 sum += l1[(size_t)w * MB + k];
                 cnt += (double)lc[(size_t)w * MB + k];
             }

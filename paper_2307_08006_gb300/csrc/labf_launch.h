@@ -38,6 +38,7 @@ void launch_bonded(const Dev &d, const HostView &hv, int w0, int w1, bool energy
 void launch_walker(const Dev &d, int w0, int w1, bool energy, cudaStream_t s);
 void launch_lambda(const Dev &d, int s0, int s1, bool prime, cudaStream_t s);
 void launch_state_io(const Dev &d, int w, int n, float *x, float *v, bool to_slots, cudaStream_t s);
+void launch_states_io(const Dev &d, int rows, float *x, float *v, bool to_slots, cudaStream_t s);
 void launch_forces_out(const Dev &d, int w, int n, float *out, cudaStream_t s);
 void launch_lambda_path(const double *lam, int n, double bv, double be, double *out, cudaStream_t s);
 void launch_positions_in(const Dev &d, int w, int n, const float *x, cudaStream_t s);
