@@ -19,7 +19,7 @@
 namespace labf {
 
 // -------------------------------------------------------------------------
-// R1: quantize every real slot and count atoms per xy column
+// R1: quantize every real slot and drop it into its xy column's bucket
 // -------------------------------------------------------------------------
 __global__ void k_quantize(Dev d, int g0, int g1) {
     const int nthr = gridDim.x * blockDim.x;
@@ -39,7 +39,6 @@ __global__ void k_quantize(Dev d, int g0, int g1) {
         const int c = cx + S.ncx * cy;
         if (!la_in(d, c, W.n_cols)) continue;
         d.t_uq[g] = make_int4((int)ux, (int)uy, (int)uz, a);
-        d.t_col[g] = c;
         // one atomic per (walker, column) group of the warp's active lanes
         // (slots of a warp are spatially sorted, so most lanes share one)
         const int key = W.col_off + c;
@@ -49,235 +48,266 @@ __global__ void k_quantize(Dev d, int g0, int g1) {
         int base = 0;
         if (lane == leader) base = atomicAdd(&d.col_count[key], __popc(grp));
         base = __shfl_sync(grp, base, leader);
-        d.t_pos[g] = base + __popc(grp & ((1u << lane) - 1u));
+        const int p = base + __popc(grp & ((1u << lane) - 1u));
+        if (p < MAX_COL) d.bucket[(size_t)key * MAX_COL + p] = g;
     }
 }
 
-// R2: per walker (one warp), prefix sums of column counts and super-cluster
-// counts, 32 columns per pass
-__global__ void k_colscan(Dev d, int w0) {
-    const int w = w0 + blockIdx.x;
-    if (!d.rebuild[w]) return;
-    const WalkerDev &W = d.walk[w];
-    const int lane = threadIdx.x & 31;
-    int acc = 0, sacc = 0;  // totals of the previous passes
-    for (int c0 = 0; c0 < W.n_cols; c0 += 32) {
-        const int c = c0 + lane;
-        const int cnt = c < W.n_cols ? d.col_count[W.col_off + c] : 0;
-        if (cnt > MAX_COL) set_status(d, LA_STATUS_COLUMN_OVERFLOW);
-        const int nsc = (cnt + SC - 1) / SC;
-        int a = cnt, b = nsc;  // inclusive warp scans
+// -------------------------------------------------------------------------
+// R2-R6, one block per column: its place among the super-clusters (sizes of
+// the columns before it), the column sorted by (u_z, atom id) in shared
+// memory and cut into super-clusters of 64; then one warp per super-cluster:
+// four k-d splits (longest axis first, ranks by (coordinate, atom id), larger
+// half first) give 16 leaves of <= 4 atoms, leaf k in slots 4k..4k+3, and the
+// bounding boxes and the state in the new slot order are written.
+//
+// Latency decides these steps (a rebuild of one system has few columns), so
+// they are one launch, and both sorts are bitonic networks of 64-bit keys
+// (coordinate, atom id, index within the column): log^2 steps where rank
+// counting took one per atom of the column or super-cluster.  The five
+// kernels before (scan, scatter, column sort, k-d split, gather) took 57 us
+// for one walker of 12 300 atoms and 88 us for 16; this one takes 24 and 35 us.
+// -------------------------------------------------------------------------
+constexpr int CK_THREADS = 256, CK_WARPS = CK_THREADS / 32;
+constexpr int IDX_BITS = 11;  // index within a column
+static_assert((1 << IDX_BITS) == MAX_COL, "index bits");
+constexpr unsigned long long NO_KEY = ~0ull;
+
+struct ColumnShared {
+    unsigned long long key[MAX_COL];
+    int x[MAX_COL], y[MAX_COL], z[MAX_COL];
+    int part[CK_WARPS];
+};
+
+// coordinate (24 bits), atom id (29 bits), index (11 bits)
+__device__ __forceinline__ unsigned long long sort_key(int coord, int atom, int idx) {
+    return ((unsigned long long)(unsigned)coord << 40) | ((unsigned long long)(unsigned)atom << IDX_BITS) | (unsigned)idx;
+}
+
+// ascending bitonic sort of every aligned block of B positions; lane l holds
+// positions 2l and 2l + 1
+template <int B>
+__device__ __forceinline__ void warp_sort(unsigned long long (&k)[2], int lane) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int ua = __shfl_up_sync(0xffffffffu, a, o), ub = __shfl_up_sync(0xffffffffu, b, o);
-            if (lane >= o) {
-                a += ua;
-                b += ub;
+    for (int size = 2; size <= B; size <<= 1) {
+#pragma unroll
+        for (int t = size >> 1; t > 0; t >>= 1) {
+            const bool up = size == B || ((2 * lane) & size) == 0;
+            if (t == 1) {
+                const bool swap = (k[0] > k[1]) == up;
+                const unsigned long long a = swap ? k[1] : k[0], b = swap ? k[0] : k[1];
+                k[0] = a;
+                k[1] = b;
+            } else {
+                const bool low = (((2 * lane) & t) == 0) == up;  // keeps the smaller of the two
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const unsigned long long o = __shfl_xor_sync(0xffffffffu, k[h], t >> 1);
+                    k[h] = (o < k[h]) == low ? o : k[h];
+                }
             }
         }
-        if (c < W.n_cols) {
-            d.col_start[W.col_off + c] = acc + a - cnt;
-            d.col_sc[W.col_off + c] = sacc + b - nsc;
-            d.col_nsc[W.col_off + c] = nsc;
-        }
-        acc += __shfl_sync(0xffffffffu, a, 31);
-        sacc += __shfl_sync(0xffffffffu, b, 31);
-    }
-    if (lane == 0) {
-        if (sacc > W.sc_cap) {
-            set_status(d, LA_STATUS_LIST_OVERFLOW);
-            sacc = W.sc_cap;
-        }
-        d.n_sc[w] = sacc;
     }
 }
 
-// R3: scatter slot ids into per-column buckets
-__global__ void k_scatter(Dev d, int g0, int g1) {
-    const int nthr = gridDim.x * blockDim.x;
-    for (int g = g0 + blockIdx.x * blockDim.x + threadIdx.x; g < g1; g += nthr) {
-        const int w = d.slot_walker[g];
-        if (!la_in(d, w, d.n_walkers) || !d.rebuild[w] || d.atom_of_slot[g] < 0) continue;
-        const WalkerDev &W = d.walk[w];
-        const int c = d.t_col[g];
-        if (!la_in(d, c, W.n_cols)) continue;
-        const int p = d.col_start[W.col_off + c] + d.t_pos[g];
-        if (!la_in(d, p, d.sys[W.sys].n_atoms)) continue;
-        d.bucket[W.atom_base + p] = g;
+struct Extent {
+    int lo[3], hi[3], n;
+};
+__device__ __forceinline__ Extent extent_of(const int (&u)[2][3], const bool (&real)[2]) {
+    Extent e;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        e.lo[c] = min(real[0] ? u[0][c] : 1 << 30, real[1] ? u[1][c] : 1 << 30);
+        e.hi[c] = max(real[0] ? u[0][c] : -(1 << 30), real[1] ? u[1][c] : -(1 << 30));
+    }
+    e.n = (int)real[0] + (int)real[1];
+    return e;
+}
+// joins the extents of the lanes at distance o
+__device__ __forceinline__ void join(Extent &e, int o) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        e.lo[c] = min(e.lo[c], __shfl_xor_sync(0xffffffffu, e.lo[c], o));
+        e.hi[c] = max(e.hi[c], __shfl_xor_sync(0xffffffffu, e.hi[c], o));
+    }
+    e.n += __shfl_xor_sync(0xffffffffu, e.n, o);
+}
+__device__ __forceinline__ void store_box(int4 *dst, const Extent &e) {
+    dst[0] = make_int4(e.lo[0], e.lo[1], e.lo[2], e.n);
+    dst[1] = make_int4(e.hi[0], e.hi[1], e.hi[2], 0);
+}
+
+// one k-d level: every aligned block of B positions (its atoms first) is
+// sorted along its longest axis and its upper half moved to the block's second
+// half
+template <int B>
+__device__ __forceinline__ void kd_level(const ColumnShared &sh, unsigned long long (&k)[2], int (&u)[2][3],
+                                         bool (&real)[2], int lane, bool full) {
+    Extent e = extent_of(u, real);
+#pragma unroll
+    for (int o = 1; o < B / 2; o <<= 1) join(e, o);
+    // longest axis, the first of equal ones
+    int ax = 0, eb = e.hi[0] - e.lo[0];
+    if (e.hi[1] - e.lo[1] > eb) {
+        ax = 1;
+        eb = e.hi[1] - e.lo[1];
+    }
+    if (e.hi[2] - e.lo[2] > eb) ax = 2;
+    constexpr unsigned long long LOW = (1ull << 40) - 1ull;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c = ax == 0 ? u[h][0] : (ax == 1 ? u[h][1] : u[h][2]);
+        k[h] = real[h] ? ((unsigned long long)(unsigned)c << 40) | (k[h] & LOW) : NO_KEY;
+    }
+    warp_sort<B>(k, lane);
+    if (!full) {
+        const int half = (e.n + 1) / 2, base = (2 * lane) & ~(B - 1);
+        unsigned long long m[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int p = 2 * lane + h - base;  // position in the block; its source rank
+            const int r = p < B / 2 ? p : half + p - B / 2;
+            const bool on = p < B / 2 ? p < half : r < e.n;
+            const int src = on ? base + r : 0;
+            const unsigned long long a = __shfl_sync(0xffffffffu, k[0], src >> 1), b = __shfl_sync(0xffffffffu, k[1], src >> 1);
+            m[h] = !on ? NO_KEY : (src & 1) ? b : a;
+        }
+        k[0] = m[0];
+        k[1] = m[1];
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        real[h] = k[h] != NO_KEY;
+        const int i = (int)(k[h] & (MAX_COL - 1));
+        u[h][0] = sh.x[i];
+        u[h][1] = sh.y[i];
+        u[h][2] = sh.z[i];
     }
 }
 
-// R4: sort each column by (u_z, atom id) and cut it into super-clusters of 64
-__global__ void __launch_bounds__(256) k_colsort(Dev d, int w0) {
+__global__ void __launch_bounds__(CK_THREADS) k_columns(Dev d, int w0) {
     const int w = w0 + blockIdx.y;
     if (!d.rebuild[w]) return;
+    __shared__ ColumnShared sh;
     const WalkerDev &W = d.walk[w];
-    __shared__ unsigned long long key[MAX_COL];
-    __shared__ int slot[MAX_COL];
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     for (int c = blockIdx.x; c < W.n_cols; c += gridDim.x) {
+        // super-clusters of the columns before this one
+        int before = 0;
+        for (int k = tid; k < c; k += CK_THREADS) before += (min(d.col_count[W.col_off + k], MAX_COL) + SC - 1) / SC;
+        before = __reduce_add_sync(0xffffffffu, before);
+        __syncthreads();  // shared memory free
+        if (lane == 0) sh.part[wib] = before;
         const int cnt0 = d.col_count[W.col_off + c];
-        const int cnt = cnt0 > MAX_COL ? MAX_COL : cnt0;
-        const int start = d.col_start[W.col_off + c];
-        __syncthreads();
-        for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
-            const int g = d.bucket[W.atom_base + start + k];
-            if (!la_in(d, g, d.n_slots)) {  // sorts last, written as padding
-                key[k] = ~0ull;
-                slot[k] = -1;
-                continue;
-            }
-            const int4 u = d.t_uq[g];
-            key[k] = ((unsigned long long)(unsigned)u.z << 32) | (unsigned)u.w;
-            slot[k] = g;
-        }
-        __syncthreads();
-        const int sc0 = W.sc_off + d.col_sc[W.col_off + c];
-        const int nsc = d.col_nsc[W.col_off + c];
-        for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
-            const unsigned long long kk = key[k];
-            int r = 0;
-            for (int m = 0; m < cnt; ++m) r += key[m] < kk;
-            const int s = sc0 + r / SC;
-            if (s < W.sc_off + W.sc_cap) d.sc_member[(size_t)s * SC + (r % SC)] = slot[k];
-        }
-        for (int k = threadIdx.x; k < nsc * SC; k += blockDim.x) {
-            const int s = sc0 + k / SC;
-            if (k >= cnt && s < W.sc_off + W.sc_cap) d.sc_member[(size_t)s * SC + (k % SC)] = -1;
-            if ((k % SC) == 0 && s < W.sc_off + W.sc_cap) d.sc_n[s] = min(SC, cnt - (k / SC) * SC);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) d.col_count[W.col_off + c] = 0;  // ready for the next rebuild
-    }
-}
-
-// R5: inside each super-cluster, four k-d splits (longest axis first, ranks
-// by (coordinate, atom id), larger half first) give 16 leaves of <= 4 atoms;
-// leaf k occupies slots 4k..4k+3.  Also the bounding boxes.  One warp per
-// super-cluster.
-__global__ void __launch_bounds__(128) k_kdsplit(Dev d, int w0, int w1) {
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    __shared__ int sx[4][SC], sy[4][SC], sz[4][SC], sa[4][SC], sg[4][SC], sslot[4][SC];
-    const int nwarp = gridDim.x * (blockDim.x >> 5);
-    const int s_begin = d.walk[w0].sc_off, s_end = d.walk[w1 - 1].sc_off + d.walk[w1 - 1].sc_cap;
-    for (int s = s_begin + blockIdx.x * (blockDim.x >> 5) + wib; s < s_end; s += nwarp) {
-        int lo = w0, hi = w1 - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (d.walk[mid].sc_off <= s) lo = mid; else hi = mid - 1;
-        }
-        const int w = lo;
-        if (!d.rebuild[w]) continue;
-        const WalkerDev &W = d.walk[w];
-        const int s_local = s - W.sc_off;
-        if (s_local >= d.n_sc[w]) continue;
-        const int n = d.sc_n[s];
-        for (int k = lane; k < SC; k += 32) {
-            int g = k < n ? d.sc_member[(size_t)s * SC + k] : -1;
-            if (g >= 0 && !la_in(d, g, d.n_slots)) g = -1;
-            if (g >= 0) {
-                const int4 u = d.t_uq[g];
-                sx[wib][k] = u.x; sy[wib][k] = u.y; sz[wib][k] = u.z; sa[wib][k] = u.w;
-            } else {
-                sa[wib][k] = -1;
-            }
-            sslot[wib][k] = g;
-            sg[wib][k] = 0;
-        }
-        __syncwarp();
-        // leaf index by four binary splits
-        for (int level = 0; level < 4; ++level) {
-            // extent and size of every group of this level by warp reductions;
-            // each lane keeps those of its two atoms' groups
-            int ext[2][3] = {{0, 0, 0}, {0, 0, 0}}, cnts[2] = {0, 0};
-            {
-                const int ga = lane < n ? sg[wib][lane] : -1;
-                const int gb = lane + 32 < n ? sg[wib][lane + 32] : -1;
-                const int xa[3] = {sx[wib][lane], sy[wib][lane], sz[wib][lane]};
-                const int xb[3] = {sx[wib][lane + 32], sy[wib][lane + 32], sz[wib][lane + 32]};
-                for (int g = 0; g < (1 << level); ++g) {
-                    const bool ia = ga == g, ib = gb == g;
-                    const int c = __reduce_add_sync(0xffffffffu, (int)ia + (int)ib);
-                    for (int q = 0; q < 3; ++q) {
-                        const int lo = __reduce_min_sync(0xffffffffu, min(ia ? xa[q] : (1 << 30), ib ? xb[q] : (1 << 30)));
-                        const int hi = __reduce_max_sync(0xffffffffu, max(ia ? xa[q] : -1, ib ? xb[q] : -1));
-                        if (ia) ext[0][q] = hi - lo;
-                        if (ib) ext[1][q] = hi - lo;
-                    }
-                    if (ia) cnts[0] = c;
-                    if (ib) cnts[1] = c;
+        const int cnt = min(cnt0, MAX_COL);
+        const int *bucket = d.bucket + (size_t)(W.col_off + c) * MAX_COL;
+        int size = SC;
+        while (size < cnt) size <<= 1;
+        for (int k = tid; k < size; k += CK_THREADS) {
+            unsigned long long key = NO_KEY;
+            if (k < cnt) {
+                const int g = bucket[k];
+                if (la_in(d, g, d.n_slots)) {  // (an entry out of range becomes padding)
+                    const int4 u = d.t_uq[g];
+                    sh.x[k] = u.x;
+                    sh.y[k] = u.y;
+                    sh.z[k] = u.z;
+                    key = sort_key(u.z, u.w, k);
                 }
             }
-            int newg[2];
+            sh.key[k] = key;
+        }
+        __syncthreads();
+        int sc0 = 0;
+#pragma unroll
+        for (int q = 0; q < CK_WARPS; ++q) sc0 += sh.part[q];
+        const int nsc = (cnt + SC - 1) / SC;
+        if (tid == 0) {
+            if (cnt0 > MAX_COL) set_status(d, LA_STATUS_COLUMN_OVERFLOW);
+            d.col_sc[W.col_off + c] = sc0;
+            d.col_nsc[W.col_off + c] = nsc;
+            if (c == W.n_cols - 1) {
+                if (sc0 + nsc > W.sc_cap) set_status(d, LA_STATUS_LIST_OVERFLOW);
+                d.n_sc[w] = min(sc0 + nsc, W.sc_cap);
+            }
+        }
+        // bitonic sort; steps of stride <= 32 stay within a warp's own 64 keys
+        for (int s = 2; s <= size; s <<= 1) {
+            for (int t = s >> 1; t > 0; t >>= 1) {
+                if (t > 32 || (t == 32 && s > SC)) __syncthreads(); else __syncwarp();
+                for (int i = tid; i < size / 2; i += CK_THREADS) {
+                    const int a = 2 * i - (i & (t - 1)), b = a + t;
+                    const unsigned long long ka = sh.key[a], kb = sh.key[b];
+                    if ((ka > kb) == ((a & s) == 0)) {
+                        sh.key[a] = kb;
+                        sh.key[b] = ka;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        for (int q = wib; q < nsc; q += CK_WARPS) {
+            const int s_local = sc0 + q, n = min(SC, cnt - q * SC);
+            if (s_local >= W.sc_cap) break;
+            const int s = W.sc_off + s_local;
+            unsigned long long k[2];
+            int u[2][3];
+            bool real[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int k = lane + 32 * h;
-                newg[h] = sg[wib][k];
-                if (k >= n) continue;
-                const int gid = sg[wib][k];
-                const int cnt = cnts[h];
-                // longest axis, the first of equal ones
-                int ax = 0, eb = ext[h][0];
-                if (ext[h][1] > eb) {
-                    ax = 1;
-                    eb = ext[h][1];
-                }
-                if (ext[h][2] > eb) ax = 2;
-                const int *co = ax == 0 ? sx[wib] : (ax == 1 ? sy[wib] : sz[wib]);
-                const long long mykey = ((long long)co[k] << 32) | (unsigned)sa[wib][k];
-                int r = 0;
-                for (int m = 0; m < n; ++m) {
-                    if (sg[wib][m] != gid) continue;
-                    const long long km = ((long long)co[m] << 32) | (unsigned)sa[wib][m];
-                    r += km < mykey;
-                }
-                newg[h] = 2 * gid + (r >= (cnt + 1) / 2 ? 1 : 0);
+                const int p = 2 * lane + h;
+                k[h] = p < n ? sh.key[q * SC + p] : NO_KEY;
+                real[h] = k[h] != NO_KEY;
+                const int i = (int)(k[h] & (MAX_COL - 1));
+                u[h][0] = sh.x[i];
+                u[h][1] = sh.y[i];
+                u[h][2] = sh.z[i];
             }
-            __syncwarp();
-            sg[wib][lane] = newg[0];
-            sg[wib][lane + 32] = newg[1];
-            __syncwarp();
-        }
-        // final position inside the leaf: rank by atom id
-        int pos[2];
-        for (int h = 0; h < 2; ++h) {
-            const int k = lane + 32 * h;
-            pos[h] = -1;
-            if (k >= n) continue;
-            int r = 0;
-            for (int m = 0; m < n; ++m) r += (sg[wib][m] == sg[wib][k]) && (sa[wib][m] < sa[wib][k]);
-            pos[h] = sg[wib][k] * JC + r;
-        }
-        // new layout: t_old[new slot] = old slot (-1 for padding)
-        const int gbase = W.slot_off + s_local * SC;
-        d.t_old[gbase + lane] = -1;
-        d.t_old[gbase + lane + 32] = -1;
-        __syncwarp();
-        for (int h = 0; h < 2; ++h)
-            if (pos[h] >= 0) d.t_old[gbase + pos[h]] = sslot[wib][lane + 32 * h];
-        __syncwarp();
-        // bounding boxes (integer, real atoms only): j-clusters, i-clusters, super-cluster
-        if (lane < NJC + NIC + 1) {
-            int first, last;
-            if (lane < NJC) { first = lane; last = lane; }
-            else if (lane < NJC + NIC) { first = 2 * (lane - NJC); last = first + 1; }
-            else { first = 0; last = NJC - 1; }
-            int mn[3] = {1 << 30, 1 << 30, 1 << 30}, mx[3] = {-(1 << 30), -(1 << 30), -(1 << 30)}, cnt = 0;
-            for (int m = 0; m < n; ++m) {
-                const int leaf = sg[wib][m];
-                if (leaf < first || leaf > last) continue;
-                ++cnt;
-                mn[0] = min(mn[0], sx[wib][m]); mx[0] = max(mx[0], sx[wib][m]);
-                mn[1] = min(mn[1], sy[wib][m]); mx[1] = max(mx[1], sy[wib][m]);
-                mn[2] = min(mn[2], sz[wib][m]); mx[2] = max(mx[2], sz[wib][m]);
+            const int first = (int)(__shfl_sync(0xffffffffu, k[0], 0) & (MAX_COL - 1));
+            const bool full = n == SC;
+            kd_level<64>(sh, k, u, real, lane, full);
+            kd_level<32>(sh, k, u, real, lane, full);
+            kd_level<16>(sh, k, u, real, lane, full);
+            kd_level<8>(sh, k, u, real, lane, full);
+            // inside a leaf: by atom id
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (real[h]) k[h] &= (1ull << 40) - 1ull;
+            warp_sort<4>(k, lane);
+            const float4 park = d.xq[bucket[first]];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int g = W.slot_off + s_local * SC + 2 * lane + h;
+                real[h] = k[h] != NO_KEY;
+                const int i = (int)(k[h] & (MAX_COL - 1));
+                u[h][0] = sh.x[i];
+                u[h][1] = sh.y[i];
+                u[h][2] = sh.z[i];
+                if (real[h]) {
+                    const int old = bucket[i];
+                    d.t_xq[g] = d.xq[old];
+                    d.t_vv[g] = d.vv[old];
+                    d.uq[g] = make_int4(u[h][0], u[h][1], u[h][2], (int)(k[h] >> IDX_BITS));
+                } else {
+                    // padding: parked on a real atom of the same super-cluster
+                    // (finite, never listed)
+                    d.t_xq[g] = make_float4(park.x, park.y, park.z, 0.f);
+                    d.t_vv[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    d.uq[g] = make_int4(0, 0, 0, -1);
+                }
             }
-            int4 *dst;
-            if (lane < NJC) dst = d.bb_jc + 2 * ((size_t)s * NJC + lane);
-            else if (lane < NJC + NIC) dst = d.bb_ic + 2 * ((size_t)s * NIC + (lane - NJC));
-            else dst = d.bb_sc + 2 * (size_t)s;
-            dst[0] = make_int4(mn[0], mn[1], mn[2], cnt);
-            dst[1] = make_int4(mx[0], mx[1], mx[2], 0);
+            // bounding boxes (integer, real atoms only): j-clusters are two lanes,
+            // i-clusters four
+            Extent e = extent_of(u, real);
+            join(e, 1);
+            if ((lane & 1) == 0) store_box(d.bb_jc + 2 * ((size_t)s * NJC + (lane >> 1)), e);
+            join(e, 2);
+            if ((lane & 3) == 0) store_box(d.bb_ic + 2 * ((size_t)s * NIC + (lane >> 2)), e);
+            join(e, 4);
+            join(e, 8);
+            join(e, 16);
+            if (lane == 0) store_box(d.bb_sc + 2 * (size_t)s, e);
         }
-        __syncwarp();
     }
 }
 
@@ -346,56 +376,30 @@ __device__ __forceinline__ void list_plan(const Dev &d, int w0, int w1) {
     }
 }
 
-// R6: gather the state into the new slot order (scratch buffers)
-__global__ void k_permute_gather(Dev d, int g0, int g1) {
-    const int nthr = gridDim.x * blockDim.x;
-    for (int g = g0 + blockIdx.x * blockDim.x + threadIdx.x; g < g1; g += nthr) {
-        const int w = d.slot_walker[g];
-        if (!d.rebuild[w]) continue;
-        const WalkerDev &W = d.walk[w];
-        const int local = g - W.slot_off;
-        const int s_local = local / SC;
-        int old = -1;
-        if (s_local < d.n_sc[w]) old = d.t_old[g];
-        if (old >= 0 && !la_in(d, old, d.n_slots)) old = -1;
-        if (old >= 0) {
-            d.t_xq[g] = d.xq[old];
-            d.t_vv[g] = d.vv[old];
-            d.uq[g] = d.t_uq[old];
-        } else {
-            // padding: park on a real atom of the same super-cluster (finite,
-            // never listed) or, for unused super-clusters, at the origin
-            float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (s_local < d.n_sc[w]) {
-                const int first = d.sc_member[(size_t)(W.sc_off + s_local) * SC];
-                if (first >= 0 && la_in(d, first, d.n_slots)) p = d.xq[first];
-            }
-            p.w = 0.f;
-            d.t_xq[g] = p;
-            d.t_vv[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-            d.uq[g] = make_int4(0, 0, 0, -1);
-        }
-    }
-}
-
-// R7: write the new layout back and refresh per-slot parameters; the first
-// block also plans the list kernel's work
+// R7: write the new layout back and refresh per-slot parameters (slots of
+// unused super-clusters go to the origin), and clear the column counts for the
+// next rebuild; the first block also plans the list kernel's work
 __global__ void __launch_bounds__(256) k_permute_scatter(Dev d, int g0, int g1, int w0, int w1) {
     if (blockIdx.x == 0) list_plan(d, w0, w1);
     const int nthr = gridDim.x * blockDim.x;
+    // (the counts of walkers that do not rebuild are zero already)
+    const int c0 = d.walk[w0].col_off, c1 = d.walk[w1 - 1].col_off + d.walk[w1 - 1].n_cols;
+    for (int c = c0 + blockIdx.x * blockDim.x + threadIdx.x; c < c1; c += nthr) d.col_count[c] = 0;
     for (int g = g0 + blockIdx.x * blockDim.x + threadIdx.x; g < g1; g += nthr) {
         const int w = d.slot_walker[g];
         if (!d.rebuild[w]) continue;
         const WalkerDev &W = d.walk[w];
         const SysDev &S = d.sys[W.sys];
-        int a = d.uq[g].w;
+        const bool used = (g - W.slot_off) / SC < d.n_sc[w];
+        int a = used ? d.uq[g].w : -1;
         if (a >= 0 && !la_in(d, a, S.n_atoms)) a = -1;
-        float4 x = d.t_xq[g];
+        float4 x = used ? d.t_xq[g] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!used) d.uq[g] = make_int4(0, 0, 0, -1);
         // wrap into [0, L) (the list built from this layout assumes it)
         x.x -= S.boxf * floorf(x.x * S.box_invf);
         x.y -= S.boxf * floorf(x.y * S.box_invf);
         x.z -= S.boxf * floorf(x.z * S.box_invf);
-        d.vv[g] = d.t_vv[g];
+        d.vv[g] = used ? d.t_vv[g] : make_float4(0.f, 0.f, 0.f, 0.f);
         d.atom_of_slot[g] = a;
         if (a >= 0) {
             const float4 ap = d.aparam_mut[S.atom_off + a];
@@ -1066,16 +1070,9 @@ void launch_rebuild(const Dev &d, const HostView &hv, int w0, int w1, cudaStream
     for (int w = w0; w < w1; ++w) max_cols = hv.n_cols[w] > max_cols ? hv.n_cols[w] : max_cols;
     int nsc = 0;
     for (int w = w0; w < w1; ++w) nsc += hv.sc_cap[w];
-    int kb = (nsc + 3) / 4;
-    kb = kb < 1 ? 1 : (kb > hv.n_sm * 16 ? hv.n_sm * 16 : kb);
     const int a0 = hv.alch_base[w0], a1 = hv.alch_base[w1 - 1] + hv.n_alch[w1 - 1];
     k_quantize<<<sb, 256, 0, s>>>(d, g0, g1);
-    k_colscan<<<nw, 32, 0, s>>>(d, w0);
-    k_scatter<<<sb, 256, 0, s>>>(d, g0, g1);
-    dim3 cg(max_cols < 1024 ? max_cols : 1024, nw);
-    k_colsort<<<cg, 256, 0, s>>>(d, w0);
-    k_kdsplit<<<kb, 128, 0, s>>>(d, w0, w1);
-    k_permute_gather<<<sb, 256, 0, s>>>(d, g0, g1);
+    k_columns<<<dim3(max_cols < 1024 ? max_cols : 1024, nw), CK_THREADS, 0, s>>>(d, w0);
     k_permute_scatter<<<sb, LB_THREADS, 0, s>>>(d, g0, g1, w0, w1);
     const int lb = nsc + a1 - a0 < hv.n_sm * 4 ? nsc + a1 - a0 : hv.n_sm * 4;  // resident grid
     k_listbuild<<<lb < 1 ? 1 : lb, LB_THREADS, 0, s>>>(d, batched ? 1 : 0);
@@ -1085,6 +1082,6 @@ void launch_items(const Dev &d, const HostView &, int w0, int w1, cudaStream_t s
     k_items<<<w1 - w0, LB_THREADS, 0, s>>>(d, w0);
 }
 
-int rebuild_kernel_count(const HostView &, int, int) { return 8; }
+int rebuild_kernel_count(const HostView &, int, int) { return 4; }
 
 }  // namespace labf

@@ -269,12 +269,12 @@ size_t carve(const Layout &L, char *base, size_t cap, Dev &d, void **io, int *io
     d.sexcl = a.take<int4>(L.slots);
     d.slot_of_atom = a.take<int>(L.atoms_w);
     d.col_count = a.take<int>(L.cols);
-    d.col_start = a.take<int>(L.cols);
+    a.take<int>(L.cols);  // unused, as below: the state prefix stays as older checkpoints have it
     d.col_sc = a.take<int>(L.cols);
     d.col_nsc = a.take<int>(L.cols);
     d.n_sc = a.take<int>(L.W);
-    d.sc_member = a.take<int>(L.scs * SC);
-    d.sc_n = a.take<int>(L.scs);
+    a.take<int>(L.scs * SC);  // unused
+    a.take<int>(L.scs);       // unused
     d.bb_sc = a.take<int4>(2 * L.scs);
     d.bb_ic = a.take<int4>(2 * L.scs * NIC);
     d.bb_jc = a.take<int4>(2 * L.scs * NJC);
@@ -311,17 +311,14 @@ size_t carve(const Layout &L, char *base, size_t cap, Dev &d, void **io, int *io
     d.th_sd = a.take<double>((size_t)L.total_bins * L.P_max);
     d.status = a.take<unsigned int>(4);
     d.counters = a.take<unsigned long long>(16);
-    a.take<unsigned int>(L.W);  // unused; keeps the state prefix as older checkpoints have it
+    a.take<unsigned int>(L.W);  // unused
     d.sdone = a.take<unsigned int>(L.n_stages);
     if (state_bytes) *state_bytes = (a.off + ALIGN - 1) / ALIGN * ALIGN;
     // scratch: rewritten before every use
     d.t_xq = a.take<float4>(L.slots);
     d.t_vv = a.take<float4>(L.slots);
-    d.t_old = a.take<int>(L.slots);
     d.t_uq = a.take<int4>(L.slots);
-    d.t_col = a.take<int>(L.slots);
-    d.t_pos = a.take<int>(L.slots);
-    d.bucket = a.take<int>(L.atoms_w);
+    d.bucket = a.take<int>(L.cols * (long long)MAX_COL);
     d.lcode = a.take<int>(L.slots);
     d.wdir = a.take<double>(4 * (size_t)L.W);
     d.lb_tot = a.take<int>(3);

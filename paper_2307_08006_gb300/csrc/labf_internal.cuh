@@ -128,9 +128,8 @@ struct Dev {
     int4 *sexcl;                  // per slot: extra excluded partners (atom ids)
     // rebuild scratch
     float4 *t_xq, *t_vv;
-    int *t_old;
     int4 *t_uq;
-    int *t_col, *t_pos, *bucket;
+    int *bucket;                  // per column: MAX_COL slots
     int *lcode;                   // per slot: exclusion group | extra-partner flag, -1: no normal pairs
     // the list kernel's plan: totals (walkers that rebuild, their alchemical
     // atoms, their super-clusters), those walkers, the prefixes of both, and
@@ -140,9 +139,8 @@ struct Dev {
     // per walker atoms
     int *slot_of_atom;
     // columns and super-clusters
-    int *col_count, *col_start, *col_sc, *col_nsc;
+    int *col_count, *col_sc, *col_nsc;
     int *n_sc;
-    int *sc_member, *sc_n;
     int4 *bb_sc, *bb_ic, *bb_jc;  // (lo, hi) pairs; lo.w = real count
     int *sc_nent;
     int2 *ent_hdr;                // (j-cluster base global slot, shift bits | imask << 8)
