@@ -500,10 +500,10 @@ int la_destroy(la_handle *h);
  * beyond the fixed-point accumulators: skipped).  Any non-zero status
  * means the other outputs are incomplete.
  *
- * Scratch: one file-scope static device array of 3 * LA_STATIC_MAX_ATOMS
- * 64-bit force accumulators plus 4 * LA_STATIC_MAX_ALCH doubles (about
- * 3.2 MB), held by every GPU that loads the library until the process
- * exits.  Each call clears the part it uses before using it.  All calls on
+ * Scratch: one file-scope static device array of 7 * 32 64-bit partial sums
+ * per LA_STATIC_MAX_ALCH (about 1.8 MB), held by every GPU that loads the
+ * library until the process exits.  Each call clears or overwrites the part
+ * it uses before using it.  All calls on
  * a device share that one array, so calls whose GPU work overlaps (on
  * different streams, or from different threads) race and corrupt each
  * other's results; serialise them.

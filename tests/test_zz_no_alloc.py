@@ -158,3 +158,39 @@ def test_static_entry_reports_bad_index_and_nonfinite():
                                     sp.b_v, sp.b_e)
     torch.cuda.synchronize()
     assert out[5].item() == 0.0
+
+
+@pytest.mark.parametrize("n_waters, n_alch", [(1, 1), (42, 3), (43, 4), (300, 5), (1365, 31), (1366, 33), (3000, 130)])
+def test_static_entry_sizes_match_engine(n_waters, n_alch):
+    """Partly filled blocks, one to 32 chunks of atoms, one and four
+    alchemical atoms per block, more alchemical atoms than a staged tile:
+    against the engine at one lambda, tolerances as above; twice the same
+    bits."""
+    import torch
+
+    box = max(1.5, (n_waters / 32.768) ** (1.0 / 3.0))
+    sp = synth.water_box(n_waters, n_alch, seed=7, box=box, r_cut=0.6)
+    rng = np.random.default_rng(n_waters)
+    sp.x = (rng.uniform(-0.02, 0.02, sp.x.shape) + sp.x).astype(np.float32) % np.float32(box)
+    run = synth.water_run(seed=42, walkers_per_stage=1, n_bins=10)
+    eng = labf.engine_for(sp, run, synth.initial_state(sp, run, lam0=[0.45, 0.6]))
+    ref = eng.energy_forces(1)
+    eng.set_state(1, lam=0.0)
+    f0 = eng.energy_forces(1)["F"].cpu().numpy().astype(np.float64)
+    fref = ref["F"].cpu().numpy().astype(np.float64)
+    eng.close()
+    t = lambda a, dt: torch.tensor(np.ascontiguousarray(a), dtype=dt, device="cuda")
+    f32, i32 = torch.float32, torch.int32
+    args = (t(sp.x, f32), t(sp.charge, f32), t(sp.sigma, f32), t(sp.epsilon, f32), t(sp.alch, torch.uint8),
+            t(sp.excl_group, i32), t(np.nonzero(sp.alch)[0], i32), sp.box, sp.r_cut, sp.eps_rf, sp.coul, 0.6, sp.b_v,
+            sp.b_e)
+    forces, out = labf.alch_pairs_static(*args)
+    again = labf.alch_pairs_static(*args)
+    o, f = out.cpu().numpy(), forces.cpu().numpy().astype(np.float64)
+    assert o[5] == 0.0
+    assert np.array_equal(again[0].cpu().numpy(), forces.cpu().numpy()) and np.array_equal(again[1].cpu().numpy(), o)
+    scale = max(1.0, abs(o[1]) + abs(o[2]))
+    assert abs(o[0] - ref["dUdl"]) <= TOL * scale
+    assert o[3] == pytest.approx(ref["terms"][2], rel=TOL, abs=TOL)
+    assert o[4] == pytest.approx(ref["terms"][3], rel=TOL, abs=TOL * scale)
+    assert np.sqrt(((f - (fref - f0)) ** 2).sum() / max((fref ** 2).sum(), 1e-30)) < TOL
