@@ -18,39 +18,63 @@
 namespace labf {
 
 // ---------------------------------------------------------------------------
-// atoms: BAOA (with the previous step's final B when pending), lambda: BAOA
+// lambda particles [w0, w1), at most LI_WALKERS: BAOA (FP64), by one block of
+// LI_THREADS.  The three chains of a step (the noise's radius, its angle, and B and A with their
+// division) run in different warps: on the narrow FP64 pipe one thread took
+// 9 us for all of them, as long as the atoms of the smallest systems.
 // ---------------------------------------------------------------------------
-__global__ void k_integrate(Dev d, int w0, int w1, int g0, int g1) {
-    const int nthr = gridDim.x * blockDim.x;
-    // lambda particles (FP64): the first w1-w0 threads of block 0, which is
-    // scheduled first, so that this work overlaps the atoms'
-    if (blockIdx.x == 0) {
-        int w = w0 + threadIdx.x;
-        if (w < w1) {
-            const SysDev &S = d.sys[d.walk[w].sys];
-            if (S.lambda_dynamics) {
-                const StageDev &st = d.stage[d.walk[w].stage];
-                double lam = d.lam[w], p = d.plam[w];
-                const double hdt = 0.5 * S.dt_d;
-                p += hdt * d.G[w];
-                lam += hdt * p / S.m_lambda;
-                for (int it = 0; it < 64 && (lam < st.lo || lam > st.hi); ++it) {
-                    if (lam < st.lo) lam = 2.0 * st.lo - lam; else lam = 2.0 * st.hi - lam;
-                    p = -p;
-                }
-                p = S.c_lm * p + S.sd_lm * normal_lambda(S.seed, (uint32_t)d.walk[w].wlocal, d.step[w]);
-                lam += hdt * p / S.m_lambda;
-                for (int it = 0; it < 64 && (lam < st.lo || lam > st.hi); ++it) {
-                    if (lam < st.lo) lam = 2.0 * st.lo - lam; else lam = 2.0 * st.hi - lam;
-                    p = -p;
-                }
-                if (!(lam >= st.lo && lam <= st.hi)) set_status(d, LA_STATUS_NONFINITE);
-                d.lam[w] = lam;
-                d.plam[w] = p;
-            }
+constexpr int LI_THREADS = 256, LI_WALKERS = 64;
+
+__device__ __forceinline__ void lambda_drift(double &lam, double &p, double hdt, double m, const StageDev &st) {
+    lam += hdt * p / m;
+    for (int it = 0; it < 64 && (lam < st.lo || lam > st.hi); ++it) {
+        if (lam < st.lo) lam = 2.0 * st.lo - lam; else lam = 2.0 * st.hi - lam;
+        p = -p;
+    }
+}
+
+__device__ __forceinline__ void integrate_lambda(const Dev &d, int w0, int w1) {
+    __shared__ double radius[LI_WALKERS], angle[LI_WALKERS];
+    const int part = threadIdx.x / LI_WALKERS, l = threadIdx.x % LI_WALKERS;
+    const int w = w0 + l;
+    const bool on = part < 3 && w < w1 && d.sys[d.walk[w].sys].lambda_dynamics;
+    const SysDev &S = d.sys[d.walk[on ? w : w0].sys];
+    const StageDev &st = d.stage[d.walk[on ? w : w0].stage];
+    const double hdt = 0.5 * S.dt_d;
+    double lam = 0.0, p = 0.0;
+    if (on) {
+        if (part == 0) radius[l] = normal_lambda_radius(S.seed, (uint32_t)d.walk[w].wlocal, d.step[w]);
+        if (part == 1) angle[l] = normal_lambda_cos(S.seed, (uint32_t)d.walk[w].wlocal, d.step[w]);
+        if (part == 2) {
+            lam = d.lam[w];
+            p = d.plam[w] + hdt * d.G[w];
+            lambda_drift(lam, p, hdt, S.m_lambda, st);
         }
     }
-    for (int g = g0 + blockIdx.x * blockDim.x + threadIdx.x; g < g1; g += nthr) {
+    __syncthreads();
+    if (on && part == 2) {
+        p = S.c_lm * p + S.sd_lm * (radius[l] * angle[l]);
+        lambda_drift(lam, p, hdt, S.m_lambda, st);
+        if (!(lam >= st.lo && lam <= st.hi)) set_status(d, LA_STATUS_NONFINITE);
+        d.lam[w] = lam;
+        d.plam[w] = p;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// atoms: BAOA (with the previous step's final B when pending); the first
+// lambda_blocks blocks do the lambda particles.  GATE: the last block of the launch also does the
+// batched step's gate (gate_work).
+// ---------------------------------------------------------------------------
+constexpr int CTR_INTEGRATE = 12;  // blocks of a GATE launch that are through
+
+template <bool GATE>
+__global__ void __launch_bounds__(LI_THREADS) k_integrate(Dev d, int w0, int w1, int g0, int g1, int lambda_blocks,
+                                                          cudaGraphConditionalHandle handle, int conditional) {
+    const int blk = (int)blockIdx.x - lambda_blocks;
+    const int nthr = (gridDim.x - lambda_blocks) * blockDim.x;
+    if (blk < 0) integrate_lambda(d, w0 + blockIdx.x * LI_WALKERS, min(w1, w0 + (int)(blockIdx.x + 1) * LI_WALKERS));
+    for (int g = blk < 0 ? g1 : g0 + blk * blockDim.x + threadIdx.x; g < g1; g += nthr) {
         // every per-slot load is issued before the first branch (padding
         // slots are readable too), so they are all in flight together
         const int a = d.atom_of_slot[g];
@@ -133,6 +157,17 @@ __global__ void k_integrate(Dev d, int w0, int w1, int g0, int g1) {
                 for (int k = 0; k < S.w_count; ++k) d.prune[S.w_first + k] = 1;
         }
     }
+    if (GATE) {
+        __shared__ int last;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&d.counters[CTR_INTEGRATE], 1ull) == gridDim.x - 1ull;
+        __syncthreads();
+        if (!last) return;
+        if (threadIdx.x == 0) d.counters[CTR_INTEGRATE] = 0ull;
+        __threadfence();
+        gate_work(d, w0, w1, handle, conditional);
+    }
 }
 
 // atoms: the final B of the last step of a call
@@ -186,12 +221,40 @@ __global__ void k_lambda(Dev d, int s0, int prime) { lambda_work<false>(d, s0 + 
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
+static int integrate_blocks(const HostView &hv, int g0, int g1) {
+    int blocks = (g1 - g0 + LI_THREADS - 1) / LI_THREADS;
+    blocks = blocks < 1 ? 1 : blocks;
+    return blocks > hv.n_sm * 8 ? hv.n_sm * 8 : blocks;
+}
+
+static int lambda_blocks(int w0, int w1) { return (w1 - w0 + LI_WALKERS - 1) / LI_WALKERS; }
+
 void launch_integrate(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {
     const int g0 = hv.slot_off[w0], g1 = hv.slot_off[w1 - 1] + hv.slot_cap[w1 - 1];
-    int blocks = (g1 - g0 + 255) / 256;
-    blocks = blocks < 1 ? 1 : blocks;
-    blocks = blocks > hv.n_sm * 8 ? hv.n_sm * 8 : blocks;
-    k_integrate<<<blocks + 1, 256, 0, s>>>(d, w0, w1, g0, g1);
+    const int lb = lambda_blocks(w0, w1);
+    k_integrate<false><<<integrate_blocks(hv, g0, g1) + lb, LI_THREADS, 0, s>>>(d, w0, w1, g0, g1, lb, 0, 0);
+}
+
+// Integrator and gate of the batched step.  A launch of at most one block per
+// SM does the gate's work with its last block (a launch and its gap less, 3 us);
+// with more, the fence and arrival of every block cost more than that (16 x
+// 12 300 atoms: 0.8% of the step).
+bool gate_in_integrate(const HostView &hv, int w0, int w1) {
+    return integrate_blocks(hv, hv.slot_off[w0], hv.slot_off[w1 - 1] + hv.slot_cap[w1 - 1]) + lambda_blocks(w0, w1) <=
+           hv.n_sm;
+}
+
+void launch_integrate_gate(const Dev &d, const HostView &hv, int w0, int w1, cudaGraphConditionalHandle handle,
+                           bool conditional, cudaStream_t s) {
+    const int g0 = hv.slot_off[w0], g1 = hv.slot_off[w1 - 1] + hv.slot_cap[w1 - 1];
+    if (gate_in_integrate(hv, w0, w1)) {
+        const int lb = lambda_blocks(w0, w1);
+        k_integrate<true><<<integrate_blocks(hv, g0, g1) + lb, LI_THREADS, 0, s>>>(d, w0, w1, g0, g1, lb, handle,
+                                                                                  conditional ? 1 : 0);
+    } else {
+        launch_integrate(d, hv, w0, w1, s);
+        launch_gate(d, w0, w1, handle, conditional, s);
+    }
 }
 
 void launch_finish(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {

@@ -13,6 +13,7 @@
 // rule (the j super-cluster less than half-way round the index circle from
 // the i super-cluster, or the same one with a positive shift, or the same
 // one with shift 0 and slot_i < slot_j).
+#include "labf_dyn.cuh"
 #include "labf_internal.cuh"
 #include "labf_launch.h"
 
@@ -1002,41 +1003,8 @@ __global__ void __launch_bounds__(LB_THREADS, 4) k_listbuild(Dev d, int prune_fr
     }
 }
 
-// -------------------------------------------------------------------------
-// gate of the batched step, after the integrator: a walker whose pruning was
-// requested is re-pruned by this step's pair pass (prune_now = 1 + step
-// counter; the next integrator step takes the positions it starts from as the
-// walker's new reference).  When some walker must rebuild, the walkers whose
-// systems are due soon (near flags) join it (coalescing).  Inside a CUDA
-// graph one thread also sets the step's conditional handle to "some walker
-// must rebuild", so that the graph skips the list kernels otherwise; such
-// steps are counted in counters[6].
-// -------------------------------------------------------------------------
-__device__ __forceinline__ void coalesce_rebuilds(const Dev &d, int w0, int w1, int any) {
-    if (!any) return;
-    for (int w = w0 + threadIdx.x; w < w1; w += blockDim.x)
-        if (d.near[w]) d.rebuild[w] = 1;
-}
-
 __global__ void k_gate(Dev d, int w0, int w1, cudaGraphConditionalHandle handle, int conditional) {
-    __shared__ int any;
-    if (threadIdx.x == 0) any = 0;
-    __syncthreads();
-    for (int w = w0 + threadIdx.x; w < w1; w += blockDim.x) {
-        const int p = d.prune[w];
-        d.prune_now[w] = p ? d.step[w] + 1ull : 0ull;
-        if (p) {
-            d.prune[w] = 0;
-            atomicAdd(&d.counters[10], 1ull);
-        }
-        if (d.rebuild[w]) any = 1;
-    }
-    __syncthreads();
-    coalesce_rebuilds(d, w0, w1, any);
-    if (conditional && threadIdx.x == 0) {
-        cudaGraphSetConditional(handle, any ? 1u : 0u);
-        if (any) atomicAdd(&d.counters[6], 1ull);
-    }
+    gate_work(d, w0, w1, handle, conditional);
 }
 
 void launch_gate(const Dev &d, int w0, int w1, cudaGraphConditionalHandle handle, bool conditional,

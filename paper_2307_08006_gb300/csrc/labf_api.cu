@@ -350,7 +350,7 @@ struct la_handle {
     int io_floats = 0;
     la_options opt{};
     int graph_steps = 10;
-    cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph = nullptr, graph1 = nullptr;  // graph_steps steps, one step
     cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
     long long graph_launches_per_step = 0;
     int n_sm = 0, dev = 0;
@@ -472,15 +472,16 @@ size_t stage_bytes(const Layout &L) {
 // one batched MD step over all walkers: integrate, [rebuild], then one
 // launch for pairs, bonded terms, walker terms and the lambda update
 int enqueue_step(la_handle *h, int w0, int w1, cudaStream_t s) {
-    launch_integrate(h->d, h->hv, w0, w1, s);
-    launch_gate(h->d, w0, w1, 0, false, s);
+    launch_integrate_gate(h->d, h->hv, w0, w1, 0, false, s);
     launch_rebuild(h->d, h->hv, w0, w1, s, true);
     launch_pairs_fused(h->d, h->hv, (int)h->stages.size(), s);
     return 0;
 }
 
-// integrate, gate, list kernels, fused pair launch
-int kernels_per_step(la_handle *h) { return 1 + 1 + rebuild_kernel_count(h->hv, 0, h->L.W) + 1; }
+// integrate and gate (one launch or two), list kernels, fused pair launch
+int kernels_per_step(la_handle *h) {
+    return (gate_in_integrate(h->hv, 0, h->L.W) ? 1 : 2) + rebuild_kernel_count(h->hv, 0, h->L.W) + 1;
+}
 
 // evaluate forces, dU/dlambda and G at the current state of walkers [w0, w1)
 int prime(la_handle *h, int w0, int w1, bool force_rebuild, bool energy, cudaStream_t s) {
@@ -509,23 +510,20 @@ int flush_dirty(la_handle *h, cudaStream_t s) {
     return prime(h, 0, h->L.W, false, false, s);
 }
 
-int capture_graph(la_handle *h) {
-    if (h->graph) {
-        cudaGraphExecDestroy(h->graph);
-        h->graph = nullptr;
+// `steps` MD steps as one graph.  Each step: integrate, gate -> IF(some walker
+// must rebuild){rebuild chain} -> pairs, bonded, walker, lambda.  The gate sets
+// the step's conditional handle, so steps without a rebuild launch no list
+// kernel at all.
+int capture_steps(la_handle *h, int steps, cudaGraphExec_t *exec) {
+    if (*exec) {
+        cudaGraphExecDestroy(*exec);
+        *exec = nullptr;
     }
-    // Each step: integrate -> gate -> IF(some walker must rebuild){rebuild
-    // chain} -> pairs, bonded, walker, lambda.  The gate kernel sets the
-    // step's conditional handle, so steps without a rebuild launch no list
-    // kernel at all.
     const int W = h->L.W;
-    h->launches_per_step = kernels_per_step(h);
-    if (h->graph_steps == 0) return LA_OK;
     cudaStream_t cs = h->cap_stream, cb = h->cap_stream2;
     cudaGraph_t g;
     CU(h, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    for (int k = 0; k < h->graph_steps; ++k) {
-        launch_integrate(h->d, h->hv, 0, W, cs);
+    for (int k = 0; k < steps; ++k) {
         cudaStreamCaptureStatus st;
         cudaGraph_t cg;
         const cudaGraphNode_t *deps = nullptr;
@@ -533,7 +531,7 @@ int capture_graph(la_handle *h) {
         CU(h, cudaStreamGetCaptureInfo(cs, &st, nullptr, &cg, nullptr, nullptr, nullptr));
         cudaGraphConditionalHandle hc;
         CU(h, cudaGraphConditionalHandleCreate(&hc, cg, 0, cudaGraphCondAssignDefault));
-        launch_gate(h->d, 0, W, hc, true, cs);
+        launch_integrate_gate(h->d, h->hv, 0, W, hc, true, cs);
         CU(h, cudaStreamGetCaptureInfo(cs, &st, nullptr, &cg, &deps, nullptr, &nd));
         // IF (some walker must rebuild) { list kernels }
         cudaGraphNodeParams p = {cudaGraphNodeTypeConditional};
@@ -551,13 +549,24 @@ int capture_graph(la_handle *h) {
         launch_pairs_fused(h->d, h->hv, (int)h->stages.size(), cs);
     }
     CU(h, cudaStreamEndCapture(cs, &g));
-    cudaError_t e = cudaGraphInstantiate(&h->graph, g, 0);
+    cudaError_t e = cudaGraphInstantiate(exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return fail(h, LA_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
+    return LA_OK;
+}
+
+// the graph of graph_steps steps, and one of a single step for the remainder of
+// a call (as single launches every remaining step started the whole chain of
+// list kernels)
+int capture_graph(la_handle *h) {
+    h->launches_per_step = kernels_per_step(h);
+    if (h->graph_steps == 0) return LA_OK;
     // graph steps: integrate, gate, fused pairs; list kernels are counted per
     // step that runs them (device counter)
-    h->graph_launches_per_step = h->launches_per_step - rebuild_kernel_count(h->hv, 0, W);
-    return LA_OK;
+    h->graph_launches_per_step = h->launches_per_step - rebuild_kernel_count(h->hv, 0, h->L.W);
+    int rc = capture_steps(h, h->graph_steps, &h->graph);
+    if (rc != LA_OK || h->graph_steps == 1) return rc;
+    return capture_steps(h, 1, &h->graph1);
 }
 
 void set_pair_blocks(la_handle *h, int ctas_per_sm) {
@@ -1076,11 +1085,19 @@ int la_step_walkers(la_handle *h, int64_t n_steps, void *stream) {
     const int64_t gs = h->graph_steps;
     const int64_t reps = gs > 0 ? n_steps / gs : 0, rem = gs > 0 ? n_steps % gs : n_steps;
     for (int64_t r = 0; r < reps; ++r) CU(h, cudaGraphLaunch(h->graph, s));
-    for (int64_t r = 0; r < rem; ++r) enqueue_step(h, 0, h->L.W, s);
+    // (a graph with conditional nodes cannot join a caller's stream capture:
+    // there the remainder is captured launch by launch)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (rem > 0) CU(h, cudaStreamIsCapturing(s, &cap));
+    const bool single = gs > 0 && cap == cudaStreamCaptureStatusNone;
+    for (int64_t r = 0; r < rem; ++r) {
+        if (single) CU(h, cudaGraphLaunch(h->graph1, s));
+        else enqueue_step(h, 0, h->L.W, s);
+    }
     launch_finish(h->d, h->hv, 0, h->L.W, s);
     CU(h, cudaGetLastError());
     h->steps += n_steps;
-    h->launches += reps * h->graph_steps * h->graph_launches_per_step + rem * h->launches_per_step + 1;
+    h->launches += (reps * gs + (single ? rem : 0)) * h->graph_launches_per_step + (single ? 0 : rem) * h->launches_per_step + 1;
     post_status(h, s);
     return LA_OK;
 }
@@ -1768,6 +1785,7 @@ const char *la_last_error(la_handle *h) { return h ? h->err.c_str() : "no handle
 int la_destroy(la_handle *h) {
     if (!h) return LA_OK;
     if (h->graph) cudaGraphExecDestroy(h->graph);
+    if (h->graph1) cudaGraphExecDestroy(h->graph1);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->cap_stream2) cudaStreamDestroy(h->cap_stream2);
     if (h->status_ev) cudaEventDestroy(h->status_ev);

@@ -174,6 +174,7 @@ struct Dev {
     unsigned long long *counters; // [0] rebuilds [1] pairs normal [2] pairs alch [4, 5] pair
                                   // work items [6] rebuild events [8, 9] list-build work items
                                   // [10] re-pruning passes after a displacement trigger
+                                  // [12] integrator blocks that are through
 };
 
 // ---------------------------------------------------------------------------
@@ -323,15 +324,19 @@ __device__ __forceinline__ float4 normals4(uint32_t seed, uint32_t walker, unsig
     return make_float4(ra * ca, ra * sa, rb * cb, rb * sb);
 }
 
-// FP64 normal for the lambda particle (same stream definition, tag 1).
-__device__ __forceinline__ double normal_lambda(uint32_t seed, uint32_t walker, unsigned long long step) {
-    uint4 r = philox4x32_10(make_uint4(0u, (uint32_t)step, (uint32_t)(step >> 32), 1u),
-                            make_uint2(seed, walker));
-    const double s24 = 5.9604644775390625e-08;
-    double u1 = (double)((r.x >> 8) + 1u) * s24, u2 = (double)(r.y >> 8) * s24;
+// FP64 normal for the lambda particle (same stream definition, tag 1), as the
+// product of its Box-Muller radius and cosine.
+__device__ __forceinline__ double normal_lambda_radius(uint32_t seed, uint32_t walker, unsigned long long step) {
+    const uint4 r = philox4x32_10(make_uint4(0u, (uint32_t)step, (uint32_t)(step >> 32), 1u), make_uint2(seed, walker));
+    const double u1 = (double)((r.x >> 8) + 1u) * 5.9604644775390625e-08;
+    return sqrt(-2.0 * log(u1));
+}
+__device__ __forceinline__ double normal_lambda_cos(uint32_t seed, uint32_t walker, unsigned long long step) {
+    const uint4 r = philox4x32_10(make_uint4(0u, (uint32_t)step, (uint32_t)(step >> 32), 1u), make_uint2(seed, walker));
+    const double u2 = (double)(r.y >> 8) * 5.9604644775390625e-08;
     double sp, cp;
     sincospi(2.0 * u2, &sp, &cp);
-    return sqrt(-2.0 * log(u1)) * cp;
+    return cp;
 }
 
 // u = floor(frac(x L^-1) 2^24), one rounded FP64 product, no contraction.

@@ -27,6 +27,10 @@ void launch_items(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t
 // conditional: also set the graph's conditional handle (false outside graphs)
 void launch_gate(const Dev &d, int w0, int w1, cudaGraphConditionalHandle handle, bool conditional,
                  cudaStream_t s);
+// integrator and gate in one launch (gate_in_integrate) or two
+bool gate_in_integrate(const HostView &hv, int w0, int w1);
+void launch_integrate_gate(const Dev &d, const HostView &hv, int w0, int w1, cudaGraphConditionalHandle handle,
+                           bool conditional, cudaStream_t s);
 int rebuild_kernel_count(const HostView &hv, int w0, int w1);
 // rebuild coalescing of the one-walker-per-launch form (the batched step's
 // gate does the same)
