@@ -190,29 +190,20 @@ __global__ void k_finish(Dev d, int w0, int w1, int g0, int g1) {
 }
 
 // bonded terms, one thread per term
-template <bool ENERGY>
 __global__ void k_bonded(Dev d, int w0, int w1) {
     const int b0 = d.walk[w0].bo_off;
     const int b1 = d.walk[w1 - 1].bo_off + d.walk[w1 - 1].n_bo;
     const int nthr = gridDim.x * blockDim.x;
-    // warps run together (32 terms at a time) for the energy sums
-    for (int tw = b0 + blockIdx.x * blockDim.x + (threadIdx.x & ~31); tw < b1; tw += nthr) {
-        const int t = tw + (threadIdx.x & 31);
-        long long fix = 0;
-        int key = -1;
-        if (t < b1) bonded_term<ENERGY>(d, t, w0, w1, fix, key);
-        if (ENERGY) {
-            __syncwarp();
-            add_energies(d, fix, key);
-        }
-    }
+    long long fix;
+    int key;
+    for (int t = b0 + blockIdx.x * blockDim.x + threadIdx.x; t < b1; t += nthr)
+        bonded_term<false>(d, t, w0, w1, fix, key);
 }
 
 // walker terms, one warp per walker
-template <bool ENERGY>
 __global__ void k_walker(Dev d, int w0, int w1) {
     const int w = w0 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (w < w1) walker_work<ENERGY>(d, w, threadIdx.x & 31);
+    if (w < w1) walker_work(d, w, threadIdx.x & 31);
 }
 
 // ABF fold / bias / final B of lambda, one warp per stage
@@ -264,19 +255,17 @@ void launch_finish(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_
     k_finish<<<blocks, 256, 0, s>>>(d, w0, w1, g0, g1);
 }
 
-void launch_bonded(const Dev &d, const HostView &hv, int w0, int w1, bool energy, cudaStream_t s) {
+void launch_bonded(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {
     const int n = hv.bo_off[w1 - 1] + hv.n_bo[w1 - 1] - hv.bo_off[w0];
     if (n <= 0) return;
     int blocks = (n + 255) / 256;
     blocks = blocks > hv.n_sm * 8 ? hv.n_sm * 8 : blocks;
-    if (energy) k_bonded<true><<<blocks, 256, 0, s>>>(d, w0, w1);
-    else k_bonded<false><<<blocks, 256, 0, s>>>(d, w0, w1);
+    k_bonded<<<blocks, 256, 0, s>>>(d, w0, w1);
 }
 
-void launch_walker(const Dev &d, int w0, int w1, bool energy, cudaStream_t s) {
+void launch_walker(const Dev &d, int w0, int w1, cudaStream_t s) {
     const int blocks = (w1 - w0 + 3) / 4;
-    if (energy) k_walker<true><<<blocks, 128, 0, s>>>(d, w0, w1);
-    else k_walker<false><<<blocks, 128, 0, s>>>(d, w0, w1);
+    k_walker<<<blocks, 128, 0, s>>>(d, w0, w1);
 }
 
 void launch_lambda(const Dev &d, int s0, int s1, bool prime, cudaStream_t s) {

@@ -1,5 +1,6 @@
 // k_io.cu -- state and force transfer between the slot layout and the
 // system's atom order, and the lambda-path evaluator.
+#include "labf_dyn.cuh"
 #include "labf_internal.cuh"
 #include "labf_launch.h"
 
@@ -63,19 +64,6 @@ __global__ void k_states_io(Dev d, int rows, float *x, float *v, int to_slots) {
     }
 }
 
-__global__ void k_forces_out(Dev d, int w, int n, float *out) {
-    const WalkerDev &W = d.walk[w];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int g = checked_slot(d, d.slot_of_atom[W.atom_base + i]);
-        const unsigned long long *F = d.F + 3 * (size_t)g;
-        out[3 * i] = fix_to_float(F[0]);
-        out[3 * i + 1] = fix_to_float(F[1]);
-        out[3 * i + 2] = fix_to_float(F[2]);
-        if (fabsf(out[3 * i]) > FIX_LIMIT || fabsf(out[3 * i + 1]) > FIX_LIMIT || fabsf(out[3 * i + 2]) > FIX_LIMIT)
-            set_status(d, LA_STATUS_FIXED_OVERFLOW);
-    }
-}
-
 __global__ void k_lambda_path(const double *lam, int n, double bv, double be, double *out) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         double lv, le, dlv, dle;
@@ -87,28 +75,43 @@ __global__ void k_lambda_path(const double *lam, int n, double bv, double be, do
     }
 }
 
-// positions of walker w from a device array in atom order; the walker's
-// lists are rebuilt before its next force evaluation
-__global__ void k_positions_in(Dev d, int w, int n, const float *x) {
-    const WalkerDev &W = d.walk[w];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int g = checked_slot(d, d.slot_of_atom[W.atom_base + i]);
-        float4 xq = d.xq[g];
-        xq.x = x[3 * i];
-        xq.y = x[3 * i + 1];
-        xq.z = x[3 * i + 2];
-        d.xq[g] = xq;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) d.rebuild[w] = 1;
-}
+// -------------------------------------------------------------------------
+// One energy evaluation of a walker is [k_ef_in][rebuild chain][pairs, bonded
+// terms and restraints][k_ef_out]: every input in the first launch, every
+// read-out in the last.  Sixteen smaller launches and copies took 35% more
+// host time than the GPU needed for its work on 12 300 atoms.
+// -------------------------------------------------------------------------
 
-// (epsilon, sigma, q) of the alchemical atoms of system `sys` from a device
-// array; every walker of the system rebuilds (the per-slot copies of the
-// parameters are refreshed there).  Negative or non-finite epsilon or sigma:
-// the atom keeps its parameters and LA_STATUS_BAD_PARAM is set.
-__global__ void k_alch_params_in(Dev d, int sys, const double *theta) {
-    const SysDev &S = d.sys[sys];
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < S.n_alch; r += gridDim.x * blockDim.x) {
+// before the evaluation: forces and energies cleared; optionally the walker's
+// positions (atom order) and lambda, the system's alchemical parameters
+// (epsilon, sigma, q; every walker of the system then rebuilds, the per-slot
+// copies of the parameters are refreshed there) from device arrays.  rebuild:
+// the walker's lists are rebuilt before its forces are evaluated.  Negative or
+// non-finite epsilon or sigma: the atom keeps its parameters and
+// LA_STATUS_BAD_PARAM is set.
+__global__ void k_ef_in(Dev d, int w, int n, const float *x, const double *theta, const double *lam, int rebuild) {
+    const WalkerDev &W = d.walk[w];
+    const SysDev &S = d.sys[W.sys];
+    const int nthr = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned long long *F = d.F + 3 * (size_t)W.slot_off;
+    for (int i = t0; i < 3 * W.sc_cap * SC; i += nthr) F[i] = 0ull;
+    if (x)
+        for (int i = t0; i < n; i += nthr) {
+            const int g = checked_slot(d, d.slot_of_atom[W.atom_base + i]);
+            float4 xq = d.xq[g];
+            xq.x = x[3 * (size_t)i];
+            xq.y = x[3 * (size_t)i + 1];
+            xq.z = x[3 * (size_t)i + 2];
+            d.xq[g] = xq;
+        }
+    if (blockIdx.x != 0) return;
+    if (threadIdx.x < N_ETERMS) d.eterm[(size_t)N_ETERMS * w + threadIdx.x] = 0;
+    if (threadIdx.x == 0) {
+        if (x || rebuild) d.rebuild[w] = 1;
+        if (lam) d.lam[w] = *lam;
+    }
+    if (!theta) return;
+    for (int r = threadIdx.x; r < S.n_alch; r += blockDim.x) {
         const double eps = theta[3 * r], sig = theta[3 * r + 1], q = theta[3 * r + 2];
         if (!(eps >= 0.0) || !(sig >= 0.0) || !(eps < 1e30) || !(sig < 1e30) || !(fabs(q) < 1e30)) {
             set_status(d, LA_STATUS_BAD_PARAM);
@@ -121,18 +124,43 @@ __global__ void k_alch_params_in(Dev d, int sys, const double *theta) {
         p.z = (float)(2.0 * sqrt(eps));
         d.aparam_mut[S.atom_off + a] = p;
     }
-    if (blockIdx.x == 0)
-        for (int w = S.w_first + threadIdx.x; w < S.w_first + S.w_count; w += blockDim.x) d.rebuild[w] = 1;
+    for (int v = S.w_first + threadIdx.x; v < S.w_first + S.w_count; v += blockDim.x) d.rebuild[v] = 1;
 }
 
-// energies and derivatives of walker w into a device array: [0, LA_N_TERMS)
-// the energy terms, then U, dU/dlambda, dU/dtheta [P], d2U/dlambda dtheta [P]
-__global__ void k_ef_out(Dev d, int w, int P, double *out) {
+// after the evaluation: block 0 sums the walker's sample, refreshes its
+// stage's lambda forces and writes the energies and derivatives to `out` ([0,
+// LA_N_TERMS) the energy terms, then U, dU/dlambda, dU/dtheta [P],
+// d2U/dlambda dtheta [P]; NULL: left in the engine's arrays); the other
+// blocks write the forces in atom order (NULL: none)
+__global__ void k_ef_out(Dev d, int w, int n, int P, double *out, float *forces) {
+    const WalkerDev &W = d.walk[w];
+    if (blockIdx.x != 0) {
+        const int nthr = (gridDim.x - 1) * blockDim.x;
+        for (int i = (blockIdx.x - 1) * blockDim.x + threadIdx.x; i < n; i += nthr) {
+            const int g = checked_slot(d, d.slot_of_atom[W.atom_base + i]);
+            const unsigned long long *F = d.F + 3 * (size_t)g;
+            const float fx = fix_to_float(F[0]), fy = fix_to_float(F[1]), fz = fix_to_float(F[2]);
+            forces[3 * (size_t)i] = fx;
+            forces[3 * (size_t)i + 1] = fy;
+            forces[3 * (size_t)i + 2] = fz;
+            if (fabsf(fx) > FIX_LIMIT || fabsf(fy) > FIX_LIMIT || fabsf(fz) > FIX_LIMIT)
+                set_status(d, LA_STATUS_FIXED_OVERFLOW);
+        }
+        return;
+    }
+    if (threadIdx.x < 32) {
+        walker_sample<true>(d, w, threadIdx.x);
+        __syncwarp();
+        lambda_work<false>(d, W.stage, 1, threadIdx.x);
+        __threadfence();
+    }
+    __syncthreads();
+    if (!out) return;
     const int t = threadIdx.x;
     if (t == 0) {
         double u = 0.0;
         for (int k = 0; k < LA_N_TERMS; ++k) {
-            const double e = (double)d.eterm[N_ETERMS * w + k] / E_TO_FIX;
+            const double e = (double)__ldcg(d.eterm + N_ETERMS * w + k) / E_TO_FIX;
             out[k] = e;
             u += e;
         }
@@ -146,17 +174,13 @@ __global__ void k_ef_out(Dev d, int w, int P, double *out) {
     }
 }
 
-void launch_positions_in(const Dev &d, int w, int n, const float *x, cudaStream_t s) {
-    k_positions_in<<<(n + 255) / 256, 256, 0, s>>>(d, w, n, x);
+void launch_ef_in(const Dev &d, int w, int n, int slots, const float *x, const double *theta, const double *lam,
+                  bool rebuild, cudaStream_t s) {
+    k_ef_in<<<(3 * slots + 1023) / 1024, 256, 0, s>>>(d, w, n, x, theta, lam, rebuild ? 1 : 0);
 }
 
-void launch_alch_params_in(const Dev &d, int sys, int n_alch, const double *theta, cudaStream_t s) {
-    k_alch_params_in<<<1, 256, 0, s>>>(d, sys, theta);
-    (void)n_alch;
-}
-
-void launch_ef_out(const Dev &d, int w, int P, double *out, cudaStream_t s) {
-    k_ef_out<<<1, 128, 0, s>>>(d, w, P, out);
+void launch_ef_out(const Dev &d, int w, int n, int P, double *out, float *forces, cudaStream_t s) {
+    k_ef_out<<<1 + (forces ? (n + 255) / 256 : 0), 256, 0, s>>>(d, w, n, P, out, forces);
 }
 
 void launch_state_io(const Dev &d, int w, int n, float *x, float *v, bool to_slots, cudaStream_t s) {
@@ -165,10 +189,6 @@ void launch_state_io(const Dev &d, int w, int n, float *x, float *v, bool to_slo
 
 void launch_states_io(const Dev &d, int rows, float *x, float *v, bool to_slots, cudaStream_t s) {
     k_states_io<<<(rows + 255) / 256, 256, 0, s>>>(d, rows, x, v, to_slots ? 1 : 0);
-}
-
-void launch_forces_out(const Dev &d, int w, int n, float *out, cudaStream_t s) {
-    k_forces_out<<<(n + 255) / 256, 256, 0, s>>>(d, w, n, out);
 }
 
 void launch_lambda_path(const double *lam, int n, double bv, double be, double *out, cudaStream_t s) {

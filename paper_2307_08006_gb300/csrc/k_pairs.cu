@@ -571,16 +571,21 @@ __device__ __forceinline__ int walker_of_alch(const Dev &d, int w0, int w1, int 
     return w0 + n - 1;
 }
 
-// Alchemical items [a0, a1), one warp each, then (FUSED) one restraint item
+// What a pair launch does besides the pairs.  STEP (the batched step): bonded
+// terms, restraints, and the lambda update by the last arrival; lists pruned.
+// EVAL (one energy evaluation): bonded terms and restraints.  PAIRS: nothing.
+enum { PAIRS = 0, STEP = 1, EVAL = 2 };
+
+// Alchemical items [a0, a1), one warp each, then (but for PAIRS) one restraint item
 // per walker; unit `unit` of `units` takes every units-th item.
-template <bool ENERGY, int WARPS, bool FUSED>
+template <bool ENERGY, int WARPS, int MODE>
 __device__ __forceinline__ void alch_items(const Dev &d, int w0, int w1, int a0, int a1, int unit, int units) {
     const int lane = threadIdx.x & 31;
-    const int aend = FUSED ? a1 + (w1 - w0) : a1;
+    const int aend = MODE != PAIRS ? a1 + (w1 - w0) : a1;
     for (int it = a0 + unit; it < aend; it += units) {
-        if (FUSED && it >= a1) {  // restraint item of walker w0 + (it - a1)
+        if (MODE != PAIRS && it >= a1) {  // restraint item of walker w0 + (it - a1)
             walker_restraints(d, w0 + (it - a1), lane);
-            arrive_stage(d, w0 + (it - a1), lane);
+            if (MODE == STEP) arrive_stage(d, w0 + (it - a1), lane);
             continue;
         }
         const int w = walker_of_alch(d, w0, w1, it, lane);
@@ -710,20 +715,26 @@ __device__ __forceinline__ void alch_items(const Dev &d, int w0, int w1, int a0,
             }
             if (ENERGY) atomicAdd(&d.counters[2], (unsigned long long)npair);
         }
-        if (FUSED) arrive_stage(d, w, lane);
+        if (MODE == STEP) arrive_stage(d, w, lane);
         if (lane == 0) add_force(d, ga, fax, fay, faz);
     }
 }
 
-// bonded terms in the fused launch: blocks [0, nblk) of the bonded range
+// bonded terms in the same launch: blocks [0, nblk) of the bonded range
+template <bool ENERGY>
 __device__ __forceinline__ void bonded_items(const Dev &d, int w0, int w1, int blk, int nblk) {
     const int b0 = d.walk[w0].bo_off;
     const int b1 = d.walk[w1 - 1].bo_off + d.walk[w1 - 1].n_bo;
-    const int nthr = nblk * blockDim.x;
-    for (int t = b0 + blk * blockDim.x + threadIdx.x; t < b1; t += nthr) {
-        long long fix;
-        int key;
-        bonded_term<false>(d, t, w0, w1, fix, key);
+    const int nthr = nblk * blockDim.x, lane = threadIdx.x & 31;
+    // warps run together (32 terms at a time) for the energy sums
+    for (int tw = b0 + blk * blockDim.x + (threadIdx.x & ~31); tw < b1; tw += nthr) {
+        long long fix = 0;
+        int key = -1;
+        if (tw + lane < b1) bonded_term<ENERGY>(d, tw + lane, w0, w1, fix, key);
+        if (ENERGY) {
+            __syncwarp();
+            add_energies(d, fix, key);
+        }
     }
 }
 
@@ -736,7 +747,7 @@ constexpr int LAT_ITEMS_PER_SM = 8;
 // WARPS x 32 threads per CTA; MINB: resident CTAs per SM the register
 // allocation is sized for.  Variants (autotuned): 8 warps / 3 CTAs (80
 // registers), 4 warps / 7 CTAs (72), 4 warps / 8 CTAs (64).
-template <bool ENERGY, int WARPS, int MINB, bool FUSED, bool LAT>
+template <bool ENERGY, int WARPS, int MINB, int MODE, bool LAT>
 __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w1, int nblk_pairs, int a0, int a1,
                                                           int nblk_bonded, int alch_warps) {
     __shared__ std::conditional_t<LAT, PairSharedLat<WARPS>, PairShared<WARPS>> sh;
@@ -747,12 +758,12 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w
     const int nblk_alch = gridDim.x - nblk_pairs - nblk_bonded;
     if ((int)blockIdx.x < nblk_alch) {
         if ((int)(threadIdx.x >> 5) < alch_warps)
-            alch_items<ENERGY, WARPS, FUSED>(d, w0, w1, a0, a1, (threadIdx.x >> 5) * nblk_alch + blockIdx.x,
+            alch_items<ENERGY, WARPS, MODE>(d, w0, w1, a0, a1, (threadIdx.x >> 5) * nblk_alch + blockIdx.x,
                                              alch_warps * nblk_alch);
         return;
     }
-    if (FUSED && (int)blockIdx.x < nblk_alch + nblk_bonded) {
-        bonded_items(d, w0, w1, blockIdx.x - nblk_alch, nblk_bonded);
+    if (MODE != PAIRS && (int)blockIdx.x < nblk_alch + nblk_bonded) {
+        bonded_items<ENERGY>(d, w0, w1, blockIdx.x - nblk_alch, nblk_bonded);
         return;
     }
     if (threadIdx.x < 32) {  // prefix of the walkers' work items
@@ -774,11 +785,11 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w
         }
     }
     __syncthreads();
-    normal_items<ENERGY, WARPS, FUSED ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
+    normal_items<ENERGY, WARPS, MODE == STEP ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
 }
 
-template <bool ENERGY, int WARPS, int MINB, bool LAT>
-static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s, bool fused = false) {
+template <bool ENERGY, int WARPS, int MINB, int MODE, bool LAT>
+static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {
     int nblk = hv.pair_blocks * 8 / WARPS;  // pair_blocks counts 8-warp CTAs
     {  // no more blocks than a quarter above the items need (the queue serves any number)
         long long items = 0;
@@ -792,19 +803,18 @@ static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cud
     // SM.  They live on FP64 sums, and an SM's FP64 pipe does 1.9 lanes per
     // clock: eight of them in one block took turns on it (42 instead of 30 us
     // for the fused launch of 8 walkers x 772 atoms with theta statistics).
-    const int aitems = a1 - a0 + (fused ? w1 - w0 : 0);
+    const int aitems = a1 - a0 + (MODE != PAIRS ? w1 - w0 : 0);
     int awarps = (aitems + hv.n_sm - 1) / hv.n_sm;
     awarps = awarps < 1 ? 1 : (awarps > WARPS ? WARPS : awarps);
     const int ablk = (aitems + awarps - 1) / awarps;
     int bblk = 0;
-    if (fused) {  // bonded terms: about four per thread
+    if (MODE != PAIRS) {  // bonded terms: about four per thread
         const int nbo = hv.bo_off[w1 - 1] + hv.n_bo[w1 - 1] - hv.bo_off[w0];
         bblk = (nbo + 4 * WARPS * 32 - 1) / (4 * WARPS * 32);
         bblk = bblk > hv.n_sm ? hv.n_sm : bblk;
     }
     const int grid = ablk + bblk + nblk;
-    if (fused) k_pairs<ENERGY, WARPS, MINB, true, LAT><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, bblk, awarps);
-    else k_pairs<ENERGY, WARPS, MINB, false, LAT><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, 0, awarps);
+    k_pairs<ENERGY, WARPS, MINB, MODE, LAT><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, bblk, awarps);
 }
 
 // launches whose items leave an SM few enough of them take the latency form
@@ -814,21 +824,25 @@ static bool few_items(const HostView &hv, int w0, int w1) {
     return n <= (long long)LAT_ITEMS_PER_SM * hv.n_sm;
 }
 
-static void launch_pairs_any(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s, bool fused) {
-    if (hv.pair_variant == 0 && few_items(hv, w0, w1)) launch_pairs_v<false, 4, 4, true>(d, hv, w0, w1, s, fused);
-    else if (hv.pair_variant == 1) launch_pairs_v<false, 4, 7, false>(d, hv, w0, w1, s, fused);
-    else if (hv.pair_variant == 2) launch_pairs_v<false, 4, 8, false>(d, hv, w0, w1, s, fused);
-    else launch_pairs_v<false, 8, 3, false>(d, hv, w0, w1, s, fused);
+template <int MODE>
+static void launch_pairs_any(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {
+    if (hv.pair_variant == 0 && few_items(hv, w0, w1)) launch_pairs_v<false, 4, 4, MODE, true>(d, hv, w0, w1, s);
+    else if (hv.pair_variant == 1) launch_pairs_v<false, 4, 7, MODE, false>(d, hv, w0, w1, s);
+    else if (hv.pair_variant == 2) launch_pairs_v<false, 4, 8, MODE, false>(d, hv, w0, w1, s);
+    else launch_pairs_v<false, 8, 3, MODE, false>(d, hv, w0, w1, s);
 }
 
 void launch_pairs_fused(const Dev &d, const HostView &hv, int n_stages, cudaStream_t s) {
     (void)n_stages;
-    launch_pairs_any(d, hv, 0, hv.n_walkers, s, true);
+    launch_pairs_any<STEP>(d, hv, 0, hv.n_walkers, s);
 }
 
-void launch_pairs(const Dev &d, const HostView &hv, int w0, int w1, bool energy, cudaStream_t s) {
-    if (energy) launch_pairs_v<true, 8, 3, false>(d, hv, w0, w1, s);
-    else launch_pairs_any(d, hv, w0, w1, s, false);
+void launch_pairs(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {
+    launch_pairs_any<PAIRS>(d, hv, w0, w1, s);
+}
+
+void launch_pairs_energy(const Dev &d, const HostView &hv, int w, cudaStream_t s) {
+    launch_pairs_v<true, 8, 3, EVAL, false>(d, hv, w, w + 1, s);
 }
 
 }  // namespace labf

@@ -484,19 +484,32 @@ int kernels_per_step(la_handle *h) {
 }
 
 // evaluate forces, dU/dlambda and G at the current state of walkers [w0, w1)
-int prime(la_handle *h, int w0, int w1, bool force_rebuild, bool energy, cudaStream_t s) {
+int prime(la_handle *h, int w0, int w1, bool force_rebuild, cudaStream_t s) {
     // (any non-zero value marks a walker)
     if (force_rebuild) CU(h, cudaMemsetAsync(h->d.rebuild + w0, 1, sizeof(int) * (w1 - w0), s));
     const size_t g0 = h->slot_off[w0], g1 = (size_t)h->slot_off[w1 - 1] + h->slot_cap[w1 - 1];
     CU(h, cudaMemsetAsync(h->d.F + 3 * g0, 0, 3 * (g1 - g0) * sizeof(unsigned long long), s));
-    if (energy) CU(h, cudaMemsetAsync(h->d.eterm + (size_t)N_ETERMS * w0, 0,
-                                      sizeof(long long) * N_ETERMS * (w1 - w0), s));
     launch_rebuild(h->d, h->hv, w0, w1, s);
-    launch_pairs(h->d, h->hv, w0, w1, energy, s);
-    launch_bonded(h->d, h->hv, w0, w1, energy, s);
-    launch_walker(h->d, w0, w1, energy, s);
+    launch_pairs(h->d, h->hv, w0, w1, s);
+    launch_bonded(h->d, h->hv, w0, w1, s);
+    launch_walker(h->d, w0, w1, s);
     launch_lambda(h->d, 0, (int)h->stages.size(), true, s);
     h->launches += 4 + rebuild_kernel_count(h->hv, w0, w1);
+    CU(h, cudaGetLastError());
+    return LA_OK;
+}
+
+// energies, forces, dU/dlambda and theta derivatives of one walker, at
+// positions, parameters and lambda from device arrays where given; out and
+// forces as in k_ef_out
+int evaluate(la_handle *h, int w, bool rebuild, const float *x, const double *theta, const double *lam, double *out,
+             float *forces, cudaStream_t s) {
+    const SysDev &S = h->sys[h->walk[w].sys];
+    launch_ef_in(h->d, w, S.n_atoms, h->slot_cap[w], x, theta, lam, rebuild, s);
+    launch_rebuild(h->d, h->hv, w, w + 1, s);
+    launch_pairs_energy(h->d, h->hv, w, s);
+    launch_ef_out(h->d, w, S.n_atoms, S.P, out, forces, s);
+    h->launches += 3 + rebuild_kernel_count(h->hv, w, w + 1);
     CU(h, cudaGetLastError());
     return LA_OK;
 }
@@ -507,7 +520,7 @@ int prime(la_handle *h, int w0, int w1, bool force_rebuild, bool energy, cudaStr
 int flush_dirty(la_handle *h, cudaStream_t s) {
     if (!h->dirty) return LA_OK;
     h->dirty = false;
-    return prime(h, 0, h->L.W, false, false, s);
+    return prime(h, 0, h->L.W, false, s);
 }
 
 // `steps` MD steps as one graph.  Each step: integrate, gate -> IF(some walker
@@ -590,9 +603,9 @@ int refresh_forces(la_handle *h, cudaStream_t s) {
     const int W = h->L.W;
     const size_t g1 = (size_t)h->slot_off[W - 1] + h->slot_cap[W - 1];
     CU(h, cudaMemsetAsync(h->d.F, 0, 3 * g1 * sizeof(unsigned long long), s));
-    launch_pairs(h->d, h->hv, 0, W, false, s);
-    launch_bonded(h->d, h->hv, 0, W, false, s);
-    launch_walker(h->d, 0, W, false, s);
+    launch_pairs(h->d, h->hv, 0, W, s);
+    launch_bonded(h->d, h->hv, 0, W, s);
+    launch_walker(h->d, 0, W, s);
     launch_lambda(h->d, 0, (int)h->stages.size(), true, s);
     CU(h, cudaGetLastError());
     return LA_OK;
@@ -659,9 +672,9 @@ int tune_pairs(la_handle *h, cudaStream_t s, bool use_cache) {
                 h->hv.pair_variant = m;
                 for (int c : ctas) {
                     set_pair_blocks(h, c);
-                    for (int r = 0; r < 2; ++r) launch_pairs(h->d, h->hv, 0, W, false, s);  // warm
+                    for (int r = 0; r < 2; ++r) launch_pairs(h->d, h->hv, 0, W, s);  // warm
                     CU(h, cudaEventRecord(a, s));
-                    for (int r = 0; r < 10; ++r) launch_pairs(h->d, h->hv, 0, W, false, s);
+                    for (int r = 0; r < 10; ++r) launch_pairs(h->d, h->hv, 0, W, s);
                     CU(h, cudaEventRecord(b, s));
                     CU(h, cudaEventSynchronize(b));
                     float ms = 0.f;
@@ -1052,7 +1065,7 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     CU(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     CU(h, cudaStreamCreateWithFlags(&h->cap_stream2, cudaStreamNonBlocking));
 
-    rc = prime(h, 0, L.W, true, false, s);
+    rc = prime(h, 0, L.W, true, s);
     if (rc != LA_OK) return rc;
     rc = sync_status(h, s, nullptr);
     if (rc != LA_OK) return rc;
@@ -1120,9 +1133,9 @@ int la_step_walkers_plain(la_handle *h, int64_t n_steps, void *stream) {
         h->launches += 1;
         for (int w = 0; w < W; ++w) {
             launch_rebuild(h->d, h->hv, w, w + 1, s);
-            launch_pairs(h->d, h->hv, w, w + 1, false, s);
-            launch_bonded(h->d, h->hv, w, w + 1, false, s);
-            launch_walker(h->d, w, w + 1, false, s);
+            launch_pairs(h->d, h->hv, w, w + 1, s);
+            launch_bonded(h->d, h->hv, w, w + 1, s);
+            launch_walker(h->d, w, w + 1, s);
             h->launches += 3 + rebuild_kernel_count(h->hv, w, w + 1) + (h->n_bo[w] > 0 ? 1 : 0);
         }
         launch_lambda(h->d, 0, (int)h->stages.size(), false, s);
@@ -1191,11 +1204,10 @@ int la_energy_forces(la_handle *h, int walker, uint32_t flags, double *energy_te
     int rc = flush_dirty(h, s);
     if (rc != LA_OK) return rc;
     if (flags & LA_EF_COUNT_PAIRS) CU(h, cudaMemsetAsync(h->d.counters + 1, 0, 2 * sizeof(unsigned long long), s));
-    rc = prime(h, walker, walker + 1, (flags & LA_EF_REBUILD) != 0, true, s);
+    rc = evaluate(h, walker, (flags & LA_EF_REBUILD) != 0, nullptr, nullptr, nullptr, nullptr, forces, s);
     if (rc != LA_OK) return rc;
     const WalkerDev &W = h->walk[walker];
     const SysDev &S = h->sys[W.sys];
-    if (forces) launch_forces_out(h->d, walker, S.n_atoms, forces, s);
     Stage stage_io(h, s);
     const long long *et;
     const double *sw, *th;
@@ -1226,17 +1238,10 @@ int la_energy_forces_device(la_handle *h, int walker, const float *x, const doub
     if (rc != LA_OK) return rc;
     const WalkerDev &W = h->walk[walker];
     const SysDev &S = h->sys[W.sys];
-    if (theta) {
-        launch_alch_params_in(h->d, W.sys, S.n_alch, theta, s);
-        h->dirty = true;  // the system's other walkers refresh before their next use
-    }
-    if (x) launch_positions_in(h->d, walker, S.n_atoms, x, s);
-    if (lam) CU(h, cudaMemcpyAsync(h->d.lam + walker, lam, sizeof(double), cudaMemcpyDeviceToDevice, s));
-    rc = prime(h, walker, walker + 1, false, true, s);
+    // new parameters: the system's other walkers refresh before their next use
+    if (theta && S.w_count > 1) h->dirty = true;
+    rc = evaluate(h, walker, false, x, theta, lam, out, forces, s);
     if (rc != LA_OK) return rc;
-    if (forces) launch_forces_out(h->d, walker, S.n_atoms, forces, s);
-    if (out) launch_ef_out(h->d, walker, S.P, out, s);
-    CU(h, cudaGetLastError());
     post_status(h, s);
     return LA_OK;
 }
@@ -1449,7 +1454,7 @@ int la_set_alch_params(la_handle *h, int sys, const double *theta, void *stream)
     const int w0 = h->sys_w0[sys];
     int w1 = w0;
     while (w1 < h->L.W && h->walk[w1].sys == sys) ++w1;
-    int rc = prime(h, w0, w1, true, false, s);
+    int rc = prime(h, w0, w1, true, s);
     if (rc != LA_OK) return rc;
     return sync_status(h, s, nullptr);
 }

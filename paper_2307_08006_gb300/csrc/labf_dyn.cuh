@@ -302,16 +302,15 @@ __device__ __forceinline__ void theta_terms(const Dev &d, const WalkerDev &W, co
     d2 = (c < 2 ? dlv : dle) * __ldcg(o + 3);
 }
 
-// the walker's restraints and its sample, one warp (one-task launches); with
-// ENERGY also the energy terms and the theta derivatives
+// the walker's sample from the partial sums of its alchemical atoms and its
+// restraints, one warp; with ENERGY also the energy terms and the theta
+// derivatives
 template <bool ENERGY>
-__device__ __forceinline__ void walker_work(const Dev &d, int w, int lane) {
+__device__ __forceinline__ void walker_sample(const Dev &d, int w, int lane) {
     const WalkerDev &W = d.walk[w];
     const SysDev &S = d.sys[W.sys];
     double lv, le, dlv, dle;
     lambda_path(d.lam[w], S.b_v, S.b_e, lv, le, dlv, dle);
-    walker_restraints(d, w, lane);
-    __syncwarp();
     // four lanes per component
     const double v = alch_sum4(d, W.alch_base, S.n_alch, (lane >> 2) & 3, lane & 3, lane < (ENERGY ? 16 : 8));
     const double se = __shfl_sync(0xffffffffu, v, 4), usc = __shfl_sync(0xffffffffu, v, 8),
@@ -331,6 +330,13 @@ __device__ __forceinline__ void walker_work(const Dev &d, int w, int lane) {
         double *th = d.wth + (size_t)w * 2 * d.P_max;
         for (int p = lane; p < S.P; p += 32) theta_terms(d, W, S, w, p, dlv, dle, th[p], th[d.P_max + p]);
     }
+}
+
+// restraints and sample of a walker, one warp (one-task launches)
+__device__ __forceinline__ void walker_work(const Dev &d, int w, int lane) {
+    walker_restraints(d, w, lane);
+    __syncwarp();
+    walker_sample<false>(d, w, lane);
 }
 
 // ---------------------------------------------------------------------------

@@ -35,18 +35,19 @@ int rebuild_kernel_count(const HostView &hv, int w0, int w1);
 // rebuild coalescing of the one-walker-per-launch form (the batched step's
 // gate does the same)
 void launch_coalesce(const Dev &d, int w0, int w1, cudaStream_t s);
-void launch_pairs(const Dev &d, const HostView &hv, int w0, int w1, bool energy, cudaStream_t s);
+void launch_pairs(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s);
+// pairs, bonded terms and restraints of one walker with energies and derivatives
+void launch_pairs_energy(const Dev &d, const HostView &hv, int w, cudaStream_t s);
 // pairs + bonded + walker terms + lambda update of all walkers in one launch
 void launch_pairs_fused(const Dev &d, const HostView &hv, int n_stages, cudaStream_t s);
-void launch_bonded(const Dev &d, const HostView &hv, int w0, int w1, bool energy, cudaStream_t s);
-void launch_walker(const Dev &d, int w0, int w1, bool energy, cudaStream_t s);
+void launch_bonded(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s);
+void launch_walker(const Dev &d, int w0, int w1, cudaStream_t s);
 void launch_lambda(const Dev &d, int s0, int s1, bool prime, cudaStream_t s);
 void launch_state_io(const Dev &d, int w, int n, float *x, float *v, bool to_slots, cudaStream_t s);
 void launch_states_io(const Dev &d, int rows, float *x, float *v, bool to_slots, cudaStream_t s);
-void launch_forces_out(const Dev &d, int w, int n, float *out, cudaStream_t s);
 void launch_lambda_path(const double *lam, int n, double bv, double be, double *out, cudaStream_t s);
-void launch_positions_in(const Dev &d, int w, int n, const float *x, cudaStream_t s);
-void launch_alch_params_in(const Dev &d, int sys, int n_alch, const double *theta, cudaStream_t s);
-void launch_ef_out(const Dev &d, int w, int P, double *out, cudaStream_t s);
+void launch_ef_in(const Dev &d, int w, int n, int slots, const float *x, const double *theta, const double *lam,
+                  bool rebuild, cudaStream_t s);
+void launch_ef_out(const Dev &d, int w, int n, int P, double *out, float *forces, cudaStream_t s);
 
 }  // namespace labf
