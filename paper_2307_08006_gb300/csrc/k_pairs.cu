@@ -5,19 +5,29 @@
 //
 // Normal pairs: warps take work items (a chunk of one super-cluster's
 // j-list) from a global counter.  The super-cluster's 64 slots sit in shared
-// memory.  Entries are prepared 32 at a time, one per lane (header, periodic
-// shift applied to the 4 j-atoms, lane mask bytes), into shared memory; then
-// for each entry lane (ia, jb) = (lane & 7, lane >> 3) evaluates the pair
-// (i-atom ia of every flagged i-cluster, j-atom jb).  One j-cluster load and
+// memory.  Entries are prepared 32 at a time into shared memory (headers one
+// per lane, then eight entries' j-atoms per round with the periodic shift
+// applied, lane mask bytes as one contiguous copy); then for each entry lane
+// (ia, jb) = (lane >> 2, lane & 3) evaluates the pair (i-atom ia of every
+// flagged i-cluster, j-atom jb).  Four neighbouring lanes share an i-atom, so
+// the i-cluster's 128-bit shared loads take half the passes they took with
+// ia = lane & 7; neighbouring lanes also gather one j-cluster's atoms
+// together, and write them without bank conflicts, where each lane fetched a
+// whole entry (a gather of 32 rows per load).  The shared-memory pipe was 62%
+// busy before, second only to the issue slots (73%).  One j-cluster load and
 // one j-force reduction serve up to 8 x 32 pairs, and the eight i-force
 // accumulators stay in registers for the whole item.  Forces are summed in
 // FP32 and added to the 64-bit fixed-point force array with integer atomics
 // (order-free, so results are bit-reproducible).  The i-forces are flushed
 // to the fixed-point array after every 32 entries of a super-cluster's list,
 // so every kernel variant and work-item size (a multiple of 32 entries)
-// produces the same bits.  All float-to-fixed conversions use integer
-// instructions: the hardware conversion to 64-bit integers runs on the FP64
-// pipe, which is narrow on this GPU.
+// produces the same bits.  A lane whose pair is out of the cutoff skips its
+// six accumulating instructions by predicate (no select to zero per tile).
+// All float-to-fixed conversions use integer instructions: the hardware
+// conversion to 64-bit integers runs on the FP64 pipe, which is narrow on this
+// GPU.  Fused launch before / after the lane map, the staging and the
+// predicated sums: 16 x 12 300 atoms 255 / 242 us, 144 x 772 atoms 127 / 117
+// us, 2 x 9020 atoms 47 / 43 us, 16 x 96 040 atoms 2600 / 2485 us.
 //
 // Per in-cutoff pair (force only), 37 FP32 flops (FMA = 2) plus one rsqrt:
 //   d = x_i - x_j (3), r2 (5), 1/r2 (1), sigma_ij = s_i + s_j, (sigma/r)^2,
@@ -95,7 +105,7 @@ __device__ __forceinline__ void flush_i(const Dev &d, int gS, int ia, int jb, un
         for (int c = 0; c < 3; ++c) {
             const float keep = odd ? fi[ko][c] : fi[ke][c];
             const float send = odd ? fi[ke][c] : fi[ko][c];
-            k1[t][c] = keep + __shfl_xor_sync(FULL, send, 8);
+            k1[t][c] = keep + __shfl_xor_sync(FULL, send, 1);
         }
     }
 #pragma unroll
@@ -107,7 +117,7 @@ __device__ __forceinline__ void flush_i(const Dev &d, int gS, int ia, int jb, un
         for (int c = 0; c < 3; ++c) {
             const float keep = upper ? k1[t + 2][c] : k1[t][c];
             const float send = upper ? k1[t][c] : k1[t + 2][c];
-            const float v = keep + __shfl_xor_sync(FULL, send, 16);
+            const float v = keep + __shfl_xor_sync(FULL, send, 2);
             if (on) atomicAdd(p + c, f2fix(v));
         }
     }
@@ -131,15 +141,15 @@ __device__ __forceinline__ void flush_j2(const Dev &d, int gjA, int gjB, bool ha
     for (int c = 0; c < 3; ++c) {
         const float keep = h4 ? b[c] : a[c];
         const float send = h4 ? a[c] : b[c];
-        v[c] = keep + __shfl_xor_sync(FULL, send, 4);
+        v[c] = keep + __shfl_xor_sync(FULL, send, 16);
     }
     // (x, y) kept by h2 = 0, (z, 0) by h2 = 1
     const float k0 = h2 ? v[2] : v[0], k1 = h2 ? 0.f : v[1];
     const float s0 = h2 ? v[0] : v[2], s1 = h2 ? v[1] : 0.f;
-    const float w0 = k0 + __shfl_xor_sync(FULL, s0, 2);
-    const float w1 = k1 + __shfl_xor_sync(FULL, s1, 2);
+    const float w0 = k0 + __shfl_xor_sync(FULL, s0, 8);
+    const float w1 = k1 + __shfl_xor_sync(FULL, s1, 8);
     const float kk = h1 ? w1 : w0, ss = h1 ? w0 : w1;
-    const float c = kk + __shfl_xor_sync(FULL, ss, 1);
+    const float c = kk + __shfl_xor_sync(FULL, ss, 4);
     const int comp = ia & 3;
     if (comp < 3 && (h4 ? has_b : has_a)) atomicAdd(d.F + 3 * (size_t)(h4 ? gjB : gjA) + comp, f2fix(-c));
 }
@@ -156,7 +166,7 @@ template <bool ENERGY, int WARPS, int MSHIFT, bool PRUNE>
 __device__ __forceinline__ int item_entries(const Dev &d, PairShared<WARPS> &sh, const SysDev &S, int4 it, int gS,
                                             float &elj, float &erf, int &npair) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int ia = lane & 7, jb = lane >> 3;
+    const int ia = lane >> 2, jb = lane & 3, lbi = jb * IC + ia;
     const float L = S.boxf, rc2 = S.rc2, krf2 = 2.0f * S.krf, krf = S.krf, crf = S.crf;
     const float rp2 = S.rprune2;
     float fi[NIC][3];
@@ -177,22 +187,31 @@ __device__ __forceinline__ int item_entries(const Dev &d, PairShared<WARPS> &sh,
             hy_l = hdr.y;
             im_l = ((unsigned)hdr.y >> (PRUNE ? 16 : MSHIFT)) & 0xffu;
             if (!la_in(d, gj_l, d.n_slots - JC + 1)) gj_l = 0, im_l = 0;  // entry skipped
-            const float sx = (float)((hdr.y & 3) - 1) * L;
-            const float sy = (float)(((hdr.y >> 2) & 3) - 1) * L;
-            const float sz = (float)(((hdr.y >> 4) & 3) - 1) * L;
+        }
+        // lane masks: the entries' bytes are contiguous
+        {
+            const uint4 *src = reinterpret_cast<const uint4 *>(d.ent_lb + 32 * (ebase + eb));
+            uint4 *dst = reinterpret_cast<uint4 *>(&sh.lb[wib][0][0]);
 #pragma unroll
-            for (int q = 0; q < JC; ++q) {
-                float4 x = d.xq[gj_l + q];
-                x.x += sx;
-                x.y += sy;
-                x.z += sz;
-                sh.jx[wib][lane][q] = x;
-                sh.jl[wib][lane][q] = d.lj[gj_l + q];
-            }
-            const uint4 *src = reinterpret_cast<const uint4 *>(d.ent_lb + 32 * (ebase + eb + lane));
-            uint4 *dst = reinterpret_cast<uint4 *>(&sh.lb[wib][lane][0]);
-            dst[0] = src[0];
-            dst[1] = src[1];
+            for (int h = 0; h < 2; ++h)
+                if (lane + 32 * h < 2 * ne) dst[lane + 32 * h] = src[lane + 32 * h];
+        }
+        // j-atoms, eight entries per round
+#pragma unroll
+        for (int r = 0; r < EPC / IC; ++r) {
+            const int e = r * IC + (lane >> 2), q = lane & 3;
+            const int g = __shfl_sync(FULL, im_l ? gj_l : -1, e);
+            const int hy = __shfl_sync(FULL, hy_l, e);
+            if (g < 0) continue;  // pruned or absent
+            const float sx = (float)((hy & 3) - 1) * L;
+            const float sy = (float)(((hy >> 2) & 3) - 1) * L;
+            const float sz = (float)(((hy >> 4) & 3) - 1) * L;
+            float4 x = d.xq[g + q];
+            x.x += sx;
+            x.y += sy;
+            x.z += sz;
+            sh.jx[wib][e][q] = x;
+            sh.jl[wib][e][q] = d.lj[g + q];
         }
         // entries whose tiles were all pruned add nothing: skip them
         unsigned emask = __ballot_sync(FULL, im_l != 0u);
@@ -206,7 +225,7 @@ __device__ __forceinline__ int item_entries(const Dev &d, PairShared<WARPS> &sh,
             const unsigned imask = __shfl_sync(FULL, im_l, k);
             const float4 xj = sh.jx[wib][k][jb];
             const float2 lj_j = sh.jl[wib][k][jb];
-            const unsigned lb = sh.lb[wib][k][lane];
+            const unsigned lb = sh.lb[wib][k][lbi];
             touched |= imask;
             float fj[3] = {0.f, 0.f, 0.f};
             unsigned kb = 0;  // this lane's pairs within r_c + margin, per i-cluster
@@ -227,14 +246,15 @@ __device__ __forceinline__ int item_entries(const Dev &d, PairShared<WARPS> &sh,
                     const float e4s6 = li.y * lj_j.y * sr6;
                     const float qq = xi.w * xj.w;
                     const float b = fmaf(qq, rinv, e4s6 * fmaf(12.f, sr6, -6.f));
-                    float fs = fmaf(b, r2inv, -qq * krf2);
-                    fs = in ? fs : 0.f;
-                    fi[ic][0] = fmaf(fs, dx, fi[ic][0]);
-                    fi[ic][1] = fmaf(fs, dy, fi[ic][1]);
-                    fi[ic][2] = fmaf(fs, dz, fi[ic][2]);
-                    fj[0] = fmaf(fs, dx, fj[0]);
-                    fj[1] = fmaf(fs, dy, fj[1]);
-                    fj[2] = fmaf(fs, dz, fj[2]);
+                    const float fs = fmaf(b, r2inv, -qq * krf2);
+                    if (in) {  // predicated
+                        fi[ic][0] = fmaf(fs, dx, fi[ic][0]);
+                        fi[ic][1] = fmaf(fs, dy, fi[ic][1]);
+                        fi[ic][2] = fmaf(fs, dz, fi[ic][2]);
+                        fj[0] = fmaf(fs, dx, fj[0]);
+                        fj[1] = fmaf(fs, dy, fj[1]);
+                        fj[2] = fmaf(fs, dz, fj[2]);
+                    }
                     if (ENERGY) {
                         if (in) {
                             elj += e4s6 * (sr6 - 1.f);
@@ -303,7 +323,7 @@ __device__ __noinline__ int item_entries_prune(const Dev &d, PairShared<WARPS> &
 template <int WARPS, int MSHIFT, bool PRUNE>
 __device__ __forceinline__ int item_entries_lat(const Dev &d, PairSharedLat<WARPS> &sh, const SysDev &S, int4 it, int gS) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int ia = lane & 7, jb = lane >> 3;
+    const int ia = lane >> 2, jb = lane & 3, lbi = jb * IC + ia;
     const float L = S.boxf, rc2 = S.rc2, rp2 = S.rprune2, krf2 = 2.0f * S.krf;
     const f2 nkrf2 = pack2(-krf2, -krf2), c12 = pack2(12.f, 12.f), c6 = pack2(-6.f, -6.f);
     f2 fi[NIC / 2][3];
@@ -323,23 +343,32 @@ __device__ __forceinline__ int item_entries_lat(const Dev &d, PairSharedLat<WARP
             hy_l = hdr.y;
             im_l = ((unsigned)hdr.y >> (PRUNE ? 16 : MSHIFT)) & 0xffu;
             if (!la_in(d, gj_l, d.n_slots - JC + 1)) gj_l = 0, im_l = 0;  // entry skipped
-            const float sx = (float)((hdr.y & 3) - 1) * L;
-            const float sy = (float)(((hdr.y >> 2) & 3) - 1) * L;
-            const float sz = (float)(((hdr.y >> 4) & 3) - 1) * L;
+        }
+        // lane masks: the entries' bytes are contiguous
+        {
+            const uint4 *src = reinterpret_cast<const uint4 *>(d.ent_lb + 32 * (ebase + eb));
+            uint4 *dst = reinterpret_cast<uint4 *>(&sh.lb[wib][0][0]);
 #pragma unroll
-            for (int q = 0; q < JC; ++q) {
-                const float4 x = d.xq[gj_l + q];
-                const float2 l = d.lj[gj_l + q];
-                const float nx = -(x.x + sx), ny = -(x.y + sy), nz = -(x.z + sz);
-                float4 *row = &sh.j[wib][lane][3 * q];
-                row[0] = make_float4(nx, nx, ny, ny);
-                row[1] = make_float4(nz, nz, x.w, x.w);
-                row[2] = make_float4(l.x, l.x, l.y, l.y);
-            }
-            const uint4 *src = reinterpret_cast<const uint4 *>(d.ent_lb + 32 * (ebase + eb + lane));
-            uint4 *dst = reinterpret_cast<uint4 *>(&sh.lb[wib][lane][0]);
-            dst[0] = src[0];
-            dst[1] = src[1];
+            for (int h = 0; h < 2; ++h)
+                if (lane + 32 * h < 2 * ne) dst[lane + 32 * h] = src[lane + 32 * h];
+        }
+        // j-atoms, eight entries per round
+#pragma unroll
+        for (int r = 0; r < EPC / IC; ++r) {
+            const int e = r * IC + (lane >> 2), q = lane & 3;
+            const int g = __shfl_sync(FULL, im_l ? gj_l : -1, e);
+            const int hy = __shfl_sync(FULL, hy_l, e);
+            if (g < 0) continue;  // pruned or absent
+            const float sx = (float)((hy & 3) - 1) * L;
+            const float sy = (float)(((hy >> 2) & 3) - 1) * L;
+            const float sz = (float)(((hy >> 4) & 3) - 1) * L;
+            const float4 x = d.xq[g + q];
+            const float2 l = d.lj[g + q];
+            const float nx = -(x.x + sx), ny = -(x.y + sy), nz = -(x.z + sz);
+            float4 *row = &sh.j[wib][e][3 * q];
+            row[0] = make_float4(nx, nx, ny, ny);
+            row[1] = make_float4(nz, nz, x.w, x.w);
+            row[2] = make_float4(l.x, l.x, l.y, l.y);
         }
         unsigned emask = __ballot_sync(FULL, im_l != 0u);
         __syncwarp();
@@ -404,7 +433,7 @@ __device__ __forceinline__ int item_entries_lat(const Dev &d, PairSharedLat<WARP
             const bool pair = emask != 0u;
             const int k1 = pair ? __ffs(emask) - 1 : k0;
             emask &= emask - 1u;
-            const unsigned lb0 = sh.lb[wib][k0][lane], lb1 = pair ? sh.lb[wib][k1][lane] : 0u;
+            const unsigned lb0 = sh.lb[wib][k0][lbi], lb1 = pair ? sh.lb[wib][k1][lbi] : 0u;
             float na[3], nb[3];
             if (PRUNE && !pair) {
                 entry(k0, lb0, na);

@@ -144,7 +144,7 @@ struct Dev {
     int4 *bb_sc, *bb_ic, *bb_jc;  // (lo, hi) pairs; lo.w = real count
     int *sc_nent;
     int2 *ent_hdr;                // (j-cluster base global slot, shift bits | imask << 8)
-    unsigned char *ent_lb;        // 32 per entry: lane l's bit ic = pair (8 ic + (l & 7), l >> 3)
+    unsigned char *ent_lb;        // 32 per entry: byte 8 jb + ia, bit ic = pair (8 ic + ia, jb)
     int4 *items;                  // (global sc, e0, e1, walker)
     int *n_items;
     // alchemical lists and partial sums
