@@ -73,15 +73,18 @@ struct PairShared {
 
 // Shared memory of the latency form: the super-cluster's i-clusters two by
 // two (row (p, ia): atom ia of i-clusters 2p and 2p + 1 as {x x' y y'},
-// {z z' q q'}, {s s' e e'}) and the prepared j-atoms with every value twice
-// (position negated), so that packed operands are loaded as they are.
-template <int WARPS>
+// {z z' q q'}, {s s' e e'}), the prepared j-atoms with every value twice
+// (position negated), so that packed operands are loaded as they are, and the
+// pairs' forces over distance.
 struct PairSharedLat {
-    float4 si[WARPS][3][SC / 2];
-    float4 j[WARPS][EPC][3 * JC];
-    unsigned char lb[WARPS][EPC][32];
-    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], first;
+    float4 si[3][SC / 2];
+    float4 j[EPC][3 * JC];
+    unsigned char lb[EPC][32];
+    float2 f[EPC][NIC / 2][32];
+    unsigned char keep[EPC][NIC / 2];
+    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], first, next;
 };
+constexpr int LAT_WARPS = NIC / 2;
 
 // counters[4] hands out work items; counters[5] counts warps that found no
 // more work; the last one resets both for the next launch
@@ -134,7 +137,7 @@ __device__ __forceinline__ void flush_i(const Dev &d, int gS, int ia, int jb, un
 // Each sum is ((a0 + a4) + (a2 + a6)) + ((a1 + a5) + (a3 + a7)), whether or
 // not B is present.
 __device__ __forceinline__ void flush_j2(const Dev &d, int gjA, int gjB, bool has_b, int ia, const float (&a)[3],
-                                         const float (&b)[3], bool has_a = true) {
+                                         const float (&b)[3]) {
     const bool h4 = (ia & 4) != 0, h2 = (ia & 2) != 0, h1 = (ia & 1) != 0;
     float v[3];
 #pragma unroll
@@ -151,7 +154,7 @@ __device__ __forceinline__ void flush_j2(const Dev &d, int gjA, int gjB, bool ha
     const float kk = h1 ? w1 : w0, ss = h1 ? w0 : w1;
     const float c = kk + __shfl_xor_sync(FULL, ss, 4);
     const int comp = ia & 3;
-    if (comp < 3 && (h4 ? has_b : has_a)) atomicAdd(d.F + 3 * (size_t)(h4 ? gjB : gjA) + comp, f2fix(-c));
+    if (comp < 3 && (!h4 || has_b)) atomicAdd(d.F + 3 * (size_t)(h4 ? gjB : gjA) + comp, f2fix(-c));
 }
 
 // One work item's entries, prepared and evaluated 32 at a time; the
@@ -314,29 +317,39 @@ __device__ __noinline__ int item_entries_prune(const Dev &d, PairShared<WARPS> &
 
 // The same item for launches with few items (at most LAT_ITEMS_PER_SM per SM:
 // one or two boxes, small batches), where an item's own latency decides, not
-// the issue rate.  The eight tiles of an entry are evaluated without branches,
-// two i-clusters per packed FP32 instruction, so that their dependency chains
-// overlap; unlisted tiles add exact zeros, and every sum keeps the order of
-// the common form (i-forces: one entry after the other; j-forces: i-clusters
-// ascending), so the forces are the same bits.  The common form tests each
-// i-cluster and skips 46% of the tiles, with one chain at a time.
-template <int WARPS, int MSHIFT, bool PRUNE>
-__device__ __forceinline__ int item_entries_lat(const Dev &d, PairSharedLat<WARPS> &sh, const SysDev &S, int4 it, int gS) {
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+// the issue rate: a block of four warps takes it.
+//   1  warp p evaluates i-clusters 2p and 2p + 1 against all entries, both in
+//      one packed FP32 instruction and without branches, sums their i-forces
+//      and leaves every pair's force over distance in shared memory
+//   2  the entries are dealt out to the warps again, which add the j-forces
+//      over all i-clusters from those factors
+// Every sum keeps the order of the common form (i-forces: one entry after the
+// other; j-forces: i-clusters ascending; skipped pairs add exact zeros), so
+// the forces are the same bits.  One warp per item took 13 us for its 32
+// entries one after the other.
+template <int MSHIFT, bool PRUNE>
+__device__ __forceinline__ void item_entries_lat(const Dev &d, PairSharedLat &sh, const SysDev &S, int4 it, int gS) {
+    const int tid = threadIdx.x, lane = tid & 31, p = tid >> 5;
     const int ia = lane >> 2, jb = lane & 3, lbi = jb * IC + ia;
     const float L = S.boxf, rc2 = S.rc2, rp2 = S.rprune2, krf2 = 2.0f * S.krf;
-    const f2 nkrf2 = pack2(-krf2, -krf2), c12 = pack2(12.f, 12.f), c6 = pack2(-6.f, -6.f);
-    f2 fi[NIC / 2][3];
-#pragma unroll
-    for (int p = 0; p < NIC / 2; ++p) fi[p][0] = fi[p][1] = fi[p][2] = 0ull;
-    unsigned touched = 0;
-    int v_next = 0;
+    const unsigned b0 = 1u << (2 * p), b1 = 2u << (2 * p);
     const size_t ebase = (size_t)it.x * d.ent_cap;
+    if (tid < SC) {  // slot tid: atom tid & 7 of i-cluster tid >> 3
+        const float4 x = d.xq[gS + tid];
+        const float2 l = d.lj[gS + tid];
+        float *row = reinterpret_cast<float *>(&sh.si[0][(tid >> 4) * IC + (tid & 7)]) + ((tid >> 3) & 1);
+        row[0] = x.x;
+        row[2] = x.y;
+        row[2 * SC] = x.z;
+        row[2 * SC + 2] = x.w;
+        row[4 * SC] = l.x;
+        row[4 * SC + 2] = l.y;
+    }
     for (int eb = it.y; eb < it.z; eb += EPC) {
         const int ne = min(EPC, it.z - eb);
+        // headers, by every warp; each prepares eight entries' j-atoms
         int gj_l = 0, hy_l = 0;
-        unsigned im_l = 0, keep_l = 0;
-        __syncwarp();
+        unsigned im_l = 0;
         if (lane < ne) {
             const int2 hdr = d.ent_hdr[ebase + eb + lane];
             gj_l = hdr.x;
@@ -344,52 +357,39 @@ __device__ __forceinline__ int item_entries_lat(const Dev &d, PairSharedLat<WARP
             im_l = ((unsigned)hdr.y >> (PRUNE ? 16 : MSHIFT)) & 0xffu;
             if (!la_in(d, gj_l, d.n_slots - JC + 1)) gj_l = 0, im_l = 0;  // entry skipped
         }
-        // lane masks: the entries' bytes are contiguous
+        if (tid < 2 * ne)  // lane masks: the entries' bytes are contiguous
+            reinterpret_cast<uint4 *>(&sh.lb[0][0])[tid] = reinterpret_cast<const uint4 *>(d.ent_lb + 32 * (ebase + eb))[tid];
         {
-            const uint4 *src = reinterpret_cast<const uint4 *>(d.ent_lb + 32 * (ebase + eb));
-            uint4 *dst = reinterpret_cast<uint4 *>(&sh.lb[wib][0][0]);
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-                if (lane + 32 * h < 2 * ne) dst[lane + 32 * h] = src[lane + 32 * h];
-        }
-        // j-atoms, eight entries per round
-#pragma unroll
-        for (int r = 0; r < EPC / IC; ++r) {
-            const int e = r * IC + (lane >> 2), q = lane & 3;
+            const int e = p * IC + (lane >> 2), q = lane & 3;
             const int g = __shfl_sync(FULL, im_l ? gj_l : -1, e);
             const int hy = __shfl_sync(FULL, hy_l, e);
-            if (g < 0) continue;  // pruned or absent
-            const float sx = (float)((hy & 3) - 1) * L;
-            const float sy = (float)(((hy >> 2) & 3) - 1) * L;
-            const float sz = (float)(((hy >> 4) & 3) - 1) * L;
-            const float4 x = d.xq[g + q];
-            const float2 l = d.lj[g + q];
-            const float nx = -(x.x + sx), ny = -(x.y + sy), nz = -(x.z + sz);
-            float4 *row = &sh.j[wib][e][3 * q];
-            row[0] = make_float4(nx, nx, ny, ny);
-            row[1] = make_float4(nz, nz, x.w, x.w);
-            row[2] = make_float4(l.x, l.x, l.y, l.y);
+            if (g >= 0) {
+                const float4 x = d.xq[g + q];
+                const float2 l = d.lj[g + q];
+                const float nx = -(x.x + (float)((hy & 3) - 1) * L), ny = -(x.y + (float)(((hy >> 2) & 3) - 1) * L),
+                            nz = -(x.z + (float)(((hy >> 4) & 3) - 1) * L);
+                float4 *row = &sh.j[e][3 * q];
+                row[0] = make_float4(nx, nx, ny, ny);
+                row[1] = make_float4(nz, nz, x.w, x.w);
+                row[2] = make_float4(l.x, l.x, l.y, l.y);
+            }
         }
-        unsigned emask = __ballot_sync(FULL, im_l != 0u);
-        __syncwarp();
-        auto entry = [&](int k, unsigned lb, float (&fj)[3]) {
-            const ulonglong2 *rj = reinterpret_cast<const ulonglong2 *>(&sh.j[wib][k][3 * jb]);
-            const ulonglong2 j0 = rj[0], j1 = rj[1], j2 = rj[2];
-            unsigned kb = 0;  // this lane's pairs within r_c + margin, per i-cluster
-            fj[0] = fj[1] = fj[2] = 0.f;
-#pragma unroll
-            for (int p = 0; p < NIC / 2; ++p) {
-                const ulonglong2 *si = reinterpret_cast<const ulonglong2 *>(&sh.si[wib][0][p * IC + ia]);
-                const ulonglong2 i0 = si[0], i1 = si[SC / 2], i2 = si[SC];
-                const unsigned b0 = 1u << (2 * p), b1 = 2u << (2 * p);
-                const f2 dx = add2(i0.x, j0.x), dy = add2(i0.y, j0.y), dz = add2(i1.x, j1.x);
-                const f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-                float r20, r21;
-                unpack2(r2, r20, r21);
-                if (PRUNE) {
-                    kb |= ((lb & b0) && r20 < rp2) ? b0 : 0u;
-                    kb |= ((lb & b1) && r21 < rp2) ? b1 : 0u;
-                }
+        if (PRUNE) sh.keep[lane][p] = 0;
+        __syncthreads();
+        // 1: this warp's two i-clusters against the entries that flag one
+        f2 fi[3] = {0ull, 0ull, 0ull};
+        {
+            const ulonglong2 *si = reinterpret_cast<const ulonglong2 *>(&sh.si[0][p * IC + ia]);
+            const ulonglong2 i0 = si[0], i1 = si[SC / 2], i2 = si[SC];
+            const f2 nkrf2 = pack2(-krf2, -krf2), c12 = pack2(12.f, 12.f), c6 = pack2(-6.f, -6.f);
+            auto tile = [&](int k, unsigned lb, f2 &fs, f2 &dx, f2 &dy, f2 &dz) -> unsigned {
+                const ulonglong2 *rj = reinterpret_cast<const ulonglong2 *>(&sh.j[k][3 * jb]);
+                const ulonglong2 j0 = rj[0], j1 = rj[1], j2 = rj[2];
+                dx = add2(i0.x, j0.x);
+                dy = add2(i0.y, j0.y);
+                dz = add2(i1.x, j1.x);
+                float r20, r21, f0, f1;
+                unpack2(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), r20, r21);
                 const bool in0 = (lb & b0) && r20 < rc2, in1 = (lb & b1) && r21 < rc2;
                 const f2 rinv = pack2(rsqrtf(r20), rsqrtf(r21));
                 const f2 r2inv = mul2(rinv, rinv);
@@ -399,100 +399,104 @@ __device__ __forceinline__ int item_entries_lat(const Dev &d, PairSharedLat<WARP
                 const f2 e4s6 = mul2(mul2(i2.y, j2.y), sr6);
                 const f2 qq = mul2(i1.y, j1.y);
                 const f2 b = fma2(qq, rinv, mul2(e4s6, fma2(c12, sr6, c6)));
-                float f0, f1;
                 unpack2(fma2(b, r2inv, mul2(qq, nkrf2)), f0, f1);
-                f0 = in0 ? f0 : 0.f;
-                f1 = in1 ? f1 : 0.f;
-                const f2 fs = pack2(f0, f1);
-                fi[p][0] = fma2(fs, dx, fi[p][0]);
-                fi[p][1] = fma2(fs, dy, fi[p][1]);
-                fi[p][2] = fma2(fs, dz, fi[p][2]);
-                float d0, d1;
-                unpack2(dx, d0, d1);
-                fj[0] = fmaf(f1, d1, fmaf(f0, d0, fj[0]));
-                unpack2(dy, d0, d1);
-                fj[1] = fmaf(f1, d1, fmaf(f0, d0, fj[1]));
-                unpack2(dz, d0, d1);
-                fj[2] = fmaf(f1, d1, fmaf(f0, d0, fj[2]));
+                fs = pack2(in0 ? f0 : 0.f, in1 ? f1 : 0.f);
+                unsigned kb = 0;  // pairs within r_c + margin
+                if (PRUNE) kb = ((lb & b0) && r20 < rp2 ? 1u : 0u) | ((lb & b1) && r21 < rp2 ? 2u : 0u);
+                return kb;
+            };
+            unsigned m = __ballot_sync(FULL, (im_l & (b0 | b1)) != 0u);
+            while (m) {  // two entries per round
+                const int k0 = __ffs(m) - 1;
+                m &= m - 1u;
+                const bool two = m != 0u;
+                const int k1 = two ? __ffs(m) - 1 : k0;
+                m &= m - 1u;
+                f2 fa, fb, ax, ay, az, bx, by, bz;
+                const unsigned ka = tile(k0, sh.lb[k0][lbi], fa, ax, ay, az);
+                const unsigned kb = tile(k1, two ? sh.lb[k1][lbi] : 0u, fb, bx, by, bz);
+                fi[0] = fma2(fb, bx, fma2(fa, ax, fi[0]));
+                fi[1] = fma2(fb, by, fma2(fa, ay, fi[1]));
+                fi[2] = fma2(fb, bz, fma2(fa, az, fi[2]));
+                reinterpret_cast<f2 *>(sh.f[k0][p])[lane] = fa;
+                if (two) reinterpret_cast<f2 *>(sh.f[k1][p])[lane] = fb;
+                if (PRUNE) {
+                    const unsigned keep = __reduce_or_sync(FULL, ka | (kb << 2));
+                    if (lane == 0) {
+                        sh.keep[k0][p] = keep & 3u;
+                        if (two) sh.keep[k1][p] = keep >> 2;
+                    }
+                }
             }
-            if (PRUNE) {
-                const unsigned keep = __reduce_or_sync(FULL, kb);
-                keep_l = lane == k ? keep : keep_l;
-            }
-        };
-        touched = __reduce_or_sync(FULL, im_l);
-        // two entries per round (an odd last one runs with a copy of itself
-        // without pairs); the reduction of the round before shares the block
-        // with their arithmetic
-        float a[3] = {0.f, 0.f, 0.f}, b[3] = {0.f, 0.f, 0.f};
-        int gA = 0, gB = 0;
-        bool any = false, two = false;
-        while (emask) {
-            const int k0 = __ffs(emask) - 1;
-            emask &= emask - 1u;
-            const bool pair = emask != 0u;
-            const int k1 = pair ? __ffs(emask) - 1 : k0;
-            emask &= emask - 1u;
-            const unsigned lb0 = sh.lb[wib][k0][lbi], lb1 = pair ? sh.lb[wib][k1][lbi] : 0u;
-            float na[3], nb[3];
-            if (PRUNE && !pair) {
-                entry(k0, lb0, na);
-                nb[0] = nb[1] = nb[2] = 0.f;
-            } else {
-                entry(k0, lb0, na);
-                entry(k1, lb1, nb);
-            }
-            flush_j2(d, gA, gB, two, ia, a, b, any);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                a[c] = na[c];
-                b[c] = nb[c];
-            }
-            gA = __shfl_sync(FULL, gj_l, k0) + jb;
-            gB = __shfl_sync(FULL, gj_l, k1) + jb;
-            any = true;
-            two = pair;
         }
-        flush_j2(d, gA, gB, two, ia, a, b, any);
-        if (eb + EPC >= it.z && lane == 0) v_next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
-        float f[NIC][3];
+        __syncthreads();
+        // 2: the j-forces of every fourth entry with pairs
+        const unsigned emask = __ballot_sync(FULL, im_l != 0u);
+        unsigned m = __ballot_sync(FULL, im_l != 0u && (__popc(emask & ((1u << lane) - 1u)) & 3) == p);
+        if (m) {
+            f2 ix[NIC / 2], iy[NIC / 2], iz[NIC / 2];
 #pragma unroll
-        for (int p = 0; p < NIC / 2; ++p)
+            for (int q = 0; q < NIC / 2; ++q) {
+                const ulonglong2 i0 = *reinterpret_cast<const ulonglong2 *>(&sh.si[0][q * IC + ia]);
+                ix[q] = i0.x;
+                iy[q] = i0.y;
+                iz[q] = *reinterpret_cast<const f2 *>(&sh.si[1][q * IC + ia]);
+            }
+            auto sum_j = [&](int k, float (&fj)[3]) {
+                const unsigned imask = __shfl_sync(FULL, im_l, k);
+                const ulonglong2 j0 = *reinterpret_cast<const ulonglong2 *>(&sh.j[k][3 * jb]);
+                const f2 jz = *reinterpret_cast<const f2 *>(&sh.j[k][3 * jb + 1]);
+                fj[0] = fj[1] = fj[2] = 0.f;
+#pragma unroll
+                for (int q = 0; q < NIC / 2; ++q) {
+                    // (factors of pairs of i-clusters that no warp evaluated are not read)
+                    const bool on = (imask >> (2 * q)) & 3u;
+                    const float2 f = on ? sh.f[k][q][lane] : make_float2(0.f, 0.f);
+                    float d0, d1;
+                    unpack2(add2(ix[q], j0.x), d0, d1);
+                    fj[0] = fmaf(f.y, d1, fmaf(f.x, d0, fj[0]));
+                    unpack2(add2(iy[q], j0.y), d0, d1);
+                    fj[1] = fmaf(f.y, d1, fmaf(f.x, d0, fj[1]));
+                    unpack2(add2(iz[q], jz), d0, d1);
+                    fj[2] = fmaf(f.y, d1, fmaf(f.x, d0, fj[2]));
+                }
+            };
+            while (m) {
+                const int k0 = __ffs(m) - 1;
+                m &= m - 1u;
+                const bool two = m != 0u;
+                const int k1 = two ? __ffs(m) - 1 : k0;
+                m &= m - 1u;
+                float a[3], b[3];
+                sum_j(k0, a);
+                sum_j(k1, b);
+                const int gA = __shfl_sync(FULL, gj_l, k0) + jb, gB = __shfl_sync(FULL, gj_l, k1) + jb;
+                flush_j2(d, gA, gB, two, ia, a, b);
+            }
+        }
+        // the i-forces: (a0 + a1) + (a2 + a3) over the j-lanes, as flush_i; lane
+        // jb ends with i-cluster 2p + (jb & 1)
+        {
+            const bool odd = (jb & 1) != 0;
+            const bool on = (__reduce_or_sync(FULL, im_l) >> (2 * p + (jb & 1))) & 1u;
+            unsigned long long *F = d.F + 3 * (size_t)(gS + (2 * p + (jb & 1)) * IC + ia);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                unpack2(fi[p][c], f[2 * p][c], f[2 * p + 1][c]);
-                fi[p][c] = 0ull;
+                float e, o;
+                unpack2(fi[c], e, o);
+                float v = (odd ? o : e) + __shfl_xor_sync(FULL, odd ? e : o, 1);
+                v += __shfl_xor_sync(FULL, v, 2);
+                if (on && (jb >> 1) == (c == 2)) atomicAdd(F + c, f2fix(v));
             }
-        flush_i(d, gS, ia, jb, touched, f);
-        if (PRUNE && lane < ne) d.ent_hdr[ebase + eb + lane].y = (hy_l & ~0xff00) | (int)(keep_l << 8);
+        }
+        if (PRUNE && p == 0 && lane < ne) {
+            unsigned keep = 0;
+#pragma unroll
+            for (int q = 0; q < NIC / 2; ++q) keep |= (unsigned)sh.keep[lane][q] << (2 * q);
+            d.ent_hdr[ebase + eb + lane].y = (hy_l & ~0xff00) | (int)(keep << 8);
+        }
+        if (eb + EPC < it.z) __syncthreads();  // shared memory free
     }
-    return v_next;
-}
-
-template <int WARPS>
-__device__ __noinline__ int item_entries_lat_prune(const Dev &d, PairSharedLat<WARPS> &sh, const SysDev &S, int4 it,
-                                                   int gS) {
-    return item_entries_lat<WARPS, 8, true>(d, sh, S, it, gS);
-}
-
-// the item's super-cluster into shared memory, in the layout of either form
-template <int WARPS>
-__device__ __forceinline__ void stage_cluster(const Dev &d, PairShared<WARPS> &sh, int wib, int k, int g) {
-    sh.sxq[wib][k] = d.xq[g];
-    sh.slj[wib][k] = d.lj[g];
-}
-template <int WARPS>
-__device__ __forceinline__ void stage_cluster(const Dev &d, PairSharedLat<WARPS> &sh, int wib, int k, int g) {
-    const float4 x = d.xq[g];
-    const float2 l = d.lj[g];
-    // slot k: atom k & 7 of i-cluster k >> 3
-    float *row = reinterpret_cast<float *>(&sh.si[wib][0][(k >> 4) * IC + (k & 7)]) + ((k >> 3) & 1);
-    row[0] = x.x;
-    row[2] = x.y;
-    row[2 * SC] = x.z;
-    row[2 * SC + 2] = x.w;
-    row[4 * SC] = l.x;
-    row[4 * SC + 2] = l.y;
 }
 
 template <bool ENERGY, int WARPS, int MSHIFT>
@@ -501,17 +505,35 @@ __device__ __forceinline__ int run_item(const Dev &d, PairShared<WARPS> &sh, con
     if (MSHIFT == 8 && d.prune_now[w] != 0ull) return item_entries_prune<WARPS>(d, sh, S, it, gS);
     return item_entries<ENERGY, WARPS, MSHIFT, false>(d, sh, S, it, gS, elj, erf, npair);
 }
-template <bool ENERGY, int WARPS, int MSHIFT>
-__device__ __forceinline__ int run_item(const Dev &d, PairSharedLat<WARPS> &sh, const SysDev &S, int w, int4 it, int gS,
-                                        float &, float &, int &) {
-    static_assert(!ENERGY, "the latency form evaluates forces only");
-    if (MSHIFT == 8 && d.prune_now[w] != 0ull) return item_entries_lat_prune<WARPS>(d, sh, S, it, gS);
-    return item_entries_lat<WARPS, MSHIFT, false>(d, sh, S, it, gS);
+// work item v of a launch: its walker, entries and first slot; false when it
+// is out of range
+__device__ __forceinline__ bool find_item(const Dev &d, const int *pre, int w0, int nw, int v, int &w, int4 &it, int &gS) {
+    int lo = 0, hi = nw - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (pre[mid] <= v) lo = mid; else hi = mid - 1;
+    }
+    w = w0 + lo;
+    const WalkerDev &W = d.walk[w];
+    it = d.items[W.item_base + (v - pre[lo])];
+    gS = W.slot_off + (it.x - W.sc_off) * SC;
+    return la_in(d, it.x - W.sc_off, W.sc_cap) && la_in(d, it.z - 1, d.ent_cap) && la_in(d, it.y, it.z);
+}
+
+// the last one out of `parts` resets the work counters for the next launch
+__device__ __forceinline__ void items_done(const Dev &d, bool arrives, unsigned long long parts) {
+    if (!arrives) return;
+    __threadfence();
+    if (atomicAdd(&d.counters[CTR_DONE], 1ull) == parts - 1ull) {
+        d.counters[CTR_ITEM] = 0ull;
+        d.counters[CTR_DONE] = 0ull;
+        __threadfence();
+    }
 }
 
 // work items of the normal pairs, handed out by a global counter
-template <bool ENERGY, int WARPS, int MSHIFT, class Shared>
-__device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int nblk, Shared &sh) {
+template <bool ENERGY, int WARPS, int MSHIFT>
+__device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int nblk, PairShared<WARPS> &sh) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nw = w1 - w0;
     const int total = sh.pre[nw];
@@ -519,24 +541,18 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int n
     for (;;) {
         const int v = __shfl_sync(FULL, v_next, 0);
         if (v >= total) break;
-        int lo = 0, hi = nw - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (sh.pre[mid] <= v) lo = mid; else hi = mid - 1;
-        }
-        const int w = w0 + lo;
-        const WalkerDev &W = d.walk[w];
-        const SysDev &S = d.sys[W.sys];
-        const int4 it = d.items[W.item_base + (v - sh.pre[lo])];
-        if (!la_in(d, it.x - W.sc_off, W.sc_cap) || !la_in(d, it.z - 1, d.ent_cap) || !la_in(d, it.y, it.z)) {  // item skipped
+        int w, gS;
+        int4 it;
+        if (!find_item(d, sh.pre, w0, nw, v, w, it, gS)) {  // item skipped
             if (lane == 0) v_next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
             continue;
         }
-        const int sc = it.x;
-        const int gS = W.slot_off + (sc - W.sc_off) * SC;
+        const SysDev &S = d.sys[d.walk[w].sys];
         __syncwarp();
-        stage_cluster(d, sh, wib, lane, gS + lane);
-        stage_cluster(d, sh, wib, lane + 32, gS + lane + 32);
+        sh.sxq[wib][lane] = d.xq[gS + lane];
+        sh.sxq[wib][lane + 32] = d.xq[gS + lane + 32];
+        sh.slj[wib][lane] = d.lj[gS + lane];
+        sh.slj[wib][lane + 32] = d.lj[gS + lane + 32];
         float elj = 0.f, erf = 0.f;
         int npair = 0;
         v_next = run_item<ENERGY, WARPS, MSHIFT>(d, sh, S, w, it, gS, elj, erf, npair);
@@ -554,16 +570,28 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int n
             }
         }
     }
-    // the last warp out resets the work counters for the next launch
-    if (lane == 0) {
-        __threadfence();
-        const unsigned long long done = atomicAdd(&d.counters[CTR_DONE], 1ull);
-        if (done == (unsigned long long)nblk * WARPS - 1ull) {
-            d.counters[CTR_ITEM] = 0ull;
-            d.counters[CTR_DONE] = 0ull;
-            __threadfence();
+    items_done(d, lane == 0, (unsigned long long)nblk * WARPS);
+}
+
+// the same with one item per block at a time (latency form)
+template <int MSHIFT>
+__device__ __forceinline__ void normal_items_lat(const Dev &d, int w0, int w1, int nblk, PairSharedLat &sh) {
+    const int nw = w1 - w0;
+    const int total = sh.pre[nw];
+    for (int v = sh.first; v < total;) {
+        int w, gS;
+        int4 it;
+        if (find_item(d, sh.pre, w0, nw, v, w, it, gS)) {
+            const SysDev &S = d.sys[d.walk[w].sys];
+            if (MSHIFT == 8 && d.prune_now[w] != 0ull) item_entries_lat<MSHIFT, true>(d, sh, S, it, gS);
+            else item_entries_lat<MSHIFT, false>(d, sh, S, it, gS);
         }
+        if (threadIdx.x == 0) sh.next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
+        __syncthreads();
+        v = sh.next;
+        __syncthreads();
     }
+    items_done(d, threadIdx.x == 0, (unsigned long long)nblk);
 }
 
 // Fused launch: a stage's lambda update (lambda_work) needs the partial sums
@@ -767,11 +795,14 @@ __device__ __forceinline__ void bonded_items(const Dev &d, int w0, int w1, int b
     }
 }
 
-// Items per SM up to which the latency form is taken.  Fused launch, common /
-// latency form: 0.4 items per SM (4 x 257 atoms) 33 / 19 us, 5 (8 x 772 atoms)
-// 43 / 32 us, 19 (2 x 9020 atoms) 47 / 48 us, 92 (144 x 772 atoms) 127 / 128 us,
-// 200 (16 x 12 300 atoms) 252 / 308 us.
+// Items per SM up to which the latency form is taken, and its blocks per SM
+// (42.6 KB of shared memory, 122 registers).  Fused launch, common / one warp
+// per item / latency form: 0.4 items per SM (4 x 257 atoms) 33 / 19 / 17 us, 5
+// (8 x 772 atoms) 43 / 32 / 32 us (there the alchemical warps' chain decides), 19
+// (2 x 9020 atoms) 43 / - / 43 us, 92 (144 x 772 atoms) 117 / - / 174 us, 200
+// (16 x 12 300 atoms) 242 / - / 366 us.
 constexpr int LAT_ITEMS_PER_SM = 8;
+constexpr int LAT_BLOCKS_PER_SM = 4;
 
 // WARPS x 32 threads per CTA; MINB: resident CTAs per SM the register
 // allocation is sized for.  Variants (autotuned): 8 warps / 3 CTAs (80
@@ -779,7 +810,7 @@ constexpr int LAT_ITEMS_PER_SM = 8;
 template <bool ENERGY, int WARPS, int MINB, int MODE, bool LAT>
 __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w1, int nblk_pairs, int a0, int a1,
                                                           int nblk_bonded, int alch_warps) {
-    __shared__ std::conditional_t<LAT, PairSharedLat<WARPS>, PairShared<WARPS>> sh;
+    __shared__ std::conditional_t<LAT, PairSharedLat, PairShared<WARPS>> sh;
     // grid: [alchemical items][bonded terms][normal pairs]; the first two come
     // first so that they run alongside the normal pairs.  (The alchemical
     // blocks return here: when their warps went on to the normal pairs, the
@@ -810,11 +841,12 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w
         }
         if (threadIdx.x == 0) {
             sh.pre[w1 - w0] = acc;
-            sh.first = (int)atomicAdd(&d.counters[CTR_ITEM], (unsigned long long)WARPS);
+            sh.first = (int)atomicAdd(&d.counters[CTR_ITEM], LAT ? 1ull : (unsigned long long)WARPS);
         }
     }
     __syncthreads();
-    normal_items<ENERGY, WARPS, MODE == STEP ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
+    if constexpr (LAT) normal_items_lat<MODE == STEP ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
+    else normal_items<ENERGY, WARPS, MODE == STEP ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
 }
 
 template <bool ENERGY, int WARPS, int MINB, int MODE, bool LAT>
@@ -823,7 +855,9 @@ static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cud
     {  // no more blocks than a quarter above the items need (the queue serves any number)
         long long items = 0;
         for (int w = w0; w < w1; ++w) items += hv.items[w];
-        const long long need = (items + items / 4 + WARPS - 1) / WARPS;
+        const int per = LAT ? 1 : WARPS;
+        const long long need = (items + items / 4 + per - 1) / per;
+        if (LAT) nblk = LAT_BLOCKS_PER_SM * hv.n_sm;
         nblk = need < nblk ? (int)need : nblk;
         nblk = nblk < 1 ? 1 : nblk;
     }
@@ -855,7 +889,7 @@ static bool few_items(const HostView &hv, int w0, int w1) {
 
 template <int MODE>
 static void launch_pairs_any(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {
-    if (hv.pair_variant == 0 && few_items(hv, w0, w1)) launch_pairs_v<false, 4, 4, MODE, true>(d, hv, w0, w1, s);
+    if (hv.pair_variant == 0 && few_items(hv, w0, w1)) launch_pairs_v<false, LAT_WARPS, LAT_BLOCKS_PER_SM, MODE, true>(d, hv, w0, w1, s);
     else if (hv.pair_variant == 1) launch_pairs_v<false, 4, 7, MODE, false>(d, hv, w0, w1, s);
     else if (hv.pair_variant == 2) launch_pairs_v<false, 4, 8, MODE, false>(d, hv, w0, w1, s);
     else launch_pairs_v<false, 8, 3, MODE, false>(d, hv, w0, w1, s);

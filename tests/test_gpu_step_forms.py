@@ -52,3 +52,23 @@ def test_stage_sizes(walkers, shared_freq, theta):
     run = synth.lj_fluid_run(seed=9, n_walkers=walkers, n_bins=7)
     run.shared_freq, run.theta_stats = shared_freq, theta
     run_both(synth.lj_fluid(seed=12), run, 11)
+
+
+@pytest.mark.parametrize("chunk, margin", [(32, 0.05), (64, 0.0), (96, 0.05)])
+def test_latency_form_items(chunk, margin):
+    """The latency form (variant 0, few items) against the common form
+    (variant 1 takes it at any size), items of one to three 32-entry passes."""
+    from paper_2307_08006_gb300 import labf
+
+    spec, out = water(17), []
+    run = synth.water_run(seed=8, walkers_per_stage=1, n_bins=8)
+    run.stages = [synth.Stage(0.0, 1.0, 8, 3)]
+    state = synth.initial_state(spec, run, lam0=[0.1, 0.5, 0.9])
+    for variant in (0, 1):
+        eng = labf.engine_for(spec, run, state, options=dict(prune_margin=margin, chunk_entries=chunk,
+                                                             pair_variant=variant))
+        eng.step(23)
+        out.append(eng.get_states())
+        eng.close()
+    for k in ("x", "v", "lam", "plam"):
+        assert np.array_equal(out[0][k], out[1][k]), k
