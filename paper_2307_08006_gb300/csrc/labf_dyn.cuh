@@ -476,8 +476,10 @@ __device__ __forceinline__ void lambda_work(const Dev &d, int si, int prime, int
                     }
                 }
             }
+            // the next 32 walkers' leaders, and the merge below, read what these
+            // lanes stored (shuffles and votes do not order memory)
+            __syncwarp();
         }
-        __syncwarp();
         if (K > 1 && (d.step[w0] + 1ull) % (unsigned long long)K == 0ull) {
             for (int q = lane; q < st.n_bins; q += 32) {
                 double s1 = d.abf_sum[st.bin_off + q], s2 = d.abf_sumsq[st.bin_off + q];

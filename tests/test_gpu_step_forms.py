@@ -72,3 +72,27 @@ def test_latency_form_items(chunk, margin):
         eng.close()
     for k in ("x", "v", "lam", "plam"):
         assert np.array_equal(out[0][k], out[1][k]), k
+
+
+@pytest.mark.parametrize("walkers, n_bins", [(32, 3), (33, 1), (65, 3), (100, 2)])
+def test_fold_of_large_stages(walkers, n_bins):
+    """One step of a stage that merges every step, its walkers' lambdas in no
+    order, so that a bin's first walker sits in another lane in each group of
+    32: the shared statistics are the walkers' samples added in walker order."""
+    from paper_2307_08006_gb300 import labf
+
+    spec, run = synth.lj_fluid(seed=12), synth.lj_fluid_run(seed=9, n_walkers=walkers, n_bins=n_bins)
+    run.shared_freq = 1
+    lam0 = np.random.default_rng(walkers).uniform(0.05, 0.95, walkers)
+    eng = labf.engine_for(spec, run, synth.initial_state(spec, run, lam0=list(lam0)))
+    eng.step(1)
+    got, lam = eng.read_abf(0, 0), eng.get_states()["lam"]
+    ref = np.zeros((3, n_bins))
+    st = run.stages[0]
+    for w in range(walkers):
+        k = min(max(int(np.floor((lam[w] - st.lo) / ((st.hi - st.lo) / n_bins))), 0), n_bins - 1)
+        s = eng.energy_forces(w)["dUdl"]
+        ref[:, k] += (s, s * s, 1.0)
+    eng.close()
+    assert np.array_equal(got["sum"], ref[0]) and np.array_equal(got["sumsq"], ref[1])
+    assert np.array_equal(got["count"], ref[2])
