@@ -497,7 +497,8 @@ int la_destroy(la_handle *h);
  * outside [0, n_atoms) or not flagged alchemical: that atom is skipped),
  * LA_STATUS_NONFINITE (a non-finite distance or force: the pair is
  * skipped), LA_STATUS_FIXED_OVERFLOW (a force component of 2^30 or more,
- * beyond the fixed-point accumulators: skipped).  Any non-zero status
+ * of a pair or of an atom's whole force, beyond the fixed-point accumulators:
+ * skipped).  Any non-zero status
  * means the other outputs are incomplete.
  *
  * Scratch: one file-scope static device array of 7 * 32 64-bit partial sums

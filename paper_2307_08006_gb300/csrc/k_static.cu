@@ -90,9 +90,12 @@ __device__ __forceinline__ StaticAlch load_alch(const StaticParams &p, const Sta
     return A;
 }
 
-// a force component that fits the 64-bit fixed-point range, else a status bit
-__device__ __forceinline__ bool static_force_ok(float fx, float fy, float fz, unsigned *status) {
-    const float m = fmaxf(fabsf(fx), fmaxf(fabsf(fy), fabsf(fz)));
+// largest magnitude of a force's components
+__device__ __forceinline__ float static_top(float fx, float fy, float fz) {
+    return fmaxf(fabsf(fx), fmaxf(fabsf(fy), fabsf(fz)));
+}
+// a force that fits the 64-bit fixed-point range, else a status bit
+__device__ __forceinline__ bool static_force_ok(float m, unsigned *status) {
     if (m < FIX_LIMIT) return true;
     atomicOr(status, m == m ? LA_STATUS_FIXED_OVERFLOW : LA_STATUS_NONFINITE);
     return false;
@@ -107,8 +110,22 @@ __device__ __forceinline__ float static_image(float dx, float L, float Linv) {
     return dx - L * (fmaf(dx, Linv, M) - M);
 }
 
+constexpr int ST_THREADS = 128, ST_WARPS = ST_THREADS / 32;
+constexpr int ST_TILE = 64;  // alchemical atoms staged at a time
+
+// Range of an atom's whole force.  Sums of fixed-point forces may wrap: modulo
+// 2^64 they are exact whenever the whole force is in range, whatever the parts
+// are.  Whether it is in range is asked only of atoms with a part so large that
+// their number could carry the sum out of range (BIG_PAIR: at most
+// LA_STATIC_MAX_ALCH pairs; BIG_SHARE: warps of a group), and answered by
+// adding the pairs once more in FP32.  An environment atom is asked about by its
+// own thread, for its force, and by the groups that meet its big pairs, for the
+// status: they are through before the status is read (arrivals of the
+// environment blocks took 3% of the largest shapes' time).
+constexpr float BIG_PAIR = FIX_LIMIT / LA_STATIC_MAX_ALCH, BIG_SHARE = FIX_LIMIT / (LA_STATIC_CHUNKS * ST_WARPS);
+
 struct StaticPair {
-    float fs, dx, dy, dz, dsc, rf_u, usc;
+    float fs, dx, dy, dz, top, dsc, rf_u, usc;
 };
 
 // the pair (A, environment atom b at xb..zb); false when out of reach or skipped
@@ -143,11 +160,57 @@ __device__ __forceinline__ bool static_pair(const StaticParams &p, const StaticI
         o.dsc = p.dlvn * e4 * g + p.lvn * e4 * g1 * p.dsdl;
     }
     o.fs = sc_f + p.le * rf_f;
-    return static_force_ok(o.fs * o.dx, o.fs * o.dy, o.fs * o.dz, status);
+    o.top = static_top(o.fs * o.dx, o.fs * o.dy, o.fs * o.dz);
+    return static_force_ok(o.top, status);
 }
 
-constexpr int ST_THREADS = 128, ST_WARPS = ST_THREADS / 32;
-constexpr int ST_TILE = 64;  // alchemical atoms staged at a time
+// f 2^32 modulo 2^64 (f2fix clamps at 2^31; a warp's share may be 2^40)
+__device__ __forceinline__ unsigned long long f2fix_wrap(float f) {
+    return fabsf(f) < FIX_LIMIT ? f2fix(f) : (unsigned long long)(long long)f << 32;
+}
+
+// the whole force on environment atom b, by its thread
+__device__ __noinline__ bool env_force_ok(const StaticParams &p, const StaticIn &in, int b, float xb, float yb, float zb,
+                                          int gb, unsigned *status) {
+    float f[3] = {0.f, 0.f, 0.f};
+    for (int r = 0; r < p.n_alch; ++r) {
+        StaticPair o;
+        if (!static_pair(p, in, load_alch(p, in, r, status), b, xb, yb, zb, gb, status, o)) continue;
+        f[0] = fmaf(-o.fs, o.dx, f[0]);
+        f[1] = fmaf(-o.fs, o.dy, f[1]);
+        f[2] = fmaf(-o.fs, o.dz, f[2]);
+    }
+    return static_force_ok(static_top(f[0], f[1], f[2]), status);
+}
+
+// the whole force on alchemical atom A, by the block; also those on the
+// environment atoms of A's big pairs
+__device__ __noinline__ bool alch_force_ok(const StaticParams &p, const StaticIn &in, const StaticAlch &A,
+                                           float (&share)[ST_WARPS][3], unsigned *status) {
+    float f[3] = {0.f, 0.f, 0.f};
+    for (int b = threadIdx.x; b < p.n; b += ST_THREADS) {
+        StaticPair o;
+        if (in.alch[b] || !static_pair(p, in, A, b, in.x[3 * (size_t)b], in.x[3 * (size_t)b + 1], in.x[3 * (size_t)b + 2],
+                                       in.grp[b], status, o))
+            continue;
+        f[0] = fmaf(o.fs, o.dx, f[0]);
+        f[1] = fmaf(o.fs, o.dy, f[1]);
+        f[2] = fmaf(o.fs, o.dz, f[2]);
+        if (!(o.top < BIG_PAIR))
+            env_force_ok(p, in, b, in.x[3 * (size_t)b], in.x[3 * (size_t)b + 1], in.x[3 * (size_t)b + 2], in.grp[b], status);
+    }
+    __syncthreads();  // share free
+    for (int c = 0; c < 3; ++c) {
+        const float v = warp_sumf(f[c]);
+        if ((threadIdx.x & 31) == 0) share[threadIdx.x >> 5][c] = v;
+    }
+    __syncthreads();
+    for (int c = 0; c < 3; ++c) {
+        f[c] = 0.f;
+        for (int q = 0; q < ST_WARPS; ++q) f[c] += share[q][c];
+    }
+    return static_force_ok(static_top(f[0], f[1], f[2]), status);
+}
 
 // sum over the warp, on every lane
 __device__ __forceinline__ double static_sum(double v, bool any) { return any ? warp_sum(v) : 0.0; }
@@ -155,12 +218,14 @@ __device__ __forceinline__ double static_sum(double v, bool any) { return any ? 
 // RA: alchemical atoms per alchemical block (4 once the grid is full: their
 // atoms' loads are shared)
 template <int RA>
-__global__ void __launch_bounds__(ST_THREADS) k_static(StaticParams p, StaticIn in, int n_env_blocks, int chunks,
-                                                       unsigned long long *part, double *sums, unsigned *status,
+__global__ void __launch_bounds__(ST_THREADS) k_static(const __grid_constant__ StaticParams p,
+                                                       const __grid_constant__ StaticIn in, int n_env_blocks,
+                                                       int chunks, unsigned long long *part, double *sums, unsigned *status,
                                                        double dlv, double dle, float *forces, double *out) {
     __shared__ StaticAlch tile[ST_TILE];
     __shared__ double wsum[ST_WARPS][RA][4];
-    __shared__ long long wfix[ST_WARPS][RA][3];
+    __shared__ unsigned long long wfix[ST_WARPS][RA][3];
+    __shared__ float wforce[ST_WARPS][3];
     __shared__ int last;
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     if ((int)blockIdx.x < n_env_blocks) {
@@ -176,6 +241,7 @@ __global__ void __launch_bounds__(ST_THREADS) k_static(StaticParams p, StaticIn 
             gb = in.grp[b];
         }
         unsigned long long f[3] = {0ull, 0ull, 0ull};
+        float top = 0.f;
         bool listed = false;  // an alchemical atom whose group writes its force
         for (int r0 = 0; r0 < p.n_alch; r0 += ST_TILE) {
             __syncthreads();
@@ -190,11 +256,13 @@ __global__ void __launch_bounds__(ST_THREADS) k_static(StaticParams p, StaticIn 
                     f[0] += f2fix(-o.fs * o.dx);
                     f[1] += f2fix(-o.fs * o.dy);
                     f[2] += f2fix(-o.fs * o.dz);
+                    top = fmaxf(top, o.top);
                 }
             }
         }
+        const bool ok = top < BIG_PAIR || env_force_ok(p, in, b, xb, yb, zb, gb, status);
         if (on && !listed)
-            for (int c = 0; c < 3; ++c) forces[3 * (size_t)b + c] = fix_to_float(f[c]);
+            for (int c = 0; c < 3; ++c) forces[3 * (size_t)b + c] = ok ? fix_to_float(f[c]) : 0.f;
         return;
     }
     {
@@ -206,6 +274,7 @@ __global__ void __launch_bounds__(ST_THREADS) k_static(StaticParams p, StaticIn 
         double s[RA][4] = {};
         float fa[RA][3] = {};
         unsigned hit = 0;
+        float top = 0.f;
         for (int b = b0 + tid; b < b1; b += ST_THREADS) {
             if (in.alch[b]) continue;
             const float xb = in.x[3 * (size_t)b], yb = in.x[3 * (size_t)b + 1], zb = in.x[3 * (size_t)b + 2];
@@ -215,6 +284,7 @@ __global__ void __launch_bounds__(ST_THREADS) k_static(StaticParams p, StaticIn 
                 StaticPair o;
                 if (r0 + r >= p.n_alch || !static_pair(p, in, tile[r], b, xb, yb, zb, gb, status, o)) continue;
                 hit |= 1u << r;
+                top = fmaxf(top, o.top);
                 fa[r][0] = fmaf(o.fs, o.dx, fa[r][0]);
                 fa[r][1] = fmaf(o.fs, o.dy, fa[r][1]);
                 fa[r][2] = fmaf(o.fs, o.dz, fa[r][2]);
@@ -224,6 +294,7 @@ __global__ void __launch_bounds__(ST_THREADS) k_static(StaticParams p, StaticIn 
                 s[r][3] += (double)(p.le * o.rf_u);
             }
         }
+        bool big = !(top < BIG_PAIR);
         hit = __reduce_or_sync(0xffffffffu, hit);
 #pragma unroll
         for (int r = 0; r < RA; ++r) {
@@ -236,10 +307,10 @@ __global__ void __launch_bounds__(ST_THREADS) k_static(StaticParams p, StaticIn 
             float f[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) f[c] = any ? warp_sumf(fa[r][c]) : 0.f;
+            big = big || !(static_top(f[0], f[1], f[2]) < BIG_SHARE);
             if (lane == 0) {
-                const bool ok = static_force_ok(f[0], f[1], f[2], status);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) wfix[wib][r][c] = ok ? (long long)f2fix(f[c]) : 0ll;
+                for (int c = 0; c < 3; ++c) wfix[wib][r][c] = f2fix_wrap(f[c]);
             }
         }
         __syncthreads();
@@ -251,44 +322,53 @@ __global__ void __launch_bounds__(ST_THREADS) k_static(StaticParams p, StaticIn 
                 for (int q = 0; q < ST_WARPS; ++q) v += wsum[q][r][c];
                 *o = (unsigned long long)__double_as_longlong(v);
             } else {
-                long long v = 0;
+                unsigned long long v = 0ull;
                 for (int q = 0; q < ST_WARPS; ++q) v += wfix[q][r][c - 4];
-                *o = (unsigned long long)v;
+                *o = v;
             }
         }
-    }
-    // ---- the group's last block adds its chunks (lane = chunk) ----
-    const int group = (blockIdx.x - n_env_blocks) / chunks, r0 = group * RA;
-    unsigned *groups_done = status + 1, *chunks_done = status + 2;
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(&chunks_done[group], 1u) == (unsigned)chunks - 1u;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int r = r0 + wib; r < min(p.n_alch, r0 + RA); r += ST_WARPS) {
-        const unsigned long long *o = part + 7ull * ((size_t)r * chunks + lane);
-        unsigned long long v[7];
-#pragma unroll
-        for (int c = 0; c < 7; ++c) v[c] = lane < chunks ? __ldcg(o + c) : 0ull;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const double t = warp_sum(__longlong_as_double((long long)v[c]));
-            if (lane == 0) sums[4 * (size_t)r + c] = t;
+        // ---- the group's last block adds its chunks (lane = chunk) ----
+        unsigned *chunks_done = status + 2;
+        __threadfence();
+        const unsigned add = __syncthreads_or(big) ? 0x10001u : 1u;
+        if (tid == 0) {  // finished chunks, those with a big pair or share from bit 16 on
+            const unsigned done = atomicAdd(&chunks_done[r0 / RA], add) + add;
+            last = (done & 0xffffu) == (unsigned)chunks ? 1 + (int)(done >> 16) : 0;
         }
-#pragma unroll
-        for (int c = 4; c < 7; ++c) {
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) v[c] += __shfl_xor_sync(0xffffffffu, v[c], d);
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        unsigned bad = 0;  // atoms of the group out of range
+        if (last > 1) {
+#pragma unroll 1
+            for (int r = 0; r < RA && r0 + r < p.n_alch; ++r)
+                if (!alch_force_ok(p, in, tile[r], wforce, status)) bad |= 1u << r;
         }
-        const int a = in.alch_idx[r];
-        if (lane < 3 && (unsigned)a < (unsigned)p.n && in.alch[a])
-            forces[3 * (size_t)a + lane] = fix_to_float(lane == 0 ? v[4] : (lane == 1 ? v[5] : v[6]));
+        for (int r = r0 + wib; r < min(p.n_alch, r0 + RA); r += ST_WARPS) {
+            const unsigned long long *o = part + 7ull * ((size_t)r * chunks + lane);
+            unsigned long long v[7];
+#pragma unroll
+            for (int c = 0; c < 7; ++c) v[c] = lane < chunks ? __ldcg(o + c) : 0ull;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const double t = warp_sum(__longlong_as_double((long long)v[c]));
+                if (lane == 0) sums[4 * (size_t)r + c] = t;
+            }
+#pragma unroll
+            for (int c = 4; c < 7; ++c) {
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) v[c] += __shfl_xor_sync(0xffffffffu, v[c], d);
+            }
+            const int a = in.alch_idx[r];
+            if (lane < 3 && (unsigned)a < (unsigned)p.n && in.alch[a])
+                forces[3 * (size_t)a + lane] =
+                    (bad >> (r - r0)) & 1u ? 0.f : fix_to_float(lane == 0 ? v[4] : (lane == 1 ? v[5] : v[6]));
+        }
     }
     // ---- the last group adds the alchemical atoms ----
     __threadfence();
     __syncthreads();
-    if (tid == 0) last = atomicAdd(groups_done, 1u) == (gridDim.x - n_env_blocks) / chunks - 1u;
+    if (tid == 0) last = atomicAdd(status + 1, 1u) == (gridDim.x - n_env_blocks) / chunks - 1u;
     __syncthreads();
     if (!last) return;
     __threadfence();

@@ -194,3 +194,55 @@ def test_static_entry_sizes_match_engine(n_waters, n_alch):
     assert o[3] == pytest.approx(ref["terms"][2], rel=TOL, abs=TOL)
     assert o[4] == pytest.approx(ref["terms"][3], rel=TOL, abs=TOL * scale)
     assert np.sqrt(((f - (fref - f0)) ** 2).sum() / max((fref ** 2).sum(), 1e-30)) < TOL
+
+
+@pytest.mark.parametrize("n_alch", [2, 200])  # one and four alchemical atoms per block
+@pytest.mark.parametrize("left, right, second, overflow", [
+    ((5,), (), False, False),                 # one pair: in range
+    ((5, 205), (), False, True),              # pairs in range, their sum is not: two chunks
+    ((5, 205, 405, 605), (), False, True),    # ... nor is it in the range of the 64-bit sums
+    ((5, 40), (), False, True),               # two warps of a chunk
+    ((5, 6), (), False, True),                # one warp
+    ((5, 6), (7, 8), False, False),           # a warp's sum in range, its lanes' are not
+    ((5, 205), (405, 605), False, False),     # the total in range, no chunk's share of it far below
+    ((5, 6, 205, 206), (405, 406, 605, 606), False, False),
+    ((5,), (), True, True),                   # an environment atom between two alchemical ones
+])
+def test_static_entry_force_range(n_alch, left, right, second, overflow):
+    """LA_STATUS_FIXED_OVERFLOW is about an atom's whole force, of alchemical
+    and environment atoms alike: 2^30 or more is reported, a sum that is in
+    range is returned whatever its parts are.  Reaction-field pairs of 0.6 x
+    2^30 along x; values by the formula, FP32 tolerance."""
+    import torch
+
+    n, box, rc, r = 1000, 8.0, 1.0, 0.5
+    krf = 1.0 / (2.0 * rc ** 3)
+    pull = 0.6 * 2.0 ** 30
+    qq = pull / ((1.0 / r ** 3 - 2.0 * krf) * r)
+    x = np.full((n, 3), 0.5, np.float32)  # everything else: far away, no charge
+    q, alch = np.zeros(n), np.zeros(n, np.uint8)
+    alch[n - n_alch:] = 1
+    x[n - n_alch:] = 2.0
+    a, a2 = n - n_alch, n - n_alch + 1
+    x[a] = 4.0
+    q[a] = np.sqrt(qq)
+    for side, atoms in ((-r, left), (r, right)):
+        for b in atoms:
+            x[b] = 4.0
+            x[b, 0] = 4.0 + side
+            q[b] = np.sqrt(qq)
+    if second:  # pulls its environment atom the same way as the first
+        x[a2], q[a2] = x[a], q[a]
+    t = lambda v, dt: torch.tensor(np.ascontiguousarray(v), dtype=dt, device="cuda")
+    f32, i32 = torch.float32, torch.int32
+    forces, out = labf.alch_pairs_static(
+        t(x, f32), t(q, f32), t(np.zeros(n), f32), t(np.zeros(n), f32), t(alch, torch.uint8),
+        t(np.full(n, -1), i32), t(np.nonzero(alch)[0], i32), box, rc, 0.0, 1.0, 1.0, 0.5, 0.5)
+    f, status = forces.cpu().numpy(), int(out[5].item())
+    assert status == (0x4 if overflow else 0)
+    if not overflow:
+        assert f[a, 0] == pytest.approx(pull * (len(left) - len(right)), abs=TOL * pull)
+        for sign, atoms in ((-1.0, left), (1.0, right)):
+            for b in atoms:
+                assert f[b, 0] == pytest.approx(sign * pull, rel=TOL)
+        assert np.abs(f[:, 1:]).max() == 0.0
