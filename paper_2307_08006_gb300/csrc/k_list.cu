@@ -321,13 +321,14 @@ static_assert(LB_COLS == 4 * LB_WARPS && LB_VCAP == 2 * LB_THREADS && 3 * (MAX_C
 // more; the last one resets both for the next launch
 constexpr int CTR_LB_ITEM = 8, CTR_LB_DONE = 9;
 
-// Staged codes: exclusion group (bits 0-29; "no group" differs on the two
-// sides, so one compare decides the group test) | EXTRA_FLAG when the slot
-// has extra excluded partners.  Slots without normal pairs (padding,
+// Staged codes: exclusion group (bits 0-29, ids below MAX_GROUPS; "no group"
+// differs on the two sides, so one compare decides the group test) |
+// EXTRA_FLAG when the slot has extra excluded partners.  Slots without normal pairs (padding,
 // alchemical) sit at FAR on the i side and -FAR on the j side, out of every
 // list radius.
 constexpr int GROUP_MASK = 0x3fffffff, EXTRA_FLAG = 0x40000000;
 constexpr int NO_GROUP_I = 0x3fffffff, NO_GROUP_J = 0x3ffffffe;
+static_assert(MAX_GROUPS == NO_GROUP_J && NO_GROUP_I == GROUP_MASK, "group ids and codes");
 constexpr float FAR = 536870912.0f;  // 2^29
 
 // exclusive scan over the block (v per thread); every thread gets the total

@@ -13,6 +13,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "labf_internal.cuh"
@@ -907,12 +908,17 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
         D.w_count = sl.W;
         h->sys.push_back(D);
         const double sqc = std::sqrt(std::max(0.0, S.coul));
+        // group ids are compared only: those beyond the list kernel's codes are
+        // replaced by the numbers of their first appearances
+        const bool renumber = *std::max_element(S.excl_group, S.excl_group + S.n_atoms) >= MAX_GROUPS;
+        std::unordered_map<int, int> group_no;
         for (int i = 0; i < S.n_atoms; ++i) {
             ap[atom_off + i] = make_float4((float)(S.charge[i] * sqc), (float)(0.5 * S.sigma[i]),
                                            (float)(2.0 * std::sqrt(std::max(0.0, S.epsilon[i]))),
                                            (float)(1.0 / S.mass[i]));
             an[atom_off + i] = (float)std::sqrt(S.kT / S.mass[i]);
-            ag[atom_off + i] = S.excl_group[i];
+            const int group = S.excl_group[i];
+            ag[atom_off + i] = group < 0 || !renumber ? group : group_no.emplace(group, (int)group_no.size()).first->second;
             ax[atom_off + i] = make_int4(S.excl_extra[4 * i], S.excl_extra[4 * i + 1], S.excl_extra[4 * i + 2],
                                          S.excl_extra[4 * i + 3]);
             aa[atom_off + i] = S.alch[i] ? 1 : 0;

@@ -31,6 +31,7 @@ constexpr int JC = 4;            // slots per j-cluster
 constexpr int NIC = SC / IC;     // i-clusters per super-cluster
 constexpr int NJC = SC / JC;     // j-clusters per super-cluster
 constexpr int MAX_COL = 2048;    // atoms per column (sort kernel capacity)
+constexpr int MAX_GROUPS = 0x3ffffffe;  // exclusion group ids of the list kernel's slot codes: below this
 constexpr int N_ETERMS = 8;      // LA_N_TERMS + spare
 constexpr float FIX_TO_F = 2.3283064365386963e-10f;  // 2^-32
 constexpr float F_TO_FIX = 4294967296.0f;            // 2^32

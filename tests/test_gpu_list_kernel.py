@@ -56,3 +56,26 @@ def test_pair_lists_match_oracle(n, r_cut, box, n_alch):
         got, gkind = eng.get_pairs(w)
         assert np.array_equal(got, ref) and np.array_equal(gkind, kind)
     eng.close()
+
+
+def test_exclusion_group_ids_of_any_size():
+    """Groups are told apart by their whole 32-bit id: ids that differ only
+    above bit 29, and the largest ones, exclude their own atoms and no others."""
+    import oracle
+    from paper_2307_08006_gb300 import labf
+
+    spec = random_spec(1000, 0.9, 2.0, 77, 6)
+    ids = np.arange(spec.n, dtype=np.int64)
+    ids[:40] = (0x3ffffffe, 0x3fffffff, 0x40000000, 0x7ffffffe, 0x7fffffff, *(0x40000000 + 300 + np.arange(35)))
+    g = np.asarray(spec.excl_group)
+    # (low ids that the large ones must not be taken for stay in use)
+    order = np.unique(g[g >= 0])
+    new = dict(zip(order, [*ids[:40], *range(300, 300 + len(order) - 40)]))
+    spec.excl_group = np.array([new.get(k, -1) for k in g], np.int64).astype(np.int32)
+    run = synth.harmonic_run(seed=5, n_walkers=1, n_bins=4)
+    run.skin = 0.09
+    eng = labf.engine_for(spec, run, options=dict(list_capacity_factor=4.0))
+    ref, kind = oracle.pair_set(oracle.OracleSystem(spec), spec.x, spec.r_cut + run.skin)
+    got, gkind = eng.get_pairs(0)
+    assert np.array_equal(got, ref) and np.array_equal(gkind, kind)
+    eng.close()
