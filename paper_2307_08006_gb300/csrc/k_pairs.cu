@@ -22,7 +22,10 @@
 // to the fixed-point array after every 32 entries of a super-cluster's list,
 // so every kernel variant and work-item size (a multiple of 32 entries)
 // produces the same bits.  A lane whose pair is out of the cutoff skips its
-// six accumulating instructions by predicate (no select to zero per tile).
+// six accumulating instructions by predicate (no select to zero per tile).  An
+// evaluation multiplies by zero instead: a distance that is not a number then
+// reaches the forces and is reported (an MD step's integrator tests the
+// positions themselves).
 // All float-to-fixed conversions use integer instructions: the hardware
 // conversion to 64-bit integers runs on the FP64 pipe, which is narrow on this
 // GPU.  Fused launch before / after the lane map, the staging and the
@@ -255,8 +258,9 @@ __device__ __forceinline__ int item_entries(const Dev &d, PairShared<WARPS> &sh,
                     const float e4s6 = li.y * lj_j.y * sr6;
                     const float qq = xi.w * xj.w;
                     const float b = fmaf(qq, rinv, e4s6 * fmaf(12.f, sr6, -6.f));
-                    const float fs = fmaf(b, r2inv, -qq * krf2);
-                    if (in) {  // predicated
+                    float fs = fmaf(b, r2inv, -qq * krf2);
+                    if (ENERGY) fs = in ? fs : 0.f;
+                    if (ENERGY || in) {  // predicated
                         fi[ic][0] = fmaf(fs, dx, fi[ic][0]);
                         fi[ic][1] = fmaf(fs, dy, fi[ic][1]);
                         fi[ic][2] = fmaf(fs, dz, fi[ic][2]);

@@ -401,3 +401,27 @@ def test_nonfinite_state_is_reported():
     assert ei.value.code in (-7, -8, -9)
     with pytest.raises(labf.LabfError):
         eng.step(1)  # sticky
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("device", [False, True])
+def test_nonfinite_position_in_an_evaluation(bad, device):
+    """A single evaluation at a position that is not a number has no forces to
+    give: it ends in an error, also for an atom with pair forces only (far from
+    the alchemical atom)."""
+    import torch
+
+    sp = synth.lj_fluid(seed=12, cells=7)
+    eng = labf.engine_for(sp, synth.lj_fluid_run(seed=9, n_walkers=1, n_bins=4))
+    x = eng.get_state(0)["x"].copy()
+    x[77, 2] = bad
+    with pytest.raises(labf.LabfError) as ei:
+        if device:
+            forces = torch.empty((sp.n, 3), dtype=torch.float32, device="cuda")
+            eng.energy_forces_device(0, x=torch.as_tensor(x, device="cuda"), forces=forces)
+            eng.sync()
+        else:
+            eng.set_state(0, x=x)
+            eng.energy_forces(0)
+    assert ei.value.code in (-7, -8)
+    eng.close()
