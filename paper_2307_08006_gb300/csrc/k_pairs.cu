@@ -85,7 +85,7 @@ struct PairSharedLat {
     unsigned char lb[EPC][32];
     float2 f[EPC][NIC / 2][32];
     unsigned char keep[EPC][NIC / 2];
-    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], first, next;
+    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], next;
 };
 constexpr int LAT_WARPS = NIC / 2;
 
@@ -580,12 +580,14 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int n
     items_done(d, lane == 0, (unsigned long long)nblk * WARPS);
 }
 
-// the same with one item per block at a time (latency form)
+// the same with one item per block at a time (latency form); block blk starts
+// with item blk, and those without a first item have no part in the queue
 template <int MSHIFT>
-__device__ __forceinline__ void normal_items_lat(const Dev &d, int w0, int w1, int nblk, PairSharedLat &sh) {
+__device__ __forceinline__ void normal_items_lat(const Dev &d, int w0, int w1, int blk, int nblk, PairSharedLat &sh) {
     const int nw = w1 - w0;
     const int total = sh.pre[nw];
-    for (int v = sh.first; v < total;) {
+    if (blk >= total) return;
+    for (int v = blk; v < total;) {
         int w, gS;
         int4 it;
         if (find_item(d, sh.pre, w0, nw, v, w, it, gS)) {
@@ -593,12 +595,12 @@ __device__ __forceinline__ void normal_items_lat(const Dev &d, int w0, int w1, i
             if (MSHIFT == 8 && d.prune_now[w] != 0ull) item_entries_lat<MSHIFT, true>(d, sh, S, it, gS);
             else item_entries_lat<MSHIFT, false>(d, sh, S, it, gS);
         }
-        if (threadIdx.x == 0) sh.next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
+        if (threadIdx.x == 0) sh.next = nblk + (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
         __syncthreads();
         v = sh.next;
         __syncthreads();
     }
-    items_done(d, threadIdx.x == 0, (unsigned long long)nblk);
+    items_done(d, threadIdx.x == 0, (unsigned long long)min(nblk, total));
 }
 
 // Fused launch: a stage's lambda update (lambda_work) needs the partial sums
@@ -848,26 +850,20 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w
         }
         if (threadIdx.x == 0) {
             sh.pre[w1 - w0] = acc;
-            sh.first = (int)atomicAdd(&d.counters[CTR_ITEM], LAT ? 1ull : (unsigned long long)WARPS);
+            if constexpr (!LAT) sh.first = (int)atomicAdd(&d.counters[CTR_ITEM], (unsigned long long)WARPS);
         }
     }
     __syncthreads();
-    if constexpr (LAT) normal_items_lat<MODE == STEP ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
+    if constexpr (LAT) normal_items_lat<MODE == STEP ? 8 : 16>(d, w0, w1, blockIdx.x - nblk_alch - nblk_bonded, nblk_pairs, sh);
     else normal_items<ENERGY, WARPS, MODE == STEP ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
 }
 
 template <bool ENERGY, int WARPS, int MINB, int MODE, bool LAT>
 static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {
-    int nblk = hv.pair_blocks * 8 / WARPS;  // pair_blocks counts 8-warp CTAs
-    {  // no more blocks than a quarter above the items need (the queue serves any number)
-        long long items = 0;
-        for (int w = w0; w < w1; ++w) items += hv.items[w];
-        const int per = LAT ? 1 : WARPS;
-        const long long need = (items + items / 4 + per - 1) / per;
-        if (LAT) nblk = LAT_BLOCKS_PER_SM * hv.n_sm;
-        nblk = need < nblk ? (int)need : nblk;
-        nblk = nblk < 1 ? 1 : nblk;
-    }
+    // (pair_blocks counts 8-warp CTAs.)  The grid does not depend on the number of
+    // items: the queue serves any number, and the lists may grow while a graph
+    // that holds the launch is replayed.
+    const int nblk = LAT ? LAT_BLOCKS_PER_SM * hv.n_sm : hv.pair_blocks * 8 / WARPS;
     const int a0 = hv.alch_base[w0], a1 = hv.alch_base[w1 - 1] + hv.n_alch[w1 - 1];
     // alchemical warps per block: one, or as few as keep the blocks at one per
     // SM.  They live on FP64 sums, and an SM's FP64 pipe does 1.9 lanes per
@@ -887,28 +883,29 @@ static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cud
     k_pairs<ENERGY, WARPS, MINB, MODE, LAT><<<grid, WARPS * 32, 0, s>>>(d, w0, w1, nblk, a0, a1, bblk, awarps);
 }
 
-// launches whose items leave an SM few enough of them take the latency form
-static bool few_items(const HostView &hv, int w0, int w1) {
+// launches whose items leave an SM few enough of them take the latency form.
+// The counts are those of the list builds that are through when the launch is
+// enqueued; both forms take any number.
+bool pairs_latency(const HostView &hv, int w0, int w1) {
     long long n = 0;
     for (int w = w0; w < w1; ++w) n += hv.items[w];
-    return n <= (long long)LAT_ITEMS_PER_SM * hv.n_sm;
+    return hv.pair_variant == 0 && n <= (long long)LAT_ITEMS_PER_SM * hv.n_sm;
 }
 
 template <int MODE>
-static void launch_pairs_any(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {
-    if (hv.pair_variant == 0 && few_items(hv, w0, w1)) launch_pairs_v<false, LAT_WARPS, LAT_BLOCKS_PER_SM, MODE, true>(d, hv, w0, w1, s);
+static void launch_pairs_any(const Dev &d, const HostView &hv, int w0, int w1, bool latency, cudaStream_t s) {
+    if (latency) launch_pairs_v<false, LAT_WARPS, LAT_BLOCKS_PER_SM, MODE, true>(d, hv, w0, w1, s);
     else if (hv.pair_variant == 1) launch_pairs_v<false, 4, 7, MODE, false>(d, hv, w0, w1, s);
     else if (hv.pair_variant == 2) launch_pairs_v<false, 4, 8, MODE, false>(d, hv, w0, w1, s);
     else launch_pairs_v<false, 8, 3, MODE, false>(d, hv, w0, w1, s);
 }
 
-void launch_pairs_fused(const Dev &d, const HostView &hv, int n_stages, cudaStream_t s) {
-    (void)n_stages;
-    launch_pairs_any<STEP>(d, hv, 0, hv.n_walkers, s);
+void launch_pairs_fused(const Dev &d, const HostView &hv, bool latency, cudaStream_t s) {
+    launch_pairs_any<STEP>(d, hv, 0, hv.n_walkers, latency, s);
 }
 
 void launch_pairs(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s) {
-    launch_pairs_any<PAIRS>(d, hv, w0, w1, s);
+    launch_pairs_any<PAIRS>(d, hv, w0, w1, pairs_latency(hv, w0, w1), s);
 }
 
 void launch_pairs_energy(const Dev &d, const HostView &hv, int w, cudaStream_t s) {

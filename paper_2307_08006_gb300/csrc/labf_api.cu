@@ -343,7 +343,7 @@ struct la_handle {
     std::vector<SysDev> sys;
     std::vector<WalkerDev> walk;
     std::vector<StageDev> stages;
-    std::vector<int> slot_off, slot_cap, sc_cap, n_cols, alch_base, n_alch, item_cap, bo_off, n_bo, items;
+    std::vector<int> slot_off, slot_cap, sc_cap, n_cols, alch_base, n_alch, item_cap, bo_off, n_bo;
     std::vector<int> sys_w0;       // first walker of each system
     std::vector<int> sys_stage0;   // first stage of each system
     std::vector<int> sys_nstage;
@@ -351,13 +351,14 @@ struct la_handle {
     int io_floats = 0;
     la_options opt{};
     int graph_steps = 10;
-    cudaGraphExec_t graph = nullptr, graph1 = nullptr;  // graph_steps steps, one step
+    cudaGraphExec_t graph[2] = {}, graph1[2] = {};  // graph_steps steps, one step; [1] with the pair latency form
     cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
     long long graph_launches_per_step = 0;
     int n_sm = 0, dev = 0;
     // page-locked: [0] the status word posted by the last call, [1] the one read
-    // by sync_status, then from STAGE_OFF on the staging area of small
-    // read-outs (held under stage_mutex until the caller's arrays are filled)
+    // by sync_status, from ITEMS_OFF on every walker's work items (written by the
+    // list builds), then from STAGE_OFF on the staging area of small read-outs
+    // (held under stage_mutex until the caller's arrays are filled)
     unsigned *h_status = nullptr;
     size_t stage_cap = 0;
     std::mutex stage_mutex;
@@ -445,7 +446,7 @@ int sync_status(la_handle *h, cudaStream_t s, unsigned *bits) {
 // Small read-outs: device arrays are copied into the page-locked staging area
 // (asynchronously: a copy to pageable memory waits for itself), and the
 // caller reads them after one synchronisation.
-constexpr size_t STAGE_OFF = 256;
+constexpr size_t ITEMS_OFF = 256, STAGE_OFF = ITEMS_OFF + 4 * LA_MAX_WALKERS;
 struct Stage {
     la_handle *h;
     cudaStream_t s;
@@ -475,7 +476,7 @@ size_t stage_bytes(const Layout &L) {
 int enqueue_step(la_handle *h, int w0, int w1, cudaStream_t s) {
     launch_integrate_gate(h->d, h->hv, w0, w1, 0, false, s);
     launch_rebuild(h->d, h->hv, w0, w1, s, true);
-    launch_pairs_fused(h->d, h->hv, (int)h->stages.size(), s);
+    launch_pairs_fused(h->d, h->hv, pairs_latency(h->hv, w0, w1), s);
     return 0;
 }
 
@@ -528,7 +529,7 @@ int flush_dirty(la_handle *h, cudaStream_t s) {
 // must rebuild){rebuild chain} -> pairs, bonded, walker, lambda.  The gate sets
 // the step's conditional handle, so steps without a rebuild launch no list
 // kernel at all.
-int capture_steps(la_handle *h, int steps, cudaGraphExec_t *exec) {
+int capture_steps(la_handle *h, int steps, bool latency, cudaGraphExec_t *exec) {
     if (*exec) {
         cudaGraphExecDestroy(*exec);
         *exec = nullptr;
@@ -560,7 +561,7 @@ int capture_steps(la_handle *h, int steps, cudaGraphExec_t *exec) {
         cudaGraph_t body_out;
         CU(h, cudaStreamEndCapture(cb, &body_out));
         CU(h, cudaStreamUpdateCaptureDependencies(cs, &prev, nullptr, 1, cudaStreamSetCaptureDependencies));
-        launch_pairs_fused(h->d, h->hv, (int)h->stages.size(), cs);
+        launch_pairs_fused(h->d, h->hv, latency, cs);
     }
     CU(h, cudaStreamEndCapture(cs, &g));
     cudaError_t e = cudaGraphInstantiate(exec, g, 0);
@@ -572,15 +573,39 @@ int capture_steps(la_handle *h, int steps, cudaGraphExec_t *exec) {
 // the graph of graph_steps steps, and one of a single step for the remainder of
 // a call (as single launches every remaining step started the whole chain of
 // list kernels)
+int capture_form(la_handle *h, bool latency) {
+    int rc = capture_steps(h, h->graph_steps, latency, &h->graph[latency]);
+    if (rc != LA_OK || h->graph_steps == 1) return rc;
+    return capture_steps(h, 1, latency, &h->graph1[latency]);
+}
+
 int capture_graph(la_handle *h) {
     h->launches_per_step = kernels_per_step(h);
     if (h->graph_steps == 0) return LA_OK;
     // graph steps: integrate, gate, fused pairs; list kernels are counted per
     // step that runs them (device counter)
     h->graph_launches_per_step = h->launches_per_step - rebuild_kernel_count(h->hv, 0, h->L.W);
-    int rc = capture_steps(h, h->graph_steps, &h->graph);
-    if (rc != LA_OK || h->graph_steps == 1) return rc;
-    return capture_steps(h, 1, &h->graph1);
+    for (int k = 0; k < 2; ++k)
+        for (cudaGraphExec_t *g : {&h->graph[k], &h->graph1[k]}) {
+            if (*g) cudaGraphExecDestroy(*g);
+            *g = nullptr;
+        }
+    return capture_form(h, pairs_latency(h->hv, 0, h->L.W));
+}
+
+// The graphs' form of the pair launch for the lists as they are now (as far as
+// the host knows: a state that was set, or a condensing one, is noticed when its
+// first list build is through).  The other form's graphs are captured when they
+// are first needed; if that fails, the ones that are there do.
+int graph_form(la_handle *h) {
+    const int k = pairs_latency(h->hv, 0, h->L.W) ? 1 : 0;
+    if (!h->graph[k] || (!h->graph1[k] && h->graph_steps > 1)) {
+        if (capture_form(h, k != 0) != LA_OK) {
+            cudaGetLastError();
+            return 1 - k;
+        }
+    }
+    return k;
 }
 
 void set_pair_blocks(la_handle *h, int ctas_per_sm) {
@@ -701,8 +726,6 @@ int tune_pairs(la_handle *h, cudaStream_t s, bool use_cache) {
         int rc = rebuild_items(h, s);
         if (rc != LA_OK) return rc;
     }
-    CU(h, cudaMemcpyAsync(h->items.data(), h->d.n_items, sizeof(int) * h->L.W, cudaMemcpyDeviceToHost, s));
-    CU(h, cudaStreamSynchronize(s));
     return refresh_forces(h, s);
 }
 
@@ -1057,8 +1080,6 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     hv.item_cap = h->item_cap.data();
     hv.bo_off = h->bo_off.data();
     hv.n_bo = h->n_bo.data();
-    h->items = h->item_cap;  // until the first lists are counted
-    hv.items = h->items.data();
     set_pair_blocks(h, h->opt.pair_ctas_per_sm > 0 ? h->opt.pair_ctas_per_sm : 4);
     h->hv.pair_variant = h->opt.pair_variant;
     // graph_steps < 0: no graph (one batched launch sequence per step)
@@ -1067,6 +1088,9 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     h->stage_cap = stage_bytes(L);
     CU(h, cudaMallocHost((void **)&h->h_status, STAGE_OFF + h->stage_cap));
     h->h_status[0] = h->h_status[1] = 0;
+    d.items_posted = (int *)((char *)h->h_status + ITEMS_OFF);
+    for (int w = 0; w < L.W; ++w) d.items_posted[w] = h->item_cap[w];  // until the first lists are counted
+    hv.items = d.items_posted;
     CU(h, cudaEventCreateWithFlags(&h->status_ev, cudaEventDisableTiming));
     CU(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
     CU(h, cudaStreamCreateWithFlags(&h->cap_stream2, cudaStreamNonBlocking));
@@ -1075,8 +1099,6 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     if (rc != LA_OK) return rc;
     rc = sync_status(h, s, nullptr);
     if (rc != LA_OK) return rc;
-
-    CU(h, cudaMemcpy(h->items.data(), d.n_items, sizeof(int) * L.W, cudaMemcpyDeviceToHost));
 
     // ---- launch-shape autotuner (pair kernel only; the state does not move) ----
     if (h->opt.autotune) {
@@ -1103,14 +1125,14 @@ int la_step_walkers(la_handle *h, int64_t n_steps, void *stream) {
     if (rc != LA_OK) return rc;
     const int64_t gs = h->graph_steps;
     const int64_t reps = gs > 0 ? n_steps / gs : 0, rem = gs > 0 ? n_steps % gs : n_steps;
-    for (int64_t r = 0; r < reps; ++r) CU(h, cudaGraphLaunch(h->graph, s));
+    for (int64_t r = 0; r < reps; ++r) CU(h, cudaGraphLaunch(h->graph[graph_form(h)], s));
     // (a graph with conditional nodes cannot join a caller's stream capture:
     // there the remainder is captured launch by launch)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (rem > 0) CU(h, cudaStreamIsCapturing(s, &cap));
     const bool single = gs > 0 && cap == cudaStreamCaptureStatusNone;
     for (int64_t r = 0; r < rem; ++r) {
-        if (single) CU(h, cudaGraphLaunch(h->graph1, s));
+        if (single) CU(h, cudaGraphLaunch(h->graph1[graph_form(h)], s));
         else enqueue_step(h, 0, h->L.W, s);
     }
     launch_finish(h->d, h->hv, 0, h->L.W, s);
@@ -1430,6 +1452,7 @@ int la_checkpoint_load(la_handle *h, const void *buf, size_t bytes, void *stream
     cudaStream_t s = (cudaStream_t)stream;
     CU(h, cudaStreamSynchronize(s));
     CU(h, cudaMemcpyAsync(h->arena, (const char *)buf + sizeof hd, h->state_bytes, cudaMemcpyHostToDevice, s));
+    CU(h, cudaMemcpyAsync(h->d.items_posted, h->d.n_items, sizeof(int) * h->L.W, cudaMemcpyDeviceToHost, s));
     h->dirty = false;
     h->steps = hd.steps;
     h->launches = hd.launches;
@@ -1744,7 +1767,7 @@ int la_time_kernels(la_handle *h, int n_steps, float *ms_out, int64_t *launches_
         cudaEventRecord(ev[4], s);
         // the fused launch of the batched step: pairs, bonded terms, walker
         // terms and the lambda update
-        launch_pairs_fused(h->d, h->hv, (int)h->stages.size(), s);
+        launch_pairs_fused(h->d, h->hv, pairs_latency(h->hv, 0, W), s);
         cudaEventRecord(ev[5], s);
         CU(h, cudaEventSynchronize(ev[5]));
         float t01 = 0.f, t12 = 0.f, t34 = 0.f, t45 = 0.f;
@@ -1795,8 +1818,9 @@ const char *la_last_error(la_handle *h) { return h ? h->err.c_str() : "no handle
 
 int la_destroy(la_handle *h) {
     if (!h) return LA_OK;
-    if (h->graph) cudaGraphExecDestroy(h->graph);
-    if (h->graph1) cudaGraphExecDestroy(h->graph1);
+    for (int k = 0; k < 2; ++k)
+        for (cudaGraphExec_t g : {h->graph[k], h->graph1[k]})
+            if (g) cudaGraphExecDestroy(g);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->cap_stream2) cudaStreamDestroy(h->cap_stream2);
     if (h->status_ev) cudaEventDestroy(h->status_ev);

@@ -148,6 +148,7 @@ struct Dev {
     unsigned char *ent_lb;        // 32 per entry: byte 8 jb + ia, bit ic = pair (8 ic + ia, jb)
     int4 *items;                  // (global sc, e0, e1, walker)
     int *n_items;
+    int *items_posted;            // n_items once more, in page-locked host memory: sizes launches
     // alchemical lists and partial sums
     int *alch_cnt, *alch_slot;
     double *alch_out;             // 4 per (walker, alch): dU/dlv, dU/dle, U_sc, le U_rf

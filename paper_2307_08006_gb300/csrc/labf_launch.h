@@ -16,7 +16,7 @@ struct HostView {
     const int *slot_off = nullptr, *slot_cap = nullptr, *sc_cap = nullptr, *n_cols = nullptr;
     const int *alch_base = nullptr, *n_alch = nullptr, *item_cap = nullptr;
     const int *bo_off = nullptr, *n_bo = nullptr;
-    const int *items = nullptr;  // pair work items per walker at creation or the last tuning (sizes launches)
+    const volatile int *items = nullptr;  // pair work items per walker, as the list builds that are through left them
 };
 
 void launch_integrate(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s);
@@ -38,8 +38,10 @@ void launch_coalesce(const Dev &d, int w0, int w1, cudaStream_t s);
 void launch_pairs(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s);
 // pairs, bonded terms and restraints of one walker with energies and derivatives
 void launch_pairs_energy(const Dev &d, const HostView &hv, int w, cudaStream_t s);
+// whether a pair launch of walkers [w0, w1) takes the latency form now
+bool pairs_latency(const HostView &hv, int w0, int w1);
 // pairs + bonded + walker terms + lambda update of all walkers in one launch
-void launch_pairs_fused(const Dev &d, const HostView &hv, int n_stages, cudaStream_t s);
+void launch_pairs_fused(const Dev &d, const HostView &hv, bool latency, cudaStream_t s);
 void launch_bonded(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s);
 void launch_walker(const Dev &d, int w0, int w1, cudaStream_t s);
 void launch_lambda(const Dev &d, int s0, int s1, bool prime, cudaStream_t s);
