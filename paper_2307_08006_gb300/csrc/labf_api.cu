@@ -697,6 +697,8 @@ int tune_pairs(la_handle *h, cudaStream_t s, bool use_cache) {
             for (int m = 0; m < LA_PAIR_VARIANTS; ++m) {
                 h->hv.pair_variant = m;
                 for (int c : ctas) {
+                    // (the latency form has its own grid)
+                    if (c != 4 && pairs_latency(h->hv, 0, W)) continue;
                     set_pair_blocks(h, c);
                     for (int r = 0; r < 2; ++r) launch_pairs(h->d, h->hv, 0, W, s);  // warm
                     CU(h, cudaEventRecord(a, s));

@@ -58,3 +58,16 @@ def test_state_of_another_density(condense, plain):
     assert best[0] <= 1.25 * best[1], best
     for eng in engines:
         eng.close()
+
+
+def test_tuning_in_the_latency_form():
+    """The grid of the latency form is fixed: a tuning on few items that ends
+    with the form's variant keeps the default grid for the common form, instead
+    of one that noise picked."""
+    from paper_2307_08006_gb300 import labf
+
+    eng = labf.engine_for(synth.lj_fluid(seed=4), synth.lj_fluid_run(seed=9, n_walkers=2, n_bins=8))
+    reports = [eng.autotune() for _ in range(6)]
+    eng.close()
+    assert any("pair_variant=0" in r for r in reports)
+    assert all("pair_ctas_per_sm=4" in r for r in reports if "pair_variant=0" in r), reports
