@@ -416,18 +416,19 @@ int la_stats(la_handle *h, int64_t *out, void *stream);
 /*
  * la_time_kernels: run n_steps batched steps outside the graph with CUDA
  * events between the launches on `stream`, in the order and with the
- * conditions of the graph's step: the integrator, the gate kernel, the list
- * kernels only on steps where some walker must rebuild (the host reads the
- * walkers' rebuild flags after the gate, as the graph's conditional node
- * does on the device), and the fused pair launch.  ms_out (host
- * [LA_N_KERNELS]) receives the mean device milliseconds per MD step of each
- * class (so that integrate + rebuild + pairs is the step's kernel time, the
- * list kernels averaged over the steps at the rebuild rate met), and
- * launches_out (host [LA_N_KERNELS], may be NULL) the launch counts.  In the
- * batched step the bonded terms, the walker terms and the lambda update run
- * inside the pair launch, so their classes read 0.  Synchronising.
+ * conditions of the graph's step: the integrator, the gate kernel (none for
+ * small batches, whose integrator launch does the gate), the list kernels
+ * only on steps where some walker must rebuild (the host reads the walkers'
+ * rebuild flags after the gate, as the graph's conditional node does on the
+ * device), and the fused pair launch.  ms_out (host [LA_N_KERNELS]) receives
+ * the mean device milliseconds per MD step of each class (so that integrate +
+ * rebuild + pairs is the step's kernel time, the list kernels averaged over
+ * the steps at the rebuild rate met), and launches_out (host [LA_N_KERNELS],
+ * may be NULL) the launch counts.  In the batched step the bonded terms, the
+ * walker terms and the lambda update run inside the pair launch, so their
+ * classes read 0.  Synchronising.
  */
-#define LA_N_KERNELS 6 /* integrate, rebuild (gate + list kernels when due), pairs, bonded, walker, lambda */
+#define LA_N_KERNELS 6 /* integrate, rebuild (gate kernel + list kernels when due), pairs, bonded, walker, lambda */
 int la_time_kernels(la_handle *h, int n_steps, float *ms_out, int64_t *launches_out, void *stream);
 
 /*

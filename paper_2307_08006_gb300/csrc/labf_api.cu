@@ -1746,7 +1746,9 @@ int la_time_kernels(la_handle *h, int n_steps, float *ms_out, int64_t *launches_
     if (rc != LA_OK) return rc;
     const int W = h->L.W;
     // integrate | gate | (host reads the flags) | list kernels when a walker
-    // must rebuild | fused pair launch; the host's gap is in no class
+    // must rebuild | fused pair launch; the host's gap is in no class.  Where the
+    // step's integrator launch does the gate, so does this one.
+    const bool one = gate_in_integrate(h->hv, 0, W);
     cudaEvent_t ev[6];
     for (auto &e : ev) CU(h, cudaEventCreate(&e));
     double acc[LA_N_KERNELS] = {0};
@@ -1754,9 +1756,10 @@ int la_time_kernels(la_handle *h, int n_steps, float *ms_out, int64_t *launches_
     std::vector<int> flags(W);
     for (int k = 0; k < n_steps; ++k) {
         cudaEventRecord(ev[0], s);
-        launch_integrate(h->d, h->hv, 0, W, s);
+        if (one) launch_integrate_gate(h->d, h->hv, 0, W, 0, false, s);
+        else launch_integrate(h->d, h->hv, 0, W, s);
         cudaEventRecord(ev[1], s);
-        launch_gate(h->d, 0, W, 0, false, s);
+        if (!one) launch_gate(h->d, 0, W, 0, false, s);
         cudaEventRecord(ev[2], s);
         // the graph's conditional node runs the list kernels only on steps
         // where some walker must rebuild: read the flags the integrator set
@@ -1778,10 +1781,10 @@ int la_time_kernels(la_handle *h, int n_steps, float *ms_out, int64_t *launches_
         cudaEventElapsedTime(&t34, ev[3], ev[4]);
         cudaEventElapsedTime(&t45, ev[4], ev[5]);
         acc[0] += t01;
-        acc[1] += t12 + (any ? t34 : 0.f);
+        acc[1] += (one ? 0.f : t12) + (any ? t34 : 0.f);
         acc[2] += t45;  // bonded, walker, lambda run inside the pair launch: 0
         cnt[0] += 1;
-        cnt[1] += 1 + (any ? rebuild_kernel_count(h->hv, 0, W) : 0);
+        cnt[1] += (one ? 0 : 1) + (any ? rebuild_kernel_count(h->hv, 0, W) : 0);
         cnt[2] += 1;
     }
     launch_finish(h->d, h->hv, 0, W, s);

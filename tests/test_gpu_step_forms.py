@@ -54,6 +54,31 @@ def test_stage_sizes(walkers, shared_freq, theta):
     run_both(synth.lj_fluid(seed=12), run, 11)
 
 
+@pytest.mark.parametrize("walkers", [2, 100])  # the gate in the integrator's launch, and in one of its own
+def test_kernel_timer_runs_the_step(walkers):
+    """The kernel timer issues the launches of the graph's step: as many, with
+    the same bits."""
+    from paper_2307_08006_gb300 import labf
+
+    spec, out, launches = water(23), [], []
+    run = synth.water_run(seed=8, walkers_per_stage=1, n_bins=8)
+    run.stages = [synth.Stage(0.0, 1.0, 8, walkers)]
+    state = synth.initial_state(spec, run, lam0=list(np.linspace(0.1, 0.9, walkers)))
+    for timed in (False, True):
+        eng = labf.engine_for(spec, run, state)
+        before = int(eng.stats()[2])
+        if timed:
+            eng.time_kernels(25)
+        else:
+            eng.step(25)
+        launches.append(int(eng.stats()[2]) - before)
+        out.append(eng.get_states())
+        eng.close()
+    assert launches[0] == launches[1]
+    for k in ("x", "v", "lam", "plam"):
+        assert np.array_equal(out[0][k], out[1][k]), k
+
+
 @pytest.mark.parametrize("chunk, margin", [(32, 0.05), (64, 0.0), (96, 0.05)])
 def test_latency_form_items(chunk, margin):
     """The latency form (variant 0, few items) against the common form
