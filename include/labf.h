@@ -460,7 +460,8 @@ const char *la_autotune_report(la_handle *h);
 /* la_last_error: message of the last failing call on h (static per handle). */
 const char *la_last_error(la_handle *h);
 
-/* la_destroy: free host metadata and CUDA graphs; never touches the arena. */
+/* la_destroy: wait for the last asynchronous call on h, then free host metadata
+ * and CUDA graphs; never touches the arena. */
 int la_destroy(la_handle *h);
 
 /*

@@ -1823,6 +1823,8 @@ const char *la_last_error(la_handle *h) { return h ? h->err.c_str() : "no handle
 
 int la_destroy(la_handle *h) {
     if (!h) return LA_OK;
+    // list builds of the last asynchronous call may still post item counts
+    if (h->status_ev) cudaEventSynchronize(h->status_ev);
     for (int k = 0; k < 2; ++k)
         for (cudaGraphExec_t g : {h->graph[k], h->graph1[k]})
             if (g) cudaGraphExecDestroy(g);

@@ -71,3 +71,21 @@ def test_tuning_in_the_latency_form():
     eng.close()
     assert any("pair_variant=0" in r for r in reports)
     assert all("pair_ctas_per_sm=4" in r for r in reports if "pair_variant=0" in r), reports
+
+
+def test_close_waits_for_the_steps():
+    """The list builds write host memory that the engine owns: it is not given
+    back before they are through."""
+    import torch
+
+    from paper_2307_08006_gb300 import labf
+
+    eng = labf.engine_for(synth.lj_fluid(seed=4, cells=7), synth.lj_fluid_run(seed=9, n_walkers=16, n_bins=8))
+    arena = eng.arena
+    eng.step(2000)
+    done = torch.cuda.Event()
+    done.record()
+    eng.step(1)
+    eng.close()
+    assert done.query()
+    del arena
