@@ -292,7 +292,7 @@ size_t carve(const Layout &L, char *base, size_t cap, Dev &d, void **io, int *io
     d.plam = a.take<double>(L.W);
     d.G = a.take<double>(L.W);
     d.s = a.take<double>(L.W);
-    d.dl_direct = a.take<double>(L.W);
+    a.take<double>(L.W);  // unused
     d.wth = a.take<double>((size_t)L.W * 2 * L.P_max);
     d.step = a.take<unsigned long long>(L.W);
     d.pending = a.take<int>(L.W);
@@ -343,7 +343,7 @@ struct la_handle {
     std::vector<SysDev> sys;
     std::vector<WalkerDev> walk;
     std::vector<StageDev> stages;
-    std::vector<int> slot_off, slot_cap, sc_cap, n_cols, alch_base, n_alch, item_cap, bo_off, n_bo;
+    std::vector<int> slot_off, slot_cap, sc_cap, n_cols, alch_base, n_alch, bo_off, n_bo;
     std::vector<int> sys_w0;       // first walker of each system
     std::vector<int> sys_stage0;   // first stage of each system
     std::vector<int> sys_nstage;
@@ -470,7 +470,6 @@ size_t stage_bytes(const Layout &L) {
     return 8 * (3 * nb * P + 3 * nb + 3 * W * nb + 3 * W + 2 * P + 64) + 16 * 16;
 }
 
-// one batched MD step over walkers [w0, w1)
 // one batched MD step over all walkers: integrate, [rebuild], then one
 // launch for pairs, bonded terms, walker terms and the lambda update
 int enqueue_step(la_handle *h, int w0, int w1, cudaStream_t s) {
@@ -1007,7 +1006,6 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
                 h->n_cols.push_back(sl.n_cols);
                 h->alch_base.push_back(W.alch_base);
                 h->n_alch.push_back(sl.n_alch);
-                h->item_cap.push_back(W.item_cap);
                 h->bo_off.push_back(W.bo_off);
                 h->n_bo.push_back(W.n_bo);
                 slot_off += sl.slot_cap;
@@ -1079,7 +1077,6 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     hv.n_cols = h->n_cols.data();
     hv.alch_base = h->alch_base.data();
     hv.n_alch = h->n_alch.data();
-    hv.item_cap = h->item_cap.data();
     hv.bo_off = h->bo_off.data();
     hv.n_bo = h->n_bo.data();
     set_pair_blocks(h, h->opt.pair_ctas_per_sm > 0 ? h->opt.pair_ctas_per_sm : 4);
@@ -1091,7 +1088,7 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
     CU(h, cudaMallocHost((void **)&h->h_status, STAGE_OFF + h->stage_cap));
     h->h_status[0] = h->h_status[1] = 0;
     d.items_posted = (int *)((char *)h->h_status + ITEMS_OFF);
-    for (int w = 0; w < L.W; ++w) d.items_posted[w] = h->item_cap[w];  // until the first lists are counted
+    for (int w = 0; w < L.W; ++w) d.items_posted[w] = h->walk[w].item_cap;  // until the first lists are counted
     hv.items = d.items_posted;
     CU(h, cudaEventCreateWithFlags(&h->status_ev, cudaEventDisableTiming));
     CU(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));

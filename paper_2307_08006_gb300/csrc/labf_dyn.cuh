@@ -323,7 +323,6 @@ __device__ __forceinline__ void walker_sample(const Dev &d, int w, int lane) {
             atomicAdd((unsigned long long *)&et[2], (unsigned long long)__double2ll_rn(usc * E_TO_FIX));
             atomicAdd((unsigned long long *)&et[3], (unsigned long long)__double2ll_rn(urf * E_TO_FIX));
             atomicAdd((unsigned long long *)&et[6], (unsigned long long)__double2ll_rn(__ldcg(dir + 1) * E_TO_FIX));
-            d.dl_direct[w] = __ldcg(dir);
         }
     }
     if (ENERGY) {

@@ -154,7 +154,7 @@ struct Dev {
     double *alch_out;             // 4 per (walker, alch): dU/dlv, dU/dle, U_sc, le U_rf
     double *alch_th;              // 6 per (walker, alch): dU/d(eps, sig, q), d2 v(eps, sig), d2 e(q)
     // per walker
-    double *lam, *plam, *G, *s, *dl_direct, *wth;
+    double *lam, *plam, *G, *s, *wth;
     unsigned long long *step;
     int *pending, *rebuild;
     long long *eterm;             // N_ETERMS per walker, 2^-24 fixed point

@@ -14,7 +14,7 @@ struct HostView {
     int n_walkers = 0, n_sm = 0, pair_blocks = 0;
     int pair_variant = 0;  // 0: 8 warps/CTA, 80 regs; 1: 4 warps, 72; 2: 4 warps, 64
     const int *slot_off = nullptr, *slot_cap = nullptr, *sc_cap = nullptr, *n_cols = nullptr;
-    const int *alch_base = nullptr, *n_alch = nullptr, *item_cap = nullptr;
+    const int *alch_base = nullptr, *n_alch = nullptr;
     const int *bo_off = nullptr, *n_bo = nullptr;
     const volatile int *items = nullptr;  // pair work items per walker, as the list builds that are through left them
 };
