@@ -928,7 +928,6 @@ __device__ __forceinline__ void make_items(const Dev &d, ItemShared &sh, int w, 
     if (threadIdx.x == 0) {
         if (done > W.item_cap) set_status(d, LA_STATUS_LIST_OVERFLOW);
         d.n_items[w] = min(done, W.item_cap);
-        *(volatile int *)(d.items_posted + w) = min(done, W.item_cap);
         d.rebuild[w] = 0;
         d.near[w] = 0;
         if (prune_fresh && d.sys[W.sys].prune_disp2 > 0.f) d.prune_now[w] = d.step[w] + 1ull;

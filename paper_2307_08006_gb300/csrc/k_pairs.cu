@@ -71,7 +71,7 @@ struct PairShared {
     float4 jx[WARPS][EPC][JC];  // prepared j-atoms (shift applied)
     float2 jl[WARPS][EPC][JC];
     unsigned char lb[WARPS][EPC][32];
-    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], first;
+    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], first, parts;
 };
 
 // Shared memory of the latency form: the super-cluster's i-clusters two by
@@ -85,7 +85,7 @@ struct PairSharedLat {
     unsigned char lb[EPC][32];
     float2 f[EPC][NIC / 2][32];
     unsigned char keep[EPC][NIC / 2];
-    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], next;
+    int pre[LA_MAX_WALKERS_PER_LAUNCH + 1], first, next, parts;
 };
 constexpr int LAT_WARPS = NIC / 2;
 
@@ -540,7 +540,7 @@ __device__ __forceinline__ void items_done(const Dev &d, bool arrives, unsigned 
 
 // work items of the normal pairs, handed out by a global counter
 template <bool ENERGY, int WARPS, int MSHIFT>
-__device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int nblk, PairShared<WARPS> &sh) {
+__device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, PairShared<WARPS> &sh) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nw = w1 - w0;
     const int total = sh.pre[nw];
@@ -577,17 +577,15 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, int n
             }
         }
     }
-    items_done(d, lane == 0, (unsigned long long)nblk * WARPS);
+    items_done(d, lane == 0, (unsigned long long)sh.parts * WARPS);
 }
 
-// the same with one item per block at a time (latency form); block blk starts
-// with item blk, and those without a first item have no part in the queue
+// the same with one item per block at a time (latency form)
 template <int MSHIFT>
-__device__ __forceinline__ void normal_items_lat(const Dev &d, int w0, int w1, int blk, int nblk, PairSharedLat &sh) {
+__device__ __forceinline__ void normal_items_lat(const Dev &d, int w0, int w1, PairSharedLat &sh) {
     const int nw = w1 - w0;
     const int total = sh.pre[nw];
-    if (blk >= total) return;
-    for (int v = blk; v < total;) {
+    for (int v = sh.first; v < total;) {
         int w, gS;
         int4 it;
         if (find_item(d, sh.pre, w0, nw, v, w, it, gS)) {
@@ -595,12 +593,12 @@ __device__ __forceinline__ void normal_items_lat(const Dev &d, int w0, int w1, i
             if (MSHIFT == 8 && d.prune_now[w] != 0ull) item_entries_lat<MSHIFT, true>(d, sh, S, it, gS);
             else item_entries_lat<MSHIFT, false>(d, sh, S, it, gS);
         }
-        if (threadIdx.x == 0) sh.next = nblk + (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
+        if (threadIdx.x == 0) sh.next = (int)atomicAdd(&d.counters[CTR_ITEM], 1ull);
         __syncthreads();
         v = sh.next;
         __syncthreads();
     }
-    items_done(d, threadIdx.x == 0, (unsigned long long)min(nblk, total));
+    items_done(d, threadIdx.x == 0, (unsigned long long)sh.parts);
 }
 
 // Fused launch: a stage's lambda update (lambda_work) needs the partial sums
@@ -835,6 +833,14 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w
         bonded_items<ENERGY>(d, w0, w1, blockIdx.x - nblk_alch, nblk_bonded);
         return;
     }
+    constexpr int PER = LAT ? 1 : WARPS;  // items of a block at a time
+    const int blk = blockIdx.x - nblk_alch - nblk_bonded;
+    // The item counts go to the host here, where nothing waits for the store.
+    // (By the list build's last block, which fences after it, a rebuild took 2 us
+    // longer.)
+    if (blk == 0 && threadIdx.x >= 32)
+        for (int w = w0 + threadIdx.x - 32; w < w1; w += blockDim.x - 32)
+            *(volatile int *)(d.items_posted + w) = d.n_items[w];
     if (threadIdx.x < 32) {  // prefix of the walkers' work items
         int acc = 0;
         for (int b = 0; b < w1 - w0; b += 32) {
@@ -848,14 +854,20 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w
             if (k < w1 - w0) sh.pre[k] = acc + x - n;
             acc += __shfl_sync(FULL, x, 31);
         }
+        // the blocks that take part: as many as a quarter more items would need
+        // (idle blocks cost the others their atomics on the queue: 0.5 us of 17 us
+        // for 4 x 257 atoms, 3 us of 35 us for 14 x 2049)
+        const int parts = min(nblk_pairs, (acc + acc / 4 + PER - 1) / PER);
         if (threadIdx.x == 0) {
             sh.pre[w1 - w0] = acc;
-            if constexpr (!LAT) sh.first = (int)atomicAdd(&d.counters[CTR_ITEM], (unsigned long long)WARPS);
+            sh.parts = parts;
+            if (blk < parts) sh.first = (int)atomicAdd(&d.counters[CTR_ITEM], (unsigned long long)PER);
         }
     }
     __syncthreads();
-    if constexpr (LAT) normal_items_lat<MODE == STEP ? 8 : 16>(d, w0, w1, blockIdx.x - nblk_alch - nblk_bonded, nblk_pairs, sh);
-    else normal_items<ENERGY, WARPS, MODE == STEP ? 8 : 16>(d, w0, w1, nblk_pairs, sh);
+    if (blk >= sh.parts) return;
+    if constexpr (LAT) normal_items_lat<MODE == STEP ? 8 : 16>(d, w0, w1, sh);
+    else normal_items<ENERGY, WARPS, MODE == STEP ? 8 : 16>(d, w0, w1, sh);
 }
 
 template <bool ENERGY, int WARPS, int MINB, int MODE, bool LAT>
@@ -884,8 +896,8 @@ static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cud
 }
 
 // launches whose items leave an SM few enough of them take the latency form.
-// The counts are those of the list builds that are through when the launch is
-// enqueued; both forms take any number.
+// The counts are those that the last pair launch met; both forms take any
+// number.
 bool pairs_latency(const HostView &hv, int w0, int w1) {
     long long n = 0;
     for (int w = w0; w < w1; ++w) n += hv.items[w];

@@ -357,7 +357,7 @@ struct la_handle {
     int n_sm = 0, dev = 0;
     // page-locked: [0] the status word posted by the last call, [1] the one read
     // by sync_status, from ITEMS_OFF on every walker's work items (written by the
-    // list builds), then from STAGE_OFF on the staging area of small read-outs
+    // pair launches), then from STAGE_OFF on the staging area of small read-outs
     // (held under stage_mutex until the caller's arrays are filled)
     unsigned *h_status = nullptr;
     size_t stage_cap = 0;
@@ -594,7 +594,7 @@ int capture_graph(la_handle *h) {
 
 // The graphs' form of the pair launch for the lists as they are now (as far as
 // the host knows: a state that was set, or a condensing one, is noticed when its
-// first list build is through).  The other form's graphs are captured when they
+// first pair launch runs).  The other form's graphs are captured when they
 // are first needed; if that fails, the ones that are there do.
 int graph_form(la_handle *h) {
     const int k = pairs_latency(h->hv, 0, h->L.W) ? 1 : 0;
@@ -656,6 +656,7 @@ int rebuild_items(la_handle *h, cudaStream_t s) {
     std::vector<int> one(W, 1);
     CU(h, cudaMemcpyAsync(h->d.rebuild, one.data(), sizeof(int) * W, cudaMemcpyHostToDevice, s));
     launch_items(h->d, h->hv, 0, W, s);
+    CU(h, cudaMemcpyAsync(h->d.items_posted, h->d.n_items, sizeof(int) * W, cudaMemcpyDeviceToHost, s));
     CU(h, cudaMemcpyAsync(h->d.counters, &nreb, sizeof nreb, cudaMemcpyHostToDevice, s));  // not a rebuild
     CU(h, cudaStreamSynchronize(s));
     return LA_OK;
@@ -1820,7 +1821,7 @@ const char *la_last_error(la_handle *h) { return h ? h->err.c_str() : "no handle
 
 int la_destroy(la_handle *h) {
     if (!h) return LA_OK;
-    // list builds of the last asynchronous call may still post item counts
+    // pair launches of the last asynchronous call may still post item counts
     if (h->status_ev) cudaEventSynchronize(h->status_ev);
     for (int k = 0; k < 2; ++k)
         for (cudaGraphExec_t g : {h->graph[k], h->graph1[k]})

@@ -74,7 +74,7 @@ def test_tuning_in_the_latency_form():
 
 
 def test_close_waits_for_the_steps():
-    """The list builds write host memory that the engine owns: it is not given
+    """The pair launches write host memory that the engine owns: it is not given
     back before they are through."""
     import torch
 
