@@ -164,13 +164,18 @@ __device__ __forceinline__ bool static_pair(const StaticParams &p, const StaticI
     return static_force_ok(o.top, status);
 }
 
-// f 2^32 modulo 2^64 (f2fix clamps at 2^31; a warp's share may be 2^40)
+// f 2^32 modulo 2^64 (f2fix clamps at 2^31; a warp's share may be 2^40), by
+// shifting the mantissa: the conversion to 64-bit integers runs on the FP64
+// pipe (2.5% of the time of 27 100 x 100 atoms)
 __device__ __forceinline__ unsigned long long f2fix_wrap(float f) {
-    return fabsf(f) < FIX_LIMIT ? f2fix(f) : (unsigned long long)(long long)f << 32;
+    if (fabsf(f) < FIX_LIMIT) return f2fix(f);
+    const unsigned bits = __float_as_uint(fabsf(f));
+    const unsigned long long v = (unsigned long long)((bits & 0x7fffffu) | 0x800000u) << (((int)(bits >> 23) - 118) & 63);
+    return f < 0.f ? 0ull - v : v;
 }
 
 // the whole force on environment atom b, by its thread
-__device__ __noinline__ bool env_force_ok(const StaticParams &p, const StaticIn &in, int b, float xb, float yb, float zb,
+__device__ __forceinline__ bool env_force_ok(const StaticParams &p, const StaticIn &in, int b, float xb, float yb, float zb,
                                           int gb, unsigned *status) {
     float f[3] = {0.f, 0.f, 0.f};
     for (int r = 0; r < p.n_alch; ++r) {
@@ -185,7 +190,7 @@ __device__ __noinline__ bool env_force_ok(const StaticParams &p, const StaticIn 
 
 // the whole force on alchemical atom A, by the block; also those on the
 // environment atoms of A's big pairs
-__device__ __noinline__ bool alch_force_ok(const StaticParams &p, const StaticIn &in, const StaticAlch &A,
+__device__ __forceinline__ bool alch_force_ok(const StaticParams &p, const StaticIn &in, const StaticAlch &A,
                                            float (&share)[ST_WARPS][3], unsigned *status) {
     float f[3] = {0.f, 0.f, 0.f};
     for (int b = threadIdx.x; b < p.n; b += ST_THREADS) {
