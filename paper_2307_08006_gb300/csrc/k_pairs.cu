@@ -803,12 +803,15 @@ __device__ __forceinline__ void bonded_items(const Dev &d, int w0, int w1, int b
 }
 
 // Items per SM up to which the latency form is taken, and its blocks per SM
-// (42.6 KB of shared memory, 122 registers).  Fused launch, common / one warp
-// per item / latency form: 0.4 items per SM (4 x 257 atoms) 33 / 19 / 17 us, 5
-// (8 x 772 atoms) 43 / 32 / 32 us (there the alchemical warps' chain decides), 19
-// (2 x 9020 atoms) 43 / - / 43 us, 92 (144 x 772 atoms) 117 / - / 174 us, 200
-// (16 x 12 300 atoms) 242 / - / 366 us.
-constexpr int LAT_ITEMS_PER_SM = 8;
+// (42.6 KB of shared memory, 124 registers).  The line lies where the two forms
+// take the same time, so that a batch whose lists drift across it does not
+// notice.  Fused launch, common / latency form, by items per SM: 3.5 (4 x 2049 LJ
+// atoms) 28 / 19 us, 4.8 (8 x 772 atoms) 32 / 26, 9.3 (9020 atoms) 36 / 31, 12.1
+// (14 x 2049) 31 / 28, 14.3 (128 x 257) 48 / 48, 14.7 (17 x 2049) 34 / 31, 17.2
+// (20 x 2049) 35 / 35, 17.9 (160 x 257) 57 / 58, 18.6 (2 x 9020) 43 / 42, 20.7
+// (24 x 2049) 35 / 40, 23.9 (2 x 12 300) 47 / 52, 31 (36 x 2049) 43 / 54, 200 (16
+// x 12 300) 242 / 366.
+constexpr int LAT_ITEMS_PER_SM = 17;
 constexpr int LAT_BLOCKS_PER_SM = 4;
 
 // WARPS x 32 threads per CTA; MINB: resident CTAs per SM the register

@@ -46,6 +46,14 @@ def test_pair_forms(walkers, margin):
     run_both(water(31), run, 23, prune_margin=margin)
 
 
+@pytest.mark.parametrize("walkers", [17, 24])
+def test_pair_forms_near_the_line(walkers):
+    """2049 LJ atoms per walker: 15 items per SM (latency form) and 21 (common
+    form)."""
+    run = synth.lj_fluid_run(seed=9, n_walkers=walkers, n_bins=7)
+    run_both(synth.lj_fluid(seed=12, cells=8), run, 11)
+
+
 @pytest.mark.parametrize("walkers, shared_freq, theta", [(1, 1, True), (3, 2, True), (33, 1, True), (70, 3, False),
                                                          (64, 1, False)])
 def test_stage_sizes(walkers, shared_freq, theta):
