@@ -42,6 +42,10 @@ __device__ __forceinline__ void integrate_lambda(const Dev &d, int w0, int w1) {
     const StageDev &st = d.stage[d.walk[on ? w : w0].stage];
     const double hdt = 0.5 * S.dt_d;
     double lam = 0.0, p = 0.0;
+    // the fourth part's threads leave the walkers' item counts with the host (the
+    // store is through long before the block's fence; by the list build's last
+    // block a rebuild took 2 us longer, by the pair launch its common form 0.5%)
+    if (part == 3 && w < w1) *(volatile int *)(d.items_posted + w) = d.n_items[w];
     if (on) {
         if (part == 0) radius[l] = normal_lambda_radius(S.seed, (uint32_t)d.walk[w].wlocal, d.step[w]);
         if (part == 1) angle[l] = normal_lambda_cos(S.seed, (uint32_t)d.walk[w].wlocal, d.step[w]);

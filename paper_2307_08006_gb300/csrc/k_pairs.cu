@@ -577,7 +577,7 @@ __device__ __forceinline__ void normal_items(const Dev &d, int w0, int w1, PairS
             }
         }
     }
-    items_done(d, lane == 0, (unsigned long long)sh.parts * WARPS);
+    items_done(d, lane == 0 && sh.parts > 0, (unsigned long long)sh.parts * WARPS);
 }
 
 // the same with one item per block at a time (latency form)
@@ -598,7 +598,7 @@ __device__ __forceinline__ void normal_items_lat(const Dev &d, int w0, int w1, P
         v = sh.next;
         __syncthreads();
     }
-    items_done(d, threadIdx.x == 0, (unsigned long long)sh.parts);
+    items_done(d, threadIdx.x == 0 && sh.parts > 0, (unsigned long long)sh.parts);
 }
 
 // Fused launch: a stage's lambda update (lambda_work) needs the partial sums
@@ -838,12 +838,6 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w
     }
     constexpr int PER = LAT ? 1 : WARPS;  // items of a block at a time
     const int blk = blockIdx.x - nblk_alch - nblk_bonded;
-    // The item counts go to the host here, where nothing waits for the store.
-    // (By the list build's last block, which fences after it, a rebuild took 2 us
-    // longer.)
-    if (blk == 0 && threadIdx.x >= 32)
-        for (int w = w0 + threadIdx.x - 32; w < w1; w += blockDim.x - 32)
-            *(volatile int *)(d.items_posted + w) = d.n_items[w];
     if (threadIdx.x < 32) {  // prefix of the walkers' work items
         int acc = 0;
         for (int b = 0; b < w1 - w0; b += 32) {
@@ -857,18 +851,18 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_pairs(Dev d, int w0, int w
             if (k < w1 - w0) sh.pre[k] = acc + x - n;
             acc += __shfl_sync(FULL, x, 31);
         }
-        // the blocks that take part: as many as a quarter more items would need
-        // (idle blocks cost the others their atomics on the queue: 0.5 us of 17 us
-        // for 4 x 257 atoms, 3 us of 35 us for 14 x 2049)
+        // the blocks that take part: as many as a quarter more items would need;
+        // the others find the queue at its end without touching it (idle blocks'
+        // atomics cost the others 0.5 us of 17 us for 4 x 257 atoms, 3 us of 35 us
+        // for 14 x 2049)
         const int parts = min(nblk_pairs, (acc + acc / 4 + PER - 1) / PER);
         if (threadIdx.x == 0) {
             sh.pre[w1 - w0] = acc;
-            sh.parts = parts;
-            if (blk < parts) sh.first = (int)atomicAdd(&d.counters[CTR_ITEM], (unsigned long long)PER);
+            sh.parts = blk < parts ? parts : 0;
+            sh.first = blk < parts ? (int)atomicAdd(&d.counters[CTR_ITEM], (unsigned long long)PER) : acc;
         }
     }
     __syncthreads();
-    if (blk >= sh.parts) return;
     if constexpr (LAT) normal_items_lat<MODE == STEP ? 8 : 16>(d, w0, w1, sh);
     else normal_items<ENERGY, WARPS, MODE == STEP ? 8 : 16>(d, w0, w1, sh);
 }
@@ -899,8 +893,8 @@ static void launch_pairs_v(const Dev &d, const HostView &hv, int w0, int w1, cud
 }
 
 // launches whose items leave an SM few enough of them take the latency form.
-// The counts are those that the last pair launch met; both forms take any
-// number.
+// The counts are those that the last integrator launch met; both forms take
+// any number.
 bool pairs_latency(const HostView &hv, int w0, int w1) {
     long long n = 0;
     for (int w = w0; w < w1; ++w) n += hv.items[w];

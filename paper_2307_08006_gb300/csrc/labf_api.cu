@@ -357,7 +357,7 @@ struct la_handle {
     int n_sm = 0, dev = 0;
     // page-locked: [0] the status word posted by the last call, [1] the one read
     // by sync_status, from ITEMS_OFF on every walker's work items (written by the
-    // pair launches), then from STAGE_OFF on the staging area of small read-outs
+    // integrator), then from STAGE_OFF on the staging area of small read-outs
     // (held under stage_mutex until the caller's arrays are filled)
     unsigned *h_status = nullptr;
     size_t stage_cap = 0;
@@ -594,7 +594,7 @@ int capture_graph(la_handle *h) {
 
 // The graphs' form of the pair launch for the lists as they are now (as far as
 // the host knows: a state that was set, or a condensing one, is noticed when its
-// first pair launch runs).  The other form's graphs are captured when they
+// second step runs).  The other form's graphs are captured when they
 // are first needed; if that fails, the ones that are there do.
 int graph_form(la_handle *h) {
     const int k = pairs_latency(h->hv, 0, h->L.W) ? 1 : 0;
@@ -1097,6 +1097,7 @@ int la_create_system(const la_system_desc *sys, int n_sys, const la_options *opt
 
     rc = prime(h, 0, L.W, true, s);
     if (rc != LA_OK) return rc;
+    CU(h, cudaMemcpyAsync(d.items_posted, d.n_items, sizeof(int) * L.W, cudaMemcpyDeviceToHost, s));
     rc = sync_status(h, s, nullptr);
     if (rc != LA_OK) return rc;
 
@@ -1821,7 +1822,7 @@ const char *la_last_error(la_handle *h) { return h ? h->err.c_str() : "no handle
 
 int la_destroy(la_handle *h) {
     if (!h) return LA_OK;
-    // pair launches of the last asynchronous call may still post item counts
+    // the steps of the last asynchronous call may still post item counts
     if (h->status_ev) cudaEventSynchronize(h->status_ev);
     for (int k = 0; k < 2; ++k)
         for (cudaGraphExec_t g : {h->graph[k], h->graph1[k]})

@@ -16,7 +16,7 @@ struct HostView {
     const int *slot_off = nullptr, *slot_cap = nullptr, *sc_cap = nullptr, *n_cols = nullptr;
     const int *alch_base = nullptr, *n_alch = nullptr;
     const int *bo_off = nullptr, *n_bo = nullptr;
-    const volatile int *items = nullptr;  // pair work items per walker, as the last pair launch met them
+    const volatile int *items = nullptr;  // pair work items per walker, as the last integrator launch met them
 };
 
 void launch_integrate(const Dev &d, const HostView &hv, int w0, int w1, cudaStream_t s);

@@ -74,8 +74,8 @@ def test_tuning_in_the_latency_form():
 
 
 def test_close_waits_for_the_steps():
-    """The pair launches write host memory that the engine owns: it is not given
-    back before they are through."""
+    """The steps write host memory that the engine owns: it is not given back
+    before they are through."""
     import torch
 
     from paper_2307_08006_gb300 import labf
