@@ -445,8 +445,8 @@ __global__ void __launch_bounds__(256) k_permute_scatter(Dev d, int g0, int g1, 
 // launches for the alchemical lists and the work items: the last block of a
 // walker cuts its lists into work items.
 //
-// Bound by instruction issue (67% of the slots; 48% of the ALU pipe, 43% of
-// the FMA pipe).  One j-atom per lane keeps every lane on a candidate
+// Bound by instruction issue (68% of the slots; the ALU pipe is active in 49%
+// of the cycles, the FMA pipe in 43%).  One j-atom per lane keeps every lane on a candidate
 // j-cluster and puts the distances on the FMA pipe; per two i-atoms a lane
 // spends 8 packed FP32 and 7 ALU instructions, against about 55 for the two
 // half tiles with 64-bit integer arithmetic.  A rebuild of 16 walkers x 12 300

@@ -169,8 +169,9 @@ __device__ __forceinline__ void flush_j2(const Dev &d, int gjA, int gjB, bool ha
 // vote per tile, which also skips the force arithmetic of the others), which
 // later steps read; every tile that is skipped adds exact zeros, so results do
 // not depend on the pruning.  Without the skip a re-pruning launch took 287 us
-// against 229 us for a common one (16 x 12 300 atoms, ncu); with it the passes
-// of hot starts, where two launches in five re-prune, are 1.2-1.8% shorter.
+// against 229 us for a common one (16 x 12 300 atoms, ncu), with it 279 us; the
+// passes of hot starts, where two launches in five re-prune, are 1.2-1.8%
+// shorter.
 template <bool ENERGY, int WARPS, int MSHIFT, bool PRUNE>
 __device__ __forceinline__ int item_entries(const Dev &d, PairShared<WARPS> &sh, const SysDev &S, int4 it, int gS,
                                             float &elj, float &erf, int &npair) {
